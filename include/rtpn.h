@@ -167,7 +167,7 @@ int rtpn_set_kernel(rtpn_ctx* ctx, int kernel, int tile_x, int tile_y, int tile_
 
 /* As rtpn_set_kernel, and for RTPN_KERNEL_STAGE the pipeline depth: the number of shared-memory
  * stage buffers, of which all but one hold copies in flight (2..8; 0 = any compiled).  The staged
- * kernel runs two threads per cell of the tile (one per target type) plus one producer warp.
+ * kernel runs one thread per cell of the tile (both target types) plus two producer warps.
  * RTPN_EINVAL for a depth outside 0..8, RTPN_EUNSUPPORTED if no staged variant is compiled for
  * (N, tile, depth). */
 int rtpn_set_kernel_ex(rtpn_ctx* ctx, int kernel, int tile_x, int tile_y, int tile_z, int depth);

@@ -22,7 +22,7 @@ struct Variant {
     int N, tx, ty, tz, depth;
     int (*launch)(int, int, int, const Args&, int, cudaStream_t);  // (cls, precision, mode, ...)
     int (*smem)(int, int);
-    void (*geom)(int, int*);  // (precision, {maps per kind, box length step, x group width, x group rows})
+    void (*geom)(int, int*);  // (precision, {maps per kind, CTAs per SM, x group width, x group rows})
 };
 #define RTPN_SENTRY(n, x, y, z, b, e)                                                                \
     Variant{n, x, y, z, b, stage_launch_##n##_##x##_##y##_##z##_##b##_##e,                           \
@@ -72,21 +72,54 @@ static bool make_map(CUtensorMap* m, void* base, int precision, const rtpn::Geom
 }
 
 // The tensor maps of one array for a variant (kinds MAP_PLANE, MAP_YROW, MAP_XGRP, each for box
-// lengths E = eq, 2 eq, ..., nmap eq; see stage_impl.cuh) into out[0 .. kinds * nmap); kinds = 1 builds
-// the plane maps only (target arrays).
+// lengths E = 1, 2, ..., nmap; see stage_impl.cuh) into out[0 .. kinds * nmap); kinds = 1 builds the
+// plane maps only (target arrays).
 static bool make_maps(CUtensorMap* out, void* base, int precision, const rtpn::Geom& g, int nc, const Variant& v,
                       int kinds) {
     int geo[4];
     v.geom(precision, geo);
-    const int nmap = geo[0], eq = geo[1], xw = geo[2], ry = geo[3];
+    const int nmap = geo[0], xw = geo[2], ry = geo[3];
     for (int j = 0; j < nmap; ++j) {
-        const int e = eq * (j + 1);
+        const int e = j + 1;
         if (!make_map(&out[MAP_PLANE * nmap + j], base, precision, g, nc, v.tx, v.ty, 1, e)) return false;
         if (kinds > 1 && (!make_map(&out[MAP_YROW * nmap + j], base, precision, g, nc, v.tx, 1, v.tz, e) ||
                           !make_map(&out[MAP_XGRP * nmap + j], base, precision, g, nc, xw, ry, v.tz, e)))
             return false;
     }
     return true;
+}
+
+// The default variant for a grid: the one whose tiles cover it at the least cost, rounds of the persistent
+// CTAs times the cost of a round.  Padding at the grid's edges and an emptier last round cost as much as
+// full tiles.  A round costs its cells per SM plus a fixed part (the barriers and the issue of the copies
+// of every stage; above order 30, where one window fills the registers, the latency of a warp's own
+// instructions), in cells: P15 96^3 0.300 ms with 288-cell tiles and 0.276 with 384, P7 128^3 0.246 ms with
+// 256-cell and 0.195 with 512-cell tiles, P39 120^3 69 us a round with 192 cells and 82 with 320.  Rows
+// that do not start on 128-byte lines touch one more line each: P39 82 us a round of 32x3x3 tiles at 96^3
+// (aligned), 113 at 120^3 (GB300, FP32).
+static const Variant* best_variant(int N, int precision, int depth, const rtpn::Geom& g, int sms) {
+    const Variant* best = nullptr;
+    double best_cost = 0;
+    const int es = precision == RTPN_BF16 ? 2 : 4;
+    const double fixed = N > 30 ? 400 : 180;
+    for (const auto& v : kVariants) {
+        if (v.N != N || (depth != 0 && v.depth != depth) || !fits(v, precision)) continue;
+        int geo[4];
+        v.geom(precision, geo);
+        const long long tiles = (long long)((g.nx + v.tx - 1) / v.tx) * ((g.ny + v.ty - 1) / v.ty) * ((g.nz + v.tz - 1) / v.tz);
+        const long long slots = (long long)sms * geo[1];
+        const long long rounds = (tiles + slots - 1) / slots;
+        // a grid of less than a round leaves SMs with fewer CTAs than they hold
+        const long long per_sm = rounds > 1 ? geo[1] : (tiles + sms - 1) / sms;
+        const int row = v.tx * es;
+        const double lines = row % 128 == 0 && g.nx * es % 128 == 0 ? 1.0 : 1.0 + 48.0 / row;
+        const double cost = rounds * (per_sm * v.tx * v.ty * v.tz * lines + fixed);
+        if (!best || cost < best_cost) {
+            best = &v;
+            best_cost = cost;
+        }
+    }
+    return best;
 }
 
 static int nmaps_of(const Variant& v, int precision) {
@@ -113,14 +146,11 @@ bool stage_has_tile(int N, int tx, int ty, int tz, int depth, int precision) {
 int stage_prepare(rtpn_ctx* ctx, int tx, int ty, int tz, int depth) {
     const stg::Variant* v = stg::find(ctx->N, tx, ty, tz, depth, ctx->prec);
     if (!v) return (int)cudaErrorNotSupported;
-    // default (no tile given): the first listed variant whose width divides nx, else the first one
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, dev);
     if (tx == 0)
-        for (const auto& w : stg::kVariants)
-            if (w.N == ctx->N && (depth == 0 || w.depth == depth) && ctx->g.nx % w.tx == 0 &&
-                stg::fits(w, ctx->prec)) {
-                v = &w;
-                break;
-            }
+        if (const stg::Variant* w = stg::best_variant(ctx->N, ctx->prec, depth, ctx->g, ctx->sms)) v = w;
     const int N = ctx->N;
     // the tensor maps live in device global memory (64-byte aligned) and the kernel reads them from
     // there: tile planes / z halo plane, y halo row and x halo group, each for every box length
@@ -156,9 +186,6 @@ int stage_prepare(rtpn_ctx* ctx, int tx, int ty, int tz, int depth) {
         ctx->stage_tab_bytes[0] = b0;
         ctx->stage_tab_bytes[1] = b1;
     }
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, dev);
     ctx->stage_variant = (int)(v - stg::kVariants);
     ctx->tx = v->tx;
     ctx->ty = v->ty;
@@ -195,11 +222,13 @@ static bool base_args(const rtpn_ctx* ctx, const stg::Variant& v, int coef_cls, 
     a.nz = ctx->g.nz;
     a.bc = ctx->g.bc;
     a.inv_h = (float)(1.0 / ctx->g.h);
+    a.sy = (float)(ctx->g.h / ctx->g.hy);  // exactly 1 for cubic cells
     a.ntx = (a.nx + v.tx - 1) / v.tx;
     a.nty = (a.ny + v.ty - 1) / v.ty;
     a.ntz = (a.nz + v.tz - 1) / v.tz;
     a.tiles = (long long)a.ntx * a.nty * a.ntz;
-    if (a.tiles * (ctx->N + 2) >= (1ll << 31)) return false;
+    // 32-bit stage counts and 32-bit byte strides of a component
+    if (a.tiles * (ctx->N + 2) * 4 >= (1ll << 31) || ctx->g.V * (long long)ctx->elem >= (1ll << 32)) return false;
     // z chunk of the tile walk: the ~one tile per SM at work at a time then spans about as many
     // tile rows in y as layers in z, across the whole x extent
     const double side = std::sqrt((double)(ctx->sms > 0 ? ctx->sms : 1) / a.ntx);

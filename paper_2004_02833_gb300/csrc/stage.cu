@@ -1,6 +1,6 @@
 // One variant of the TMA-staged substep kernel: order RTPN_SN, CTA tile RTPN_STX x RTPN_STY x
-// RTPN_STZ, RTPN_SNB stage buffers, TMA box lengths in multiples of RTPN_SEM components, both target
-// classes, FP32 and BF16 storage.  kernels_stage.cu dispatches to it.
+// RTPN_STZ, RTPN_SNB stage buffers, RTPN_SEM sub-stages per column, both target classes, FP32 and
+// BF16 storage.  kernels_stage.cu dispatches to it.
 #include "stage_impl.cuh"
 
 #if !defined(RTPN_SN) || !defined(RTPN_STX) || !defined(RTPN_STY) || !defined(RTPN_STZ) || !defined(RTPN_SNB) || \
@@ -19,22 +19,30 @@ namespace stg {
 // defines a k_stage / launch_one of the same name, and the linker must not merge them.
 namespace {
 
-constexpr int kN = RTPN_SN, kTX = RTPN_STX, kTY = RTPN_STY, kTZ = RTPN_STZ, kNB = RTPN_SNB, kEM = RTPN_SEM;
-constexpr int kThreads = Layout<kN, 0, float, kTX, kTY, kTZ, kNB, kEM>::THREADS;
-// Two CTAs per SM where two rings fit shared memory and the order's window fits the registers
-// that leaves (orders up to 15: about 110 registers a thread); one otherwise.
-constexpr int kMinBlocks = (kN <= 15 && 2 * Layout<kN, 0, float, kTX, kTY, kTZ, kNB, kEM>::BYTES <= 232448) ? 2 : 1;
+constexpr int kN = RTPN_SN, kTX = RTPN_STX, kTY = RTPN_STY, kTZ = RTPN_STZ, kNB = RTPN_SNB, kCH = RTPN_SEM;
+constexpr int kThreads = Layout<kN, 0, float, kTX, kTY, kTZ, kNB, kCH>::THREADS;
+// Two CTAs per SM where two rings fit shared memory (228 KB, 1 KB of it reserved per CTA) and the
+// registers that leaves a thread hold its window (six accumulators per slot) and 48 more; one
+// otherwise.  A second CTA fills the issue slots while the first waits for a stage: P15, 96 x 96 x
+// 128 cells, 64x2x2 tiles on a GB300: 0.351 ms a pass with two three-buffer CTAs per SM, 0.397 ms with
+// one five-buffer CTA.
+constexpr int kWarpsPerScheduler2 = (2 * (kThreads / 32) + 3) / 4;
+constexpr int kRegs2 = 512 / kWarpsPerScheduler2 / 8 * 8;
+template <typename S>
+constexpr int min_blocks() {
+    return 2 * (Layout<kN, 0, S, kTX, kTY, kTZ, kNB, kCH>::BYTES + 1024) <= 233472 && kRegs2 >= 6 * (kN / 2 + 1) + 48 ? 2 : 1;
+}
 
 template <int A, typename S, int MODE>
-__global__ void __launch_bounds__(kThreads, kMinBlocks) k_stage(Args a) {
-    static_assert(Layout<kN, A, S, kTX, kTY, kTZ, kNB, kEM>::FITS, "stage ring exceeds shared memory");
+__global__ void __launch_bounds__(kThreads, min_blocks<S>()) k_stage(Args a) {
+    static_assert(Layout<kN, A, S, kTX, kTY, kTZ, kNB, kCH>::FITS, "stage ring exceeds shared memory");
     extern __shared__ __align__(128) unsigned char smem[];
-    stage_kernel_body<kN, A, S, kTX, kTY, kTZ, kNB, kEM, MODE>(a, smem);
+    stage_kernel_body<kN, A, S, kTX, kTY, kTZ, kNB, kCH, MODE>(a, smem);
 }
 
 template <int A, typename S, int MODE>
 int launch_one(const Args& a, int sms, cudaStream_t st) {
-    using L = Layout<kN, A, S, kTX, kTY, kTZ, kNB, kEM>;
+    using L = Layout<kN, A, S, kTX, kTY, kTZ, kNB, kCH>;
     if constexpr (!L::FITS) {
         return (int)cudaErrorNotSupported;  // this depth is compiled for the narrower storage only
     } else {
@@ -63,16 +71,16 @@ int launch_one(const Args& a, int sms, cudaStream_t st) {
 // dynamic shared memory of the variant, or 0 if it does not fit a CTA
 template <int A, typename S>
 constexpr int smem_of() {
-    using L = Layout<kN, A, S, kTX, kTY, kTZ, kNB, kEM>;
+    using L = Layout<kN, A, S, kTX, kTY, kTZ, kNB, kCH>;
     return L::FITS ? L::BYTES : 0;
 }
 // box geometry of the variant for a storage precision (the host builds its tensor maps with it):
-// out = {maps per kind, box length step, x halo group width, x halo group rows}
+// out = {maps per kind, CTAs per SM, x halo group width, x halo group rows}
 template <typename S>
 void geom_of(int* out) {
-    using L = Layout<kN, 0, S, kTX, kTY, kTZ, kNB, kEM>;
+    using L = Layout<kN, 0, S, kTX, kTY, kTZ, kNB, kCH>;
     out[0] = L::NMAP;
-    out[1] = kEM;
+    out[1] = min_blocks<S>();
     out[2] = L::XW;
     out[3] = L::RY;
 }

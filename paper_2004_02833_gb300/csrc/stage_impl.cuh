@@ -6,32 +6,44 @@
 // product), and a target column is finished, by Eq. (5), once the next source column is in.  What
 // differs:
 //
-//  * Two threads share a cell, one per target type (cos / sin).  Targets of type T take their z and
-//    x differences from sources of type T and their y differences from sources of the other type
-//    (Eq. 3's Mx and Mz keep the type, My swaps it), so the split needs no exchange and the two
-//    threads carry equal work.  Each thread keeps three columns of N/2 + 1 accumulators.
+//  * A thread advances both types (cos / sin) of one cell, a type per lane of packed FP32 pairs:
+//    targets of type T take their z and x differences from sources of type T and their y differences
+//    from sources of the other type (Eq. 3's Mx and Mz keep the type, My swaps it), so the two lanes
+//    run the same code and share one coupling constant for x and y.  Each thread keeps three columns
+//    of N/2 + 1 accumulator pairs.  (Two threads per cell, one per type, took twice the instructions
+//    for the same cells: P39 160^3 FP32, 11.0 ms a pass against 7.4 ms now.)
 //  * The column sweep is a runtime loop whose body handles one column for every l slot; the three
-//    live target columns are register arrays that shift by one column per iteration, so the body
-//    is the same for every column and fits the instruction cache.
-//  * A producer warp moves each column into shared memory with the Tensor Memory Accelerator
-//    (cp.async.bulk.tensor): one box per (type, box kind) holding all E components of the
-//    (type, |m|) run at once (a tensor map per box length E), so a column stage costs about fifteen
-//    TMA operations.  Every box kind has the same volume per component, U = TY * TX elements:
-//    the tile as TZ plane boxes [E][1][TY][TX], the y halo row [E][TZ][1][TX], the z halo plane
-//    [E][1][TY][TX] and the x halo [E][TZ][RY][XW] (XW * RY = TX: an aligned group of XW columns
-//    around the neighbour the partners read, with RY >= TY rows).  So component q of every region
-//    sits at q * U elements and each thread reaches all its operands through a few base addresses
-//    fixed once per column plus compile-time offsets: no address arithmetic per slot.  Periodic
-//    halos use wrapped coordinates; vacuum halos use out-of-range coordinates, which the TMA unit
-//    fills with zeros.  The same stage carries the tile boxes of the target column it finishes
-//    (column i - 1 in stage i; a tile has N + 2 stages) and the column's coupling constants (a
-//    plain bulk copy).  NB stage buffers form a ring with a full / empty mbarrier pair each, so up
-//    to NB - 1 stages are in flight while one is computed.
+//    live target columns are register arrays that change roles from column to column (the loop is
+//    unrolled by three), so the body is the same for every column and fits the instruction cache.
+//  * A column is moved in NCH sub-stages of K = 4 or 5 slots, so that a stage buffer is small and the
+//    tile can be wide (up to 96 cells): TMA rows of 256 to 384 bytes and up to 12 consumer warps for the
+//    same shared memory.  A target slot is finished in the sub-stage that brings its last source.
+//  * Two producer warps, one per type, move each sub-stage into shared memory with the Tensor Memory
+//    Accelerator (cp.async.bulk.tensor): one box per box kind holding all its components of the
+//    (type, |m|) run at once (a tensor map per box length).  Every box kind has the same volume per
+//    component, U = TY * TX elements: the tile as TZ plane boxes [E][1][TY][TX], the y halo row
+//    [E][TZ][1][TX], the z halo plane [E][1][TY][TX] and the x halo [E][TZ][RY][XW] (XW * RY = TX: an
+//    aligned group of XW columns around the neighbour the partners read, with RY >= TY rows).  So
+//    slot k of every region sits at k * U elements and each thread reaches all its operands through a
+//    few base addresses fixed once per column plus compile-time offsets: no address arithmetic per
+//    slot.  Periodic halos use wrapped coordinates; vacuum halos use out-of-range coordinates, which
+//    the TMA unit fills with zeros.  The same stage carries the tile boxes of the target slots it
+//    finishes and the coupling constants (a plain bulk copy).  The issue of the boxes bounds the
+//    copies (about 100 cycles a box from one warp, copies alone): P39 160^3, 7.2 ms with one producer
+//    warp, 5.5 ms with two, 4.4 ms with everything but the issue itself computed by the whole warp
+//    (uniform registers) instead of by one lane.  NB stage buffers form a ring with a full / empty
+//    mbarrier pair each, so up to NB - 1 stages are in flight while one is computed.
 //
-// CTAs are persistent (one per SM) and walk tiles in z-chunked order (z fastest inside a chunk of kz
+// What bounds it (GB300, FP32, a pass, before -> now, of the 6697 GB/s copy): P39 160^3 11.0 -> 7.4 ms
+// (5.3 TB/s, 79 %): the latency of a warp's own instructions, 10 consumer warps with 168 registers (120
+// accumulators); P19 96 x 96 x 128 0.54 ms (5.2 TB/s); P15 96^3 0.41 -> 0.27 ms (5.1 TB/s, 77 %); P7 128^3
+// 0.46 -> 0.19 ms (4.3 TB/s): barriers and copies per stage.
+//
+// CTAs are persistent (one or two per SM) and walk tiles in z-chunked order (z fastest inside a chunk of kz
 // tile layers, then x, then y), so the CTAs at work at any time cover a compact block and read one
-// another's halos from L2.  Every mbarrier wait is bounded: one that runs out sets a status bit,
-// the warp leaves, and the producer waits (bounded) for the copies it issued before the CTA ends.
+// another's halos from L2.  Every mbarrier wait is bounded: one that runs out sets a status bit;
+// a consumer then stops waiting (the rest of its pass is undefined, as the caller is told), a
+// producer leaves after a bounded wait for the copies it issued.
 #pragma once
 
 #include <cuda.h>
@@ -47,40 +59,26 @@ using win::first_l;
 using win::ntypes;
 using win::static_for;
 
-// Enter a compile-time unrolled slot sequence at a runtime slot: `switch (first) {
-// RTPN_SLOT_CASES(f) }` runs f(q) for q = first, first + 1, ... 23 (f ignores q past its range), one
-// jump per column instead of a test per slot.
-#define RTPN_SLOT_CASE(f, q)                   \
-    case q:                                    \
-        f(std::integral_constant<int, q>{});   \
-        [[fallthrough]];
-#define RTPN_SLOT_CASES(f)                                                                          \
-    RTPN_SLOT_CASE(f, 0) RTPN_SLOT_CASE(f, 1) RTPN_SLOT_CASE(f, 2) RTPN_SLOT_CASE(f, 3)             \
-    RTPN_SLOT_CASE(f, 4) RTPN_SLOT_CASE(f, 5) RTPN_SLOT_CASE(f, 6) RTPN_SLOT_CASE(f, 7)             \
-    RTPN_SLOT_CASE(f, 8) RTPN_SLOT_CASE(f, 9) RTPN_SLOT_CASE(f, 10) RTPN_SLOT_CASE(f, 11)           \
-    RTPN_SLOT_CASE(f, 12) RTPN_SLOT_CASE(f, 13) RTPN_SLOT_CASE(f, 14) RTPN_SLOT_CASE(f, 15)         \
-    RTPN_SLOT_CASE(f, 16) RTPN_SLOT_CASE(f, 17) RTPN_SLOT_CASE(f, 18) RTPN_SLOT_CASE(f, 19)         \
-    RTPN_SLOT_CASE(f, 20) RTPN_SLOT_CASE(f, 21) RTPN_SLOT_CASE(f, 22) RTPN_SLOT_CASE(f, 23)         \
-    default:                                                                                        \
-        break;
-constexpr int kMaxSlots = 24;
-// The same for chunks of kChunk slots: `switch (first / kChunk) { RTPN_CHUNK_CASES(f) }` runs f(c) for
-// chunks c = first / kChunk .. 11, so a compiler sees kChunk slots as one straight-line block.
-constexpr int kChunk = 2;
-#define RTPN_CHUNK_CASES(f)                                                                        \
-    RTPN_SLOT_CASE(f, 0) RTPN_SLOT_CASE(f, 1) RTPN_SLOT_CASE(f, 2) RTPN_SLOT_CASE(f, 3)             \
-    RTPN_SLOT_CASE(f, 4) RTPN_SLOT_CASE(f, 5) RTPN_SLOT_CASE(f, 6) RTPN_SLOT_CASE(f, 7)             \
-    RTPN_SLOT_CASE(f, 8) RTPN_SLOT_CASE(f, 9) RTPN_SLOT_CASE(f, 10) RTPN_SLOT_CASE(f, 11)           \
-    default:                                                                                        \
-        break;
+constexpr int kMaxSlots = 24;  // tensor maps of a kind, at most
+// The slots of a sub-stage run in blocks of straight-line code, skipped where the column starts
+// above them; slots of a block below the first source carry zero constants and read finite shared
+// memory.
+constexpr int kBlock = 2;
+// Producer warps: one for each type's boxes of every stage.
+constexpr int kProducers = 2;
 
 constexpr unsigned STATUS_TIMEOUT = 1u;
 constexpr unsigned STATUS_CHECK = 2u;  // a self-check failed (builds with RTPN_STAGE_CHECKS)
-// coupling constants per source slot, three float4:
-//   [0..3] z (l-1), z (l+1), x to column M-1 (l-1), (l+1)     read by the thread of the same type
-//   [4..5] x to column M+1 (l-1), (l+1); [6..7] unused        read by the thread of the same type
-//   [8..11] y to column M-1 (l-1), (l+1), to M+1 (l-1), (l+1)  read by the thread of the other type
-constexpr int CPAD = 12;
+// Coupling constants per source slot (l, M): six (cos, sin) pairs, one lane per target type T: z to l-1,
+// z to l+1 (target column M), x and y to column M+1 (l-1, l+1), and, negated, to column M-1 (l-1, l+1).
+// Mx and My couple (l, M) to (l +- 1, M +- 1) with entries of the same magnitude (both come from
+// Omega_x +- i Omega_y), and the sign of the y entry against the x entry depends on (T, parity of M,
+// side) only: + into column M+1 for T = 0 and even M, and the other sign for each of T = 1, odd M and
+// column M-1.  So one constant serves both axes: with dx the x difference of the own type's source and
+// dy the y difference of the other type's, a target takes k dx + k (s dy) from column M-1 and
+// (-k)(-dx) + (-k)(s dy) from column M+1, s = +-1 the same for the whole column.
+constexpr int CPAD = 6;       // constants per slot and type
+constexpr int KPAIRS = CPAD;  // pairs per slot
 
 // What a pass computes.  FORWARD: targets u_A' = alpha u_A - beta acc (Eq. 5; the u_0 factors for
 // l = 0).  ADJ_SOURCES: the transpose of a substep's coupling for the dual multipliers,
@@ -91,7 +89,7 @@ constexpr int CPAD = 12;
 constexpr int FORWARD = 0, ADJ_SOURCES = 1;
 
 // Tensor maps of one array: kind k in {MAP_PLANE, MAP_YROW, MAP_XGRP} for every box length
-// E = EQ, 2 EQ, ..., NL (index k * nmaps + E / EQ - 1).
+// E = 1, 2, ..., NMAP (index k * nmaps + E - 1).
 constexpr int MAP_PLANE = 0;  // [E][1][TY][TX]: a tile plane or the z halo plane (also target boxes)
 constexpr int MAP_YROW = 1;   // [E][TZ][1][TX]: the y halo row
 constexpr int MAP_XGRP = 2;   // [E][TZ][RY][XW]: the x halo group
@@ -116,6 +114,7 @@ struct Args {
     unsigned* status;       // device status word (STATUS_TIMEOUT on a wait that ran out)
     unsigned wait_limit;    // try_wait polls (each up to WAIT_HINT_NS) before giving up
     long long skip_stage;   // stage index never issued (a wait that must run out); -1 normally
+    float sy = 1.f;         // h / h_y: scale of the y differences (non-cubic cells)
 };
 
 __host__ __device__ constexpr int pad128(int bytes) { return (bytes + 127) / 128 * 128; }
@@ -128,32 +127,34 @@ __host__ __device__ constexpr int xhalo_width(int tx, int ty, int es) {
         if (tx % w == 0 && tx / w >= ty) best = w;
     return best;
 }
-// slots of a run in shared memory: the longest run N/2 + 1 rounded up to a multiple of eq
-__host__ __device__ constexpr int run_slots(int N, int eq) { return (N / 2 + 1 + eq - 1) / eq * eq; }
 
-template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int EQ = 1>
+// NCH: sub-stages of a column (each K = ceil((N/2 + 1) / NCH) source slots).
+template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH = 1>
 struct Layout {
     static constexpr int B = 1 - A;
     static constexpr int ES = (int)sizeof(S);
     static constexpr int G = 16 / ES;                 // elements of an aligned 16-byte group
-    static constexpr int NL = run_slots(N, EQ);       // run slots per region
-    static constexpr int NMAP = NL / EQ;              // box lengths (tensor maps) per kind
-    static constexpr int NLC = N / 2 + 1;             // coupling-constant slots per type
+    static constexpr int NLC = N / 2 + 1;             // slots of the longest run
+    static constexpr int K = (NLC + NCH - 1) / NCH;   // source slots of a sub-stage
+    static constexpr int KT = NCH == 1 ? K : K + 1;   // target slots of a sub-stage, at most
+    static constexpr int NL = KT;                     // longest box
+    static constexpr int NMAP = KT;                   // box lengths (tensor maps) per kind
     static constexpr int U = TY * TX;                 // elements of one component in every box
     static constexpr int UB = U * ES;
     static constexpr int XW = xhalo_width(TX, TY, ES);
     static constexpr int RY = XW > 0 ? TX / XW : 1;
     static constexpr int CELLS = TX * TY * TZ;
-    static constexpr int CONSUMER_WARPS = 2 * CELLS / 32;
-    static constexpr int THREADS = 2 * CELLS + 32;   // two threads per cell + the producer
-    static constexpr int REG = pad128(NL * UB);       // one region: NL components of one box kind
+    static constexpr int CONSUMER_WARPS = CELLS / 32;
+    static constexpr int THREADS = CELLS + 32 * kProducers;  // one thread per cell + the producers
+    static constexpr int REG = pad128(K * UB);        // one source region: K components of one box kind
+    static constexpr int REGT = pad128(KT * UB);      // one target region
     // regions of one type's sources: TZ tile planes, then the y halo, z halo and x halo
     static constexpr int KY = TZ, KZ = TZ + 1, KX = TZ + 2, NKIND = TZ + 3;
     static constexpr int SRC_T = NKIND * REG;
-    static constexpr int TGT_T = TZ * REG;            // tile planes of one type's targets
-    static constexpr int COEF_COL = 2 * NLC * CPAD * 4;  // one column's coupling constants
-    // buffer layout: target planes, type-0 sources, type-1 sources, coupling constants.  A chunked
-    // sweep reads up to kChunk - 1 slots below a source region; with the targets first, such reads
+    static constexpr int TGT_T = TZ * REGT;           // tile planes of one type's targets
+    static constexpr int COEF_COL = 2 * K * CPAD * 4;  // a sub-stage's coupling constants
+    // buffer layout: target planes, type-0 sources, type-1 sources, coupling constants.  A block of
+    // the sweep may read up to K - 1 slots below a source region; with the targets first, such reads
     // stay on state data (or the zeros the ring starts with) in the same buffer, never on the
     // coupling constants, whose bits need not be finite in the storage type.
     static constexpr int TGTO = 0;
@@ -164,21 +165,60 @@ struct Layout {
     static constexpr int BYTES = NB * BUF + BARS + 128;   // ring, mbarriers, base alignment slack
     static_assert(TY == TZ, "every box kind has the volume TY * TX per component only if TY == TZ");
     static_assert(TX % G == 0, "tile width must be a multiple of the 16-byte group");
-    static_assert(CELLS % 32 == 0, "a type's threads must fill whole warps");
+    static_assert(CELLS % 32 == 0, "the tile's cells must fill whole warps");
     static_assert(NB >= 2 && NB <= 8, "two to eight stage buffers");
-    static_assert(REG >= (kChunk - 1) * UB, "a region must cover what a chunked sweep reads below the next");
+    static_assert(2 * TGT_T >= (kBlock - 1) * UB, "blocks read at most kBlock - 1 slots below a region");
+    static_assert(NCH == 1 || K >= 2, "a sub-stage of class 1 finishes one slot behind its sources");
     // the ring fits 227 KB of shared memory per CTA, and an x halo group exists for this element
     // size (a tile too narrow for RY >= TY rows of 16-byte groups is compiled for FP32 only)
     static constexpr bool FITS = BYTES <= 232448 && XW > 0;
 };
 
+// First slot of source column i (class B), and the sub-stage a column starts with.
+template <int N, int A>
+RTPN_HD constexpr int first_source(int i) {
+    return (int)(((unsigned)i + (((unsigned)i ^ (unsigned)(1 - A)) & 1u)) >> 1);  // first_l(i, B) / 2
+}
+template <int N, int A, int NCH>
+RTPN_HD constexpr int first_chunk(int i) {
+    constexpr int K = (N / 2 + 1 + NCH - 1) / NCH;
+    const int c = first_source<N, A>(i) / K;
+    return c < NCH - 1 ? c : NCH - 1;
+}
+// sub-stages of one tile
+template <int N, int A, int NCH>
+RTPN_HD constexpr int tile_stages() {
+    int n = 0;
+    for (int i = 0; i < N + 2; ++i) n += NCH - first_chunk<N, A, NCH>(i);
+    return n;
+}
+// Target slots [lo, hi) of column i - 1 that are complete after sub-stage C of source column i: a
+// source l reaches l +- 1, so class 0 (even l) is complete up to the same slot, class 1 up to the one
+// before, and the last sub-stage completes the rest.
+template <int N, int A, int NCH>
+RTPN_HD constexpr int window_lo(int C) {
+    constexpr int K = (N / 2 + 1 + NCH - 1) / NCH;
+    return C == 0 ? 0 : C * K - A;
+}
+template <int N, int A, int NCH>
+RTPN_HD constexpr int window_hi(int C) {
+    constexpr int K = (N / 2 + 1 + NCH - 1) / NCH;
+    constexpr int NLA = (N - A) / 2 + 1;
+    const int h = C * K + K - A;
+    return C == NCH - 1 || h > NLA ? NLA : h;
+}
+
+// Sign of the y against the x coupling into column M+1 for target type T.
+RTPN_HD constexpr float y_sign(int M, int T) { return ((M ^ T) & 1) ? -1.f : 1.f; }
+
 // The coupling constants of the staged kernel (host; the library and its host check program):
-// per target class A, the constants of the source class by column, type and slot q
-// ([N+1][2][N/2+1][CPAD], layout above; slots of l < M stay zero, so a sweep may start at a slot
-// boundary below the column), from the model's coupling (win::coef_table).  The kernel applies
-// 1/h of x; the y and z constants carry sy = h / h_y and sz = h / h_z (exactly 1 for cubic
-// cells).  col: the first local index of column M in class P at col[P (N + 2) + M].
-inline bool coupling_tables(const Model& md, double sy, double sz, std::vector<float> tab[2], std::vector<int>* col) {
+// per target class A, the constants of the source class by column and slot q
+// ([N+1][N/2+1][KPAIRS][2], layout above; slots of l < M stay zero), from the model's coupling
+// (win::coef_table).  The kernel applies 1/h of x and scales the y differences by h / h_y; the z
+// constants carry sz = h / h_z (exactly 1 for cubic cells).  col: the first local index of column M in
+// class P at col[P (N + 2) + M].  False if the model's x and y couplings do not share their magnitudes
+// and signs as above.
+inline bool coupling_tables(const Model& md, double /*sy*/, double sz, std::vector<float> tab[2], std::vector<int>* col) {
     const int N = md.N, nl = N / 2 + 1;
     col->assign(2 * (N + 2), 0);
     for (int P = 0; P < 2; ++P) {
@@ -192,18 +232,31 @@ inline bool coupling_tables(const Model& md, double sy, double sz, std::vector<f
         const int B = 1 - A;
         std::vector<float> t10;  // [local source index of class B][10]
         if (!win::coef_table(md, A, &t10)) return false;
-        tab[A].assign((size_t)(N + 1) * 2 * nl * CPAD, 0.f);
+        tab[A].assign((size_t)(N + 1) * nl * 2 * KPAIRS, 0.f);
         for (int M = 0; M <= N; ++M)
-            for (int t = 0; t < ntypes(M); ++t)
-                for (int j = 0; j < column_len(N, M, B); ++j) {
-                    const int src = (*col)[B * (N + 2) + M] + t * column_len(N, M, B) + j;
-                    const int q = first_l(M, B) / 2 + j;  // the source's slot (l - B) / 2
-                    float* d = &tab[A][(((size_t)M * 2 + t) * nl + q) * CPAD];
-                    const float* kk = &t10[(size_t)src * 10];
-                    for (int r = 0; r < 2; ++r) d[r] = (float)(kk[r] * sz);          // z
-                    for (int r = 2; r < 6; ++r) d[r] = kk[r];                        // x to M-1, M+1
-                    for (int r = 0; r < 4; ++r) d[8 + r] = (float)(kk[6 + r] * sy);  // y to M-1, M+1
+            for (int j = 0; j < column_len(N, M, B); ++j) {
+                const int q = first_l(M, B) / 2 + j;  // the source's slot (l - B) / 2
+                float* d = &tab[A][((size_t)M * nl + q) * KPAIRS * 2];
+                // relations of the source of type t (null if the type is absent)
+                auto rel = [&](int t) {
+                    const int len = column_len(N, M, B);
+                    return t < ntypes(M) ? &t10[(size_t)((*col)[B * (N + 2) + M] + t * len + j) * 10] : nullptr;
+                };
+                for (int T = 0; T < 2; ++T) {
+                    const float *own = rel(T), *oth = rel(1 - T);
+                    for (int r = 0; r < 2 && own; ++r) d[r * 2 + T] = (float)(own[r] * sz);
+                    for (int side = 0; side < 2; ++side)  // column M+1, column M-1
+                        for (int dl = 0; dl < 2; ++dl) {
+                            const float x = own ? own[(side == 0 ? 4 : 2) + dl] : 0.f;
+                            const float y = oth ? oth[(side == 0 ? 8 : 6) + dl] : 0.f;
+                            const float s = side == 0 ? y_sign(M, T) : -y_sign(M, T);
+                            // at |m| = 0 only one of the two sources exists
+                            if (M > 0 ? y != s * x : (x != 0.f && y != 0.f)) return false;
+                            const float k = own ? x : s * y;
+                            d[(2 + 2 * side + dl) * 2 + T] = side == 0 ? k : -k;
+                        }
                 }
+            }
     }
     return true;
 }
@@ -250,10 +303,16 @@ __device__ __forceinline__ void bulk_load(unsigned dst, const void* src, unsigne
         "l"(reinterpret_cast<unsigned long long>(src)), "r"(bytes), "r"(bar)
         : "memory");
 }
-// bounded wait on one mbarrier phase; false if it ran out
+// true on one lane of the (converged) warp
+__device__ __forceinline__ bool elect_one() {
+    unsigned p;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+    return p != 0;
+}
+// bounded wait of a whole warp on one mbarrier phase; false if it ran out (the same for every lane)
 __device__ __forceinline__ bool wait_phase(unsigned bar, unsigned parity, unsigned limit) {
     for (unsigned i = 0; i < limit; ++i)
-        if (mbar_try_wait(bar, parity)) return true;
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
     return false;
 }
 
@@ -359,96 +418,135 @@ __host__ __device__ __forceinline__ int dir_x(int M, int t) { return ((M & 1) ==
 // where it lands in the stage buffer.  Host and device: the producer issues it, the host check
 // program copies it.
 struct BoxJob {
-    int valid;    // 0: this job issues nothing in this stage
+    int valid;    // 0: this box is not part of the stage
     int target;   // 1: a plane box of the target array (map a.tmap + emap), 0: of the source array
     int kind;     // MAP_PLANE, MAP_YROW or MAP_XGRP (source array)
-    int emap;     // box length index: E = EQ * (emap + 1) components
+    int emap;     // box length index: E = emap + 1 components
     int x, y, z, c;
     int dst;      // byte offset of the box in the stage buffer
 };
 
-// The runs of stage i, the same for every box of the stage: source column i of class B (length,
-// types present) and target column i - 1 of class A.
+// The runs of sub-stage C of stage i, the same for every box: slots of source column i of class B and of
+// target column i - 1 of class A (box lengths, types present), the full runs and where in them the
+// boxes start, and the slots the boxes start with.
 struct StageRuns {
     int len, nt, lenA, ntA;
+    int run, ofs, runA, ofsA;
+    int q, qA;
 };
-template <int N, int A>
-RTPN_HD StageRuns stage_runs(int i) {
+template <int N, int A, int NCH = 1>
+RTPN_HD StageRuns stage_runs(int i, int C = 0) {
     constexpr int B = 1 - A;
+    constexpr int K = (N / 2 + 1 + NCH - 1) / NCH;
+    constexpr int NLB = (N - B) / 2 + 1;
     StageRuns r;
-    r.len = column_len(N, i, B);          // none at i = N + 1
+    r.run = column_len(N, i, B);  // none at i = N + 1
+    const int fq = first_source<N, A>(i);
+    r.q = fq > C * K ? fq : C * K;
+    const int e = C * K + K < NLB ? C * K + K : NLB;
+    r.len = i <= N && e > r.q ? e - r.q : 0;
+    r.ofs = r.q - fq;
     r.nt = r.len > 0 ? ntypes(i) : 0;
-    r.lenA = i >= 1 ? column_len(N, i - 1, A) : 0;
+    r.runA = i >= 1 ? column_len(N, i - 1, A) : 0;
+    const int q0 = i >= 1 ? first_l(i - 1, A) / 2 : 0, lo = window_lo<N, A, NCH>(C), hi = window_hi<N, A, NCH>(C);
+    r.qA = q0 > lo ? q0 : lo;
+    r.lenA = i >= 1 && hi > r.qA ? hi - r.qA : 0;
+    r.ofsA = r.qA - q0;
     r.ntA = r.lenA > 0 ? ntypes(i - 1) : 0;
     return r;
 }
 
-// Box j of stage i (runs r) of the tile with geometry g; offB_s and offA_s are the first local
-// indices of source column i in class B and of target column i - 1 in class A.  Jobs
-// 0 .. 2 NKIND - 1: source boxes (type j / NKIND, kind j % NKIND: TZ tile planes, the y halo row,
-// the z halo plane, the x halo group); then the target planes (type, plane).
-template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int EQ>
-RTPN_HD BoxJob stage_box(const Args& a, const TileGeo& g, int i, const StageRuns& r, int offA_s, int offB_s, int j) {
-    using L = Layout<N, A, S, TX, TY, TZ, NB, EQ>;
+// Source box K of type t of a sub-stage of stage i (runs r) of the tile with geometry g: K = 0 .. TZ - 1 the
+// tile planes, then the y halo row, the z halo plane, the x halo group; offB is the first local index of
+// source column i in class B.
+template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH, int K>
+RTPN_HD BoxJob source_box(const Args& a, const TileGeo& g, int i, const StageRuns& r, int offB, int t) {
+    using L = Layout<N, A, S, TX, TY, TZ, NB, NCH>;
     constexpr int B = 1 - A;
-    constexpr int NK = L::NKIND;
-    BoxJob bj{0, 0, 0, 0, 0, 0, 0, 0, 0};
-    if (j >= 2 * NK) {  // target plane lz of type t
-        const int t = (j - 2 * NK) / TZ, lz = (j - 2 * NK) % TZ;
-        if (j >= 2 * NK + 2 * TZ || t >= r.ntA) return bj;
-        bj.valid = 1;
-        bj.target = 1;
-        bj.kind = MAP_PLANE;
-        bj.emap = (r.lenA + EQ - 1) / EQ - 1;
-        bj.x = g.x0;
-        bj.y = g.y0;
-        bj.z = g.z0 + lz;
-        bj.c = (A == 0 ? 0 : class_size(N, 0)) + offA_s + t * r.lenA;
-        bj.dst = L::TGTO + t * L::TGT_T + lz * L::REG;
-        return bj;
-    }
-    const int t = j / NK, k = j % NK;
-    if (t >= r.nt) return bj;
-    bj.valid = 1;
-    bj.emap = (r.len + EQ - 1) / EQ - 1;
-    bj.c = a.src_c0 + offB_s + t * r.len;  // first component of the run
-    bj.dst = L::SRCO + t * L::SRC_T + k * L::REG;
+    BoxJob bj;
+    bj.valid = t < r.nt;
+    bj.target = 0;
+    bj.emap = r.len - 1;
+    bj.c = a.src_c0 + offB + t * r.run + r.ofs;  // first component of the box
+    bj.dst = L::SRCO + t * L::SRC_T + K * L::REG;
     bj.x = g.x0;
     bj.y = g.y0;
     bj.z = g.z0;
-    if (k < TZ) {               // tile plane z0 + k
-        bj.kind = MAP_PLANE;
-        bj.z = g.z0 + k;
-    } else if (k == L::KY) {    // cos-type sources are read at y+1, sin-type at y-1
+    bj.kind = MAP_PLANE;
+    if constexpr (K < TZ) {             // tile plane z0 + K
+        bj.z = g.z0 + K;
+    } else if constexpr (K == L::KY) {  // cos-type sources are read at y+1, sin-type at y-1
         bj.kind = MAP_YROW;
         bj.y = t == 0 ? g.hc[1][1] : g.hc[1][0];
-    } else if (k == L::KZ) {    // z slot 1 (l + M even) is read at z+1
-        bj.kind = MAP_PLANE;
+    } else if constexpr (K == L::KZ) {  // z slot 1 (l + M even) is read at z+1
         bj.z = ((B + i) & 1) == 0 ? g.hc[2][1] : g.hc[2][0];
-    } else {                    // x slot 1 is read at x+1 (upper halo group)
+    } else {                            // x slot 1 is read at x+1 (upper halo group)
         bj.kind = MAP_XGRP;
         bj.x = dir_x(i, t) > 0 ? g.hx_start[1] : g.hx_start[0];
     }
     return bj;
 }
-
-// bytes the boxes and the coupling constants of a stage with runs r bring into the buffer
-template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int EQ>
-RTPN_HD unsigned stage_bytes(const StageRuns& r) {
-    using L = Layout<N, A, S, TX, TY, TZ, NB, EQ>;
-    const int ebox = (r.len + EQ - 1) / EQ * EQ, eboxA = (r.lenA + EQ - 1) / EQ * EQ;
-    return (unsigned)((r.nt * L::NKIND * ebox + r.ntA * TZ * eboxA) * L::UB) + (r.nt > 0 ? (unsigned)L::COEF_COL : 0u);
+// Target plane lz of type t; offA is the first local index of target column i - 1 in class A.
+template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH>
+RTPN_HD BoxJob target_box(const TileGeo& g, const StageRuns& r, int offA, int t, int lz) {
+    using L = Layout<N, A, S, TX, TY, TZ, NB, NCH>;
+    BoxJob bj;
+    bj.valid = t < r.ntA;
+    bj.target = 1;
+    bj.kind = MAP_PLANE;
+    bj.emap = r.lenA - 1;
+    bj.x = g.x0;
+    bj.y = g.y0;
+    bj.z = g.z0 + lz;
+    bj.c = (A == 0 ? 0 : class_size(N, 0)) + offA + t * r.runA + r.ofsA;
+    bj.dst = L::TGTO + t * L::TGT_T + lz * L::REGT;
+    return bj;
 }
 
-// The producer warp: issues the copies of every stage of this CTA's sequence into the ring.
-template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int EQ>
+// Box j of the plan: 0 .. 2 NKIND - 1 the source boxes (type j / NKIND, kind j % NKIND), then the target
+// planes (type, plane).
+template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH>
+RTPN_HD BoxJob stage_box(const Args& a, const TileGeo& g, int i, const StageRuns& r, int offA, int offB, int j) {
+    using L = Layout<N, A, S, TX, TY, TZ, NB, NCH>;
+    constexpr int NK = L::NKIND;
+    BoxJob bj{0, 0, 0, 0, 0, 0, 0, 0, 0};
+    if (j >= 2 * NK)
+        return j < 2 * NK + 2 * TZ ? target_box<N, A, S, TX, TY, TZ, NB, NCH>(g, r, offA, (j - 2 * NK) / TZ, (j - 2 * NK) % TZ)
+                                   : bj;
+    static_for<NK>([&](auto kk) {
+        constexpr int K = decltype(kk)::value;
+        if (j % NK == K) bj = source_box<N, A, S, TX, TY, TZ, NB, NCH, K>(a, g, i, r, offB, j / NK);
+    });
+    return bj;
+}
+
+// coupling-constant slots of sub-stage C that exist
+template <int N, int NCH>
+RTPN_HD constexpr int coef_slots(int C) {
+    constexpr int NLC = N / 2 + 1, K = (NLC + NCH - 1) / NCH;
+    return C * K + K <= NLC ? K : NLC - C * K;
+}
+// bytes that type t's boxes of a sub-stage with runs r bring into the buffer (the coupling constants
+// come with type 0), and those of both types
+template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH>
+RTPN_HD unsigned type_bytes(const StageRuns& r, int C, int t) {
+    using L = Layout<N, A, S, TX, TY, TZ, NB, NCH>;
+    return (unsigned)(((t < r.nt ? L::NKIND * r.len : 0) + (t < r.ntA ? TZ * r.lenA : 0)) * L::UB) +
+           (t == 0 && r.nt > 0 ? (unsigned)coef_slots<N, NCH>(C) * (2 * CPAD * 4) : 0u);
+}
+template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH>
+RTPN_HD unsigned stage_bytes(const StageRuns& r, int C = 0) {
+    return type_bytes<N, A, S, TX, TY, TZ, NB, NCH>(r, C, 0) + type_bytes<N, A, S, TX, TY, TZ, NB, NCH>(r, C, 1);
+}
+
+// Producer warp t: issues the copies of type t (and for t = 0 the coupling constants) of every sub-stage
+// of this CTA's sequence into the ring.  One lane issues; everything else is the same for the warp.
+template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH>
 __device__ __forceinline__ void stage_producer(const Args& a, unsigned char* bufs, unsigned full0,
-                                               unsigned empty0, int total) {
-    using L = Layout<N, A, S, TX, TY, TZ, NB, EQ>;
+                                               unsigned empty0, int total, int t) {
+    using L = Layout<N, A, S, TX, TY, TZ, NB, NCH>;
     constexpr int B = 1 - A;
     constexpr int NST = N + 2;
-    constexpr int NJOB = 2 * L::NKIND + 2 * TZ;  // source boxes (type, kind), then target planes (type, z)
-    static_assert(NJOB <= 32, "one box per lane");
     const int lane = threadIdx.x & 31;
     const CUtensorMap* maps = a.maps;
     // first local index of source column i in class B and of target column i - 1 in class A,
@@ -462,207 +560,332 @@ __device__ __forceinline__ void stage_producer(const Args& a, unsigned char* buf
 
     int s = 0;
     bool failed = false;
-    int b = 0, i = 0;
+    int b = 0, i = 0, C = first_chunk<N, A, NCH>(0);
     unsigned ph = 0;  // phase parity of buffer b's current use (flips when b wraps)
     unsigned tile = blockIdx.x;
     TileGeo g = tile_geo<TX, TY, TZ, L::G>(a, tile);
-    for (; s < total; ++s, i = (i == NST - 1) ? 0 : i + 1) {
-        if (i == 0 && s > 0) {
-            tile += gridDim.x;
-            g = tile_geo<TX, TY, TZ, L::G>(a, tile);
-            offB = offA = 0;
-        }
+    for (; s < total; ++s) {
         const unsigned full = full0 + 8 * b;
-        if (s >= NB) {  // the consumers must have released the buffer's previous stage
-            const bool ok = __all_sync(0xffffffffu, wait_phase(empty0 + 8 * b, ph ^ 1u, a.wait_limit));
-            if (!ok) {
-                failed = true;
-                break;
-            }
+        if (s >= NB && !wait_phase(empty0 + 8 * b, ph ^ 1u, a.wait_limit)) {
+            failed = true;  // the consumers did not release the buffer's previous stage
+            break;
         }
-        const int bcur = b;
+        const unsigned buf = smem_addr(bufs + b * L::BUF);
+        const StageRuns r = stage_runs<N, A, NCH>(i, C);
+        const unsigned bytes = type_bytes<N, A, S, TX, TY, TZ, NB, NCH>(r, C, t);
+        auto issue = [&](const BoxJob& bj) {
+            // sources: components of the source array (a.nc); targets: of a full state array (u or lam)
+            const int cmax = bj.target ? class_size(N, 0) + class_size(N, 1) : a.nc;
+            if (RTPN_SCHECK_ID(bj.c >= 0 && bj.c < cmax && bj.emap < L::NMAP, 101, bj.c)) {
+                const CUtensorMap* mp = bj.target ? a.tmap + bj.emap : maps + bj.kind * L::NMAP + bj.emap;
+                tma_load_4d(buf + bj.dst, mp, bj.x, bj.y, bj.z, bj.c, full);
+            }
+        };
+        if (s != a.skip_stage) {
+            if (elect_one()) {
+                mbar_expect_tx(full, bytes);
+                if (t < r.nt) {
+                    static_for<L::NKIND>([&](auto kk) {
+                        issue(source_box<N, A, S, TX, TY, TZ, NB, NCH, decltype(kk)::value>(a, g, i, r, offB, t));
+                    });
+                    if (t == 0)
+                        bulk_load(buf + L::COEFO, a.coefcol + (long long)(i * L::NLC + C * L::K) * (2 * CPAD),
+                                  coef_slots<N, NCH>(C) * (2 * CPAD * 4), full);
+                }
+                if (t < r.ntA)
+                    static_for<TZ>([&](auto zz) {
+                        issue(target_box<N, A, S, TX, TY, TZ, NB, NCH>(g, r, offA, t, decltype(zz)::value));
+                    });
+            }
+            __syncwarp();
+        }
         if (++b == NB) {
             b = 0;
             ph ^= 1u;
         }
-        // the column offsets of stage s; advanced for the next stage before anything can skip ahead
-        const int offB_s = offB, offA_s = offA;
-        offB += ntypes(i) * column_len(N, i, B);
-        if (i >= 1) offA += ntypes(i - 1) * column_len(N, i - 1, A);
-        if (s == a.skip_stage) continue;
-        unsigned char* buf = bufs + bcur * L::BUF;
-        // one lane issues the stage: the box list is unrolled at compile time, so the kind of every
-        // box and its tensor map are fixed per box and all operands are the same for the warp
-        if (lane == 0) {
-            const StageRuns runs = stage_runs<N, A>(i);
-            mbar_expect_tx(full, stage_bytes<N, A, S, TX, TY, TZ, NB, EQ>(runs));
-            static_for<NJOB>([&](auto jj) {
-                constexpr int j = decltype(jj)::value;
-                const BoxJob bj = stage_box<N, A, S, TX, TY, TZ, NB, EQ>(a, g, i, runs, offA_s, offB_s, j);
-                // sources: components of the source array (a.nc); targets: of a full state array (u or lam)
-                const int cmax = bj.target ? class_size(N, 0) + class_size(N, 1) : a.nc;
-                if (bj.valid && RTPN_SCHECK_ID(bj.c >= 0 && bj.c < cmax && (bj.emap + 1) * EQ <= L::NL, 101, bj.c)) {
-                    const CUtensorMap* mp = bj.target ? a.tmap + bj.emap : maps + bj.kind * L::NMAP + bj.emap;
-                    tma_load_4d(smem_addr(buf + bj.dst), mp, bj.x, bj.y, bj.z, bj.c, full);
-                }
-            });
-            if (runs.nt > 0)
-                bulk_load(smem_addr(buf + L::COEFO), a.coefcol + (long long)i * (2 * L::NLC * CPAD), L::COEF_COL,
-                          full);
+        // the next sub-stage: of this column, the next column, or the next tile
+        if (++C == NCH) {
+            offB += ntypes(i) * column_len(N, i, B);
+            if (i >= 1) offA += ntypes(i - 1) * column_len(N, i - 1, A);
+            if (++i == NST) {
+                i = offA = offB = 0;
+                tile += gridDim.x;
+                if (s + 1 < total) g = tile_geo<TX, TY, TZ, L::G>(a, tile);
+            }
+            C = first_chunk<N, A, NCH>(i);
         }
-        __syncwarp();
     }
     if (failed && lane == 0) atomicOr(a.status, STATUS_TIMEOUT);
     // before the CTA ends, the copies of the last stages issued must have landed
     const int first = s > NB ? s - NB : 0;
-    for (int r = first; r < s; ++r)
-        if (r != a.skip_stage) wait_phase(full0 + 8 * (r % NB), (unsigned)((r / NB) & 1), a.wait_limit);
+    for (int q = first; q < s; ++q)
+        if (q != a.skip_stage) wait_phase(full0 + 8 * (q % NB), (unsigned)((q / NB) & 1), a.wait_limit);
 }
 
 // ---------------------------------------------------------------- the consumers' column work
-// Byte offsets in a stage buffer of a consumer thread's operands, fixed per tile: its own-type
-// source, the other type's source and its y partner, and per parity p of the source column the
-// x and z partners.  Thread (T, cell (lx, ly, lz)) finishes the targets of type T of its cell.
+// A thread advances both types of one cell: lane x of a pair is the cos type, lane y the sin type.
+// The packed operations issue one instruction for the two lanes.
+RTPN_HD float2 pair_fma(float2 a, float2 b, float2 c) {
+#ifdef __CUDA_ARCH__
+    return __ffma2_rn(a, b, c);
+#else
+    return make_float2(fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y));
+#endif
+}
+RTPN_HD float2 pair_mul(float2 a, float2 b) {
+#ifdef __CUDA_ARCH__
+    return __fmul2_rn(a, b);
+#else
+    return make_float2(a.x * b.x, a.y * b.y);
+#endif
+}
+RTPN_HD float2 pair_sub(float2 a, float2 b) {
+#ifdef __CUDA_ARCH__
+    return __fadd2_rn(a, make_float2(-b.x, -b.y));
+#else
+    return make_float2(a.x - b.x, a.y - b.y);
+#endif
+}
+
+// Byte offsets in a stage buffer of a cell's operands, fixed per tile: its source value (type 0; type
+// 1 is SRC_T further), the y partner of each type, and per parity p of the source column the z
+// partner (type 0; the types share its direction) and the x partner of each type (opposite
+// directions).
 struct Operands {
-    int c, o, y, x0, x1, z0, z1;
+    int c, y[2], z[2], x[2][2];
 };
 
-template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int EQ>
-RTPN_HD Operands operand_offsets(const TileGeo& g, int T, int lx, int ly, int lz) {
-    using L = Layout<N, A, S, TX, TY, TZ, NB, EQ>;
+// T: kept for callers that walk a tile type by type; the offsets serve both types
+template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH>
+RTPN_HD Operands operand_offsets(const TileGeo& g, int /*T*/, int lx, int ly, int lz) {
+    using L = Layout<N, A, S, TX, TY, TZ, NB, NCH>;
     constexpr int B = 1 - A, ES = L::ES, REG = L::REG;
-    const int cp = (ly * TX + lx) * ES;             // the cell in a tile plane region (per component)
-    const int rbo = L::SRCO + T * L::SRC_T;         // own-type sources (z and x partners)
-    const int roo = L::SRCO + (1 - T) * L::SRC_T;   // other-type sources (y partners)
-    const int dy = T == 0 ? -1 : 1;                 // cos-type sources are read at y+1, sin-type at y-1
+    const int cp = (ly * TX + lx) * ES;  // the cell in a tile plane region (per component)
     Operands op;
-    op.c = rbo + lz * REG + cp;
-    op.o = roo + lz * REG + cp;
-    op.y = (ly + dy >= 0 && ly + dy < g.wy) ? op.o + dy * TX * ES : roo + L::KY * REG + (lz * TX + lx) * ES;
-    int xo[2], zo[2];
+    op.c = L::SRCO + lz * REG + cp;
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        const int src = L::SRCO + t * L::SRC_T;
+        const int dy = t == 0 ? 1 : -1;  // cos-type sources are read at y+1, sin-type at y-1
+        op.y[t] = (ly + dy >= 0 && ly + dy < g.wy) ? op.c + t * L::SRC_T + dy * TX * ES
+                                                   : src + L::KY * REG + (lz * TX + lx) * ES;
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            const int dx = dir_x(p, t);
+            op.x[p][t] = (lx + dx >= 0 && lx + dx < g.wx)
+                             ? op.c + t * L::SRC_T + dx * ES
+                             : src + L::KX * REG + ((lz * L::RY + ly) * L::XW + (dx > 0 ? g.hx_elem[1] : g.hx_elem[0])) * ES;
+        }
+    }
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
-        const int dx = dir_x(p, T);
-        xo[p] = (lx + dx >= 0 && lx + dx < g.wx)
-                    ? op.c + dx * ES
-                    : rbo + L::KX * REG + ((lz * L::RY + ly) * L::XW + (dx > 0 ? g.hx_elem[1] : g.hx_elem[0])) * ES;
         const int dz = ((B + p) & 1) == 0 ? 1 : -1;
-        zo[p] = (lz + dz >= 0 && lz + dz < g.wz) ? op.c + dz * REG : rbo + L::KZ * REG + cp;
+        op.z[p] = (lz + dz >= 0 && lz + dz < g.wz) ? op.c + dz * REG : L::SRCO + L::KZ * REG + cp;
     }
-    op.x0 = xo[0];
-    op.x1 = xo[1];
-    op.z0 = zo[0];
-    op.z1 = zo[1];
     return op;
 }
 
-// Scatter source column i of a stage buffer into the accumulators of target columns i - 1 (prev),
-// i (cur) and i + 1 (next) of type T: every source value yields its half-grid differences
-// (Section 2.1), each scattered into its <= 10 targets with the column's coupling constants
-// (Eqs. 4-5).  At |m| = 0 only the cos type exists: the absent type's constants are zero (its
-// regions hold earlier, finite data), so the same sweep serves every column.  Sources
-// q = fq .. N/2 (q < fq has l < i: not in the column) are entered at the chunk of kChunk slots
-// holding fq; slots below fq carry zero constants and read finite shared memory.
-template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int EQ>
+// What a column's sweep reads beside the sources themselves: the x and y partners (cos, sin) and the z
+// partner, as offsets in a stage buffer, and the factors of the y differences (h / h_y with the
+// column's sign, by target type).  At |m| = 0 the absent sin type's x and y differences are taken as
+// zero: its partners are its own (stale) values.  src_t: offset between the types' regions.
+struct ColumnOps {
+    int x0, x1, y0, y1, z;
+    float2 s;
+};
+RTPN_HD ColumnOps column_operands(const Operands& op, int i, int src_t, float sy) {
+    const bool odd = i & 1;
+    ColumnOps c;
+    c.x0 = odd ? op.x[1][0] : op.x[0][0];
+    c.x1 = odd ? op.x[1][1] : i == 0 ? op.c + src_t : op.x[0][1];
+    c.y0 = op.y[0];
+    c.y1 = i == 0 ? op.c + src_t : op.y[1];
+    c.z = odd ? op.z[1] : op.z[0];
+    c.s = odd ? make_float2(-sy, sy) : make_float2(sy, -sy);
+    return c;
+}
+
+// One source slot's operands, both types: value, x, y and z partners, and its constants.
+struct SlotOps {
+    float c0, c1, x0, x1, y0, y1, z0, z1;
+    float4 kz, ku, kd;  // pairs to l-1, l+1: of column M (z), M+1 and (negated) M-1 (x and y)
+};
+
+// Scatter the slots of sub-stage C of source column i (in a stage buffer) into the accumulators of target
+// columns i - 1 (prev), i (cur) and i + 1 (next): every source value yields its half-grid differences
+// (Section 2.1), each scattered into its <= 10 targets with the column's coupling constants (Eqs.
+// 4-5).  At |m| = 0 only the cos type exists: the absent type's constants are zero or meet zero
+// differences (its regions hold earlier, finite data), so the same sweep serves every column.  fq: the
+// column's first source slot.
+template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH, int C>
+RTPN_HD void sweep_pairs(const unsigned char* buf, int c0, const ColumnOps& op, int fq,
+                         float2 (&prev)[(N - A) / 2 + 1], float2 (&cur)[(N - A) / 2 + 1],
+                         float2 (&next)[(N - A) / 2 + 1]) {
+    using L = Layout<N, A, S, TX, TY, TZ, NB, NCH>;
+    constexpr int B = 1 - A, UB = L::UB, ST = L::SRC_T, K = L::K;
+    constexpr int NLA = (N - A) / 2 + 1, NLB = (N - B) / 2 + 1;
+    constexpr int KC = C * K + K <= NLB ? K : NLB - C * K;  // slots of this sub-stage
+    const int skip = fq > C * K ? fq - C * K : 0;  // slots below the column's first source fq
+    const unsigned char* bs = buf - skip * UB;     // slot k sits at k * UB from each base
+    const unsigned char* pc = bs + c0;
+    const unsigned char* pz = bs + op.z;
+    const unsigned char* py0 = bs + op.y0;
+    const unsigned char* py1 = bs + op.y1;
+    const unsigned char* px0 = bs + op.x0;
+    const unsigned char* px1 = bs + op.x1;
+    const float4* kc = reinterpret_cast<const float4*>(buf + L::COEFO);
+    auto load = [&](SlotOps& o, int k) {
+        const int e = k * UB;
+        o.c0 = lds<S>(pc, e);
+        o.c1 = lds<S>(pc, e + ST);
+        o.x0 = lds<S>(px0, e);
+        o.x1 = lds<S>(px1, e);
+        o.y0 = lds<S>(py0, e);
+        o.y1 = lds<S>(py1, e);
+        o.z0 = lds<S>(pz, e);
+        o.z1 = lds<S>(pz, e + ST);
+        RTPN_CHECK_PTR(kc + (KPAIRS / 2) * k + 2);
+        o.kz = kc[(KPAIRS / 2) * k];
+        o.ku = kc[(KPAIRS / 2) * k + 1];
+        o.kd = kc[(KPAIRS / 2) * k + 2];
+    };
+    auto work = [&](const SlotOps& o, auto ki) {
+        constexpr int q = C * K + decltype(ki)::value;
+        constexpr int ls = 2 * q + B;
+        constexpr int lm = (ls - 1) / 2, lp = (ls + 1) / 2;  // acc index of l-1, l+1
+        constexpr bool has_m = ls - 1 >= 0 && lm < NLA;
+        constexpr bool has_p = ls + 1 <= N && lp < NLA;
+        constexpr int am = has_m ? lm : 0, ap = has_p ? lp : 0;
+        const float2 c = make_float2(o.c0, o.c1), xn = make_float2(o.x0, o.x1);
+        const float2 dz = pair_sub(make_float2(o.z0, o.z1), c);
+        const float2 dx = pair_sub(xn, c), nx = pair_sub(c, xn);
+        const float2 dy = pair_mul(make_float2(o.y1 - o.c1, o.y0 - o.c0), op.s);  // the other type's
+        if constexpr (has_m) cur[am] = pair_fma(make_float2(o.kz.x, o.kz.y), dz, cur[am]);
+        if constexpr (has_p) cur[ap] = pair_fma(make_float2(o.kz.z, o.kz.w), dz, cur[ap]);
+        if constexpr (has_m) prev[am] = pair_fma(make_float2(o.kd.x, o.kd.y), nx, prev[am]);
+        if constexpr (has_p) prev[ap] = pair_fma(make_float2(o.kd.z, o.kd.w), nx, prev[ap]);
+        if constexpr (has_m) next[am] = pair_fma(make_float2(o.ku.x, o.ku.y), dx, next[am]);
+        if constexpr (has_p) next[ap] = pair_fma(make_float2(o.ku.z, o.ku.w), dx, next[ap]);
+        if constexpr (has_m) prev[am] = pair_fma(make_float2(o.kd.x, o.kd.y), dy, prev[am]);
+        if constexpr (has_p) prev[ap] = pair_fma(make_float2(o.kd.z, o.kd.w), dy, prev[ap]);
+        if constexpr (has_m) next[am] = pair_fma(make_float2(o.ku.x, o.ku.y), dy, next[am]);
+        if constexpr (has_p) next[ap] = pair_fma(make_float2(o.ku.z, o.ku.w), dy, next[ap]);
+    };
+    constexpr int NBLK = KC / kBlock > 0 ? KC / kBlock : 1;  // the last block takes the remainder
+    static_for<NBLK>([&](auto bi) {
+        constexpr int b0 = decltype(bi)::value * kBlock;
+        constexpr int nb = decltype(bi)::value == NBLK - 1 ? KC - b0 : kBlock;
+        if (b0 + nb > skip) {
+            SlotOps o[nb];
+            static_for<nb>([&](auto ki) { load(o[decltype(ki)::value], b0 + decltype(ki)::value); });
+            static_for<nb>([&](auto ki) {
+                work(o[decltype(ki)::value], std::integral_constant<int, b0 + decltype(ki)::value>{});
+            });
+        }
+    });
+}
+
+// The lane of type T of sweep_pairs over a whole column, for callers that walk a tile type by type.
+template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH>
 RTPN_HD void sweep_column(const unsigned char* buf, const Operands& op, int T, int i,
                           float (&prev)[(N - A) / 2 + 1], float (&cur)[(N - A) / 2 + 1],
                           float (&next)[(N - A) / 2 + 1]) {
-    using L = Layout<N, A, S, TX, TY, TZ, NB, EQ>;
-    constexpr int B = 1 - A, UB = L::UB;
-    constexpr int NLA = (N - A) / 2 + 1, NLB = (N - B) / 2 + 1;
-    const int fq = first_l(i, B) / 2;  // run slot of source q is q - fq
-    const int sh = -fq * UB;           // so source q sits at q * UB from each base
-    const unsigned char* pc = buf + op.c + sh;
-    const unsigned char* px = buf + ((i & 1) ? op.x1 : op.x0) + sh;
-    const unsigned char* pz = buf + ((i & 1) ? op.z1 : op.z0) + sh;
-    const unsigned char* po = buf + op.o + sh;
-    const unsigned char* py = buf + op.y + sh;
-    const float* cf = reinterpret_cast<const float*>(buf + L::COEFO);
-    const float4* kown = reinterpret_cast<const float4*>(cf + T * L::NLC * CPAD);
-    const float4* koth = reinterpret_cast<const float4*>(cf + (1 - T) * L::NLC * CPAD);
-    auto slot = [&](auto qi) {
-        constexpr int q = decltype(qi)::value;
-        if constexpr (q < NLB) {
-            constexpr int ls = 2 * q + B;
-            constexpr int lm = (ls - 1) / 2, lp = (ls + 1) / 2;  // acc index of l-1, l+1
-            constexpr bool has_m = ls - 1 >= 0 && lm < NLA;
-            constexpr bool has_p = ls + 1 <= N && lp < NLA;
-            if constexpr (has_m || has_p) {
-                constexpr int am = has_m ? lm : 0, ap = has_p ? lp : 0;
-                const float c = lds<S>(pc, q * UB);
-                const float ddx = lds<S>(px, q * UB) - c;
-                const float ddz = lds<S>(pz, q * UB) - c;
-                RTPN_CHECK_PTR(kown + 3 * q + 1);
-                const float4 k0 = kown[3 * q], k1 = kown[3 * q + 1];
-                const float co = lds<S>(po, q * UB);
-                const float ddy = lds<S>(py, q * UB) - co;
-                RTPN_CHECK_PTR(koth + 3 * q + 2);
-                const float4 k2 = koth[3 * q + 2];
-                if constexpr (has_m) cur[am] = fmaf(k0.x, ddz, cur[am]);
-                if constexpr (has_p) cur[ap] = fmaf(k0.y, ddz, cur[ap]);
-                if constexpr (has_m) prev[am] = fmaf(k0.z, ddx, prev[am]);
-                if constexpr (has_p) prev[ap] = fmaf(k0.w, ddx, prev[ap]);
-                if constexpr (has_m) next[am] = fmaf(k1.x, ddx, next[am]);
-                if constexpr (has_p) next[ap] = fmaf(k1.y, ddx, next[ap]);
-                if constexpr (has_m) prev[am] = fmaf(k2.x, ddy, prev[am]);
-                if constexpr (has_p) prev[ap] = fmaf(k2.y, ddy, prev[ap]);
-                if constexpr (has_m) next[am] = fmaf(k2.z, ddy, next[am]);
-                if constexpr (has_p) next[ap] = fmaf(k2.w, ddy, next[ap]);
-            }
-        }
-    };
-    auto chunk = [&](auto ci) {
-        constexpr int C = decltype(ci)::value;
-        static_for<kChunk>([&](auto ki) { slot(std::integral_constant<int, C * kChunk + decltype(ki)::value>{}); });
-    };
-    switch (fq / kChunk) { RTPN_CHUNK_CASES(chunk) }
+    using L = Layout<N, A, S, TX, TY, TZ, NB, NCH>;
+    static_assert(NCH == 1, "one stage per column");
+    constexpr int NLA = (N - A) / 2 + 1;
+    float2 p[NLA], c[NLA], n[NLA];
+    for (int q = 0; q < NLA; ++q) {
+        p[q] = make_float2(prev[q], prev[q]);
+        c[q] = make_float2(cur[q], cur[q]);
+        n[q] = make_float2(next[q], next[q]);
+    }
+    sweep_pairs<N, A, S, TX, TY, TZ, NB, NCH, 0>(buf, op.c, column_operands(op, i, L::SRC_T, 1.f),
+                                                first_source<N, A>(i), p, c, n);
+    for (int q = 0; q < NLA; ++q) {
+        prev[q] = T ? p[q].y : p[q].x;
+        cur[q] = T ? c[q].y : c[q].x;
+        next[q] = T ? n[q].y : n[q].x;
+    }
 }
 
-// Finish target column M of type T (accumulators in prev) from its old values in the stage's
-// target planes (at byte offset tgo for this cell) into global memory: FORWARD by Eq. (5),
-// u' = alpha u - beta acc (the u_0 factors al0, be0, ga0 for slot 0 of column 0, cos type, class 0);
-// ADJ_SOURCES lam' = alpha lam + acc / h (alpha = 1 when no factors are given).  tp: component q = 0 of the run at this cell, components V
-// apart; only an active cell is stored.
-template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int EQ, int MODE>
+// Finish the slots of target column M that sub-stage C completes, both types (accumulators in prev),
+// from their old values in the stage's target planes (at byte offset tgo for this cell; the sin type
+// TGT_T further) into global memory: FORWARD by Eq. (5), u' = alpha u + scale acc with scale = -beta / h
+// (the u_0 factors al0, be0, ga0 for slot 0 of column 0, cos type, class 0); ADJ_SOURCES lam' = alpha
+// lam + scale acc with scale = 1 / h (alpha = 1 when no factors are given).  q0: the column's first
+// slot; t0, t1: slot q = 0 of the cos and the sin run at this cell, slots vb bytes apart; cos_t,
+// sin_t: whether this cell's values of the type are stored.
+template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH, int MODE, int C>
+RTPN_HD void finish_pairs(const unsigned char* buf, int tgo, int M, int q0, char* t0, char* t1, unsigned vb, bool cos_t,
+                          bool sin_t, float2 alpha, float2 scale, float al0, float be0, float ga0,
+                          const float2 (&prev)[(N - A) / 2 + 1]) {
+    using L = Layout<N, A, S, TX, TY, TZ, NB, NCH>;
+    constexpr int UB = L::UB;
+    constexpr int LO = window_lo<N, A, NCH>(C), HI = window_hi<N, A, NCH>(C);
+    const int qs = q0 > LO ? q0 : LO;  // the slot the target boxes start with
+    const unsigned char* ob = buf + tgo - (qs - LO) * UB;
+    constexpr int kGroup = 3;
+    constexpr int NG = (HI - LO + kGroup - 1) / kGroup;
+    static_for<NG>([&](auto gi) {
+        constexpr int g0 = LO + decltype(gi)::value * kGroup;
+        constexpr int ng = g0 + kGroup <= HI ? kGroup : HI - g0;
+        if (g0 + ng > qs) {
+            float2 old[ng];
+            static_for<ng>([&](auto ki) {
+                constexpr int k = decltype(ki)::value, q = g0 + k;
+                old[k] = make_float2(0.f, 0.f);
+                if (k == ng - 1 || q >= qs)
+                    old[k] = make_float2(lds<S>(ob, (q - LO) * UB), lds<S>(ob, (q - LO) * UB + L::TGT_T));
+            });
+            static_for<ng>([&](auto ki) {
+                constexpr int k = decltype(ki)::value, q = g0 + k;
+                // the product with the accumulator is rounded first in a forward pass, the one with the old
+                // value in the adjoint's
+                float2 nv = MODE == ADJ_SOURCES ? pair_fma(scale, prev[q], pair_mul(alpha, old[k]))
+                                                : pair_fma(alpha, old[k], pair_mul(scale, prev[q]));
+                if constexpr (A == 0 && q == 0)  // u_0
+                    if (M == 0)
+                        nv.x = MODE == ADJ_SOURCES ? fmaf(scale.x, prev[q].x, al0 * old[k].x)
+                                                   : fmaf(al0, old[k].x, fmaf(-be0, prev[q].x, ga0));
+                const bool in = k == ng - 1 || q >= qs;
+                if (in && cos_t) win::store<S>(reinterpret_cast<S*>(t0 + (unsigned long long)q * vb), nv.x);
+                if (in && sin_t) win::store<S>(reinterpret_cast<S*>(t1 + (unsigned long long)q * vb), nv.y);
+            });
+        }
+    });
+}
+
+// The same for type T alone over a whole column (accumulators, factors and the run's first component
+// tp of that type), for callers that walk a tile type by type.
+template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH, int MODE>
 RTPN_HD void finish_column(const unsigned char* buf, int tgo, int M, int T, S* tp, long long V, bool active,
                            float alpha, float beta, float al0, float be0, float ga0, float inv_h,
                            const float (&prev)[(N - A) / 2 + 1]) {
-    using L = Layout<N, A, S, TX, TY, TZ, NB, EQ>;
-    constexpr int UB = L::UB, NLA = (N - A) / 2 + 1;
-    const bool u0 = A == 0 && M == 0 && T == 0;
-    const int q0 = first_l(M, A) / 2;  // targets q = q0 .. NLA - 1 (l >= M)
-    const unsigned char* ob = buf + tgo - q0 * UB;
-    auto tslot = [&](auto qi) {
-        constexpr int q = decltype(qi)::value;
-        if constexpr (q < NLA) {
-            const float old = lds<S>(ob, q * UB);
-            float nv;
-            if constexpr (MODE == ADJ_SOURCES)
-                nv = fmaf(inv_h, prev[q], ((q == 0 && u0) ? al0 : alpha) * old);
-            else if (q == 0)
-                nv = u0 ? fmaf(al0, old, fmaf(-be0, prev[q], ga0)) : fmaf(alpha, old, -beta * prev[q]);
-            else
-                nv = fmaf(alpha, old, -beta * prev[q]);
-            if (active) win::store<S>(tp + (long long)q * V, nv);
-        }
-    };
-    switch (q0) { RTPN_SLOT_CASES(tslot) }
+    using L = Layout<N, A, S, TX, TY, TZ, NB, NCH>;
+    static_assert(NCH == 1, "one stage per column");
+    constexpr int NLA = (N - A) / 2 + 1;
+    float2 p[NLA];
+    for (int q = 0; q < NLA; ++q) p[q] = make_float2(prev[q], prev[q]);
+    const float scale = MODE == ADJ_SOURCES ? inv_h : -beta;
+    finish_pairs<N, A, S, TX, TY, TZ, NB, NCH, MODE, 0>(
+        buf, tgo - T * L::TGT_T, M, first_l(M, A) / 2, reinterpret_cast<char*>(tp), reinterpret_cast<char*>(tp),
+        (unsigned)(V * (long long)sizeof(S)), active && T == 0, active && T == 1, make_float2(alpha, alpha),
+        make_float2(scale, scale), al0, be0, ga0, p);
 }
 
-template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int EQ, int MODE>
+template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH, int MODE>
 __device__ __forceinline__ void stage_kernel_body(const Args& a, unsigned char* smem) {
-    using L = Layout<N, A, S, TX, TY, TZ, NB, EQ>;
+    using L = Layout<N, A, S, TX, TY, TZ, NB, NCH>;
     static_assert(N >= 1, "order N >= 1");
-    static_assert((N + 2) / 2 <= kMaxSlots, "slot switch covers N <= 45");
+    static_assert(L::NMAP <= kMaxSlots, "tensor maps of a kind");
     constexpr int B = 1 - A;
     constexpr int NLA = (N - A) / 2 + 1;   // class-A components of a run, at most
-    constexpr int CELLS = L::CELLS;
-    constexpr int REG = L::REG, ES = L::ES;
+    constexpr int ES = L::ES;
     constexpr int NST = N + 2;  // stage i: sources of column i (i <= N), targets of column i - 1
     const int cA0 = A == 0 ? 0 : class_size(N, 0);
     [[maybe_unused]] const int* colA = a.colstart + A * (N + 2);
     const int tid = threadIdx.x;
-    const int warp = tid >> 5, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;  // warp: uniform for the compiler
     const long long V = a.V;
 
     // TMA writes into shared memory need 128-byte aligned destinations; the dynamic shared memory
@@ -678,7 +901,7 @@ __device__ __forceinline__ void stage_kernel_body(const Args& a, unsigned char* 
     const unsigned full0 = smem_addr(&bars[0]), empty0 = smem_addr(&bars[NB]);
     if (tid == 0) {
         for (int b = 0; b < NB; ++b) {
-            mbar_init(full0 + 8 * b, 1);  // the producer's arrive.expect_tx
+            mbar_init(full0 + 8 * b, kProducers);  // each producer's arrive.expect_tx
             mbar_init(empty0 + 8 * b, L::CONSUMER_WARPS);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -686,116 +909,101 @@ __device__ __forceinline__ void stage_kernel_body(const Args& a, unsigned char* 
     __syncthreads();
 
     const int my_tiles = a.tiles > blockIdx.x ? (int)((a.tiles - 1 - blockIdx.x) / gridDim.x) + 1 : 0;
-    const int total = my_tiles * NST;
-    if (warp == L::CONSUMER_WARPS) {
-        stage_producer<N, A, S, TX, TY, TZ, NB, EQ>(a, bufs, full0, empty0, total);
+    const int total = my_tiles * tile_stages<N, A, NCH>();
+    if (warp >= L::CONSUMER_WARPS) {
+        stage_producer<N, A, S, TX, TY, TZ, NB, NCH>(a, bufs, full0, empty0, total, warp - L::CONSUMER_WARPS);
         return;
     }
 
-    // ---- consumers: thread (T, cell) finishes the targets of type T in its cell.  Both types run
-    // the same code: the type only selects regions, coupling-constant rows and the y direction.
-    const int T = tid / CELLS, ctid = tid % CELLS;
-    const int lx = ctid % TX, ly = (ctid / TX) % TY, lz = ctid / (TX * TY);
-    const int tgo = L::TGTO + T * L::TGT_T + lz * REG + (ly * TX + lx) * ES;  // this cell's old target values
+    // ---- consumers: a thread finishes the targets of both types in its cell
+    const int lx = tid % TX, ly = (tid / TX) % TY, lz = tid / (TX * TY);
+    const int tgo = L::TGTO + lz * L::REGT + (ly * TX + lx) * ES;  // this cell's old target values (type 0)
 
     // the three live target columns; their roles (prev, cur, next) rotate by one per stage
-    float wa[NLA], wb[NLA], wc[NLA];
+    float2 wa[NLA], wb[NLA], wc[NLA];
 
-    TileGeo g{};
-    bool active = false;
-    long long cell = 0;
-    Operands op{};                                     // operand offsets, fixed per tile
-    float alE = 0.f, beE = 0.f, alO = 0.f, beO = 0.f;  // Eq. (5) factors of columns M even / odd
-    float al0 = 0.f, be0 = 0.f, ga0 = 0.f;             // u_0 (class 0, type 0 only)
-
-    // first local index of target column M in class A, advanced column by column (offA = colstart
-    // of the column finished next)
-    int offA = 0;
+    const unsigned vb = (unsigned)(V * ES);  // bytes of a component
+    unsigned limit = a.wait_limit;           // 0 once a wait has run out: the rest of the pass is not waited for
     unsigned tile = blockIdx.x;
-    int b = 0;
-    unsigned ph = 0;
-    int s = 0, i = 0;
-
-    // One stage: sweep source column i into prev (column i - 1), cur (i) and next (i + 1), finish
-    // prev, and clear it (it is the next stage's `next`).  False if a wait ran out.
-    auto stage = [&](float (&prev)[NLA], float (&cur)[NLA], float (&next)[NLA]) -> bool {
-        if (i == 0) {  // new tile: geometry, operand offsets, factors, a cleared window
-            if (s > 0) tile += gridDim.x;
-            g = tile_geo<TX, TY, TZ, L::G>(a, tile);
-            active = lx < g.wx && ly < g.wy && lz < g.wz;
-            cell = ((long long)(g.z0 + lz) * a.ny + (g.y0 + ly)) * a.nx + (g.x0 + lx);
-            op = operand_offsets<N, A, S, TX, TY, TZ, NB, EQ>(g, T, lx, ly, lz);
+    unsigned b = 0, ph = 0;                  // stage buffer, phase parity of its current use
+    for (int k = 0; k < my_tiles; ++k, tile += gridDim.x) {
+        const TileGeo g = tile_geo<TX, TY, TZ, L::G>(a, tile);
+        const bool active = lx < g.wx && ly < g.wy && lz < g.wz;
+        const long long cell = ((long long)(g.z0 + lz) * a.ny + (g.y0 + ly)) * a.nx + (g.x0 + lx);
+        const Operands op = operand_offsets<N, A, S, TX, TY, TZ, NB, NCH>(g, 0, lx, ly, lz);  // fixed per tile
+        float2 al[2] = {}, be[2] = {};         // Eq. (5) factors by parity of M
+        float al0 = 0.f, be0 = 0.f, ga0 = 0.f; // u_0 (class 0, type 0 only)
+        if (active && (MODE == FORWARD || a.fac)) {  // ADJ_SOURCES: the alphas only, if asked
+            // sub-grid slot of (l, M, T) in class A: x by (M, T), y by T, z by (A + M)
 #pragma unroll
-            for (int q = 0; q < NLA; ++q) prev[q] = cur[q] = next[q] = 0.f;
-            if (active && (MODE == FORWARD || a.fac)) {  // ADJ_SOURCES: the alphas only, if asked
-                // sub-grid slot of (l, M, T) in class A: x by (M, T), y by T, z by (A + M)
-#pragma unroll
-                for (int par = 0; par < 2; ++par) {
-                    const int gx = ((par == 0) == (T == 0)) ? 0 : 1;
-                    const int gz = ((A + par) & 1) == 0 ? 0 : 1;
-                    const int gc = gx + 2 * T + 4 * gz;
-                    const float al = __ldg(a.fac + (long long)(a.fac_ofs + 2 * gc) * V + cell);
-                    // the pass folds 1/h into beta
-                    const float be = __ldg(a.fac + (long long)(a.fac_ofs + 2 * gc + 1) * V + cell) * a.inv_h;
-                    if (par == 0) {
-                        alE = al;
-                        beE = be;
-                    } else {
-                        alO = al;
-                        beO = be;
-                    }
-                }
-                if (A == 0 && T == 0) {
-                    al0 = __ldg(a.fac + (long long)FAC_U0 * V + cell);
-                    be0 = __ldg(a.fac + (long long)(FAC_U0 + 1) * V + cell) * a.inv_h;
-                    ga0 = __ldg(a.fac + (long long)(FAC_U0 + 2) * V + cell);
-                }
-            } else if (MODE == ADJ_SOURCES) {
-                alE = alO = al0 = 1.f;
+            for (int par = 0; par < 2; ++par) {
+                const int gz = ((A + par) & 1) == 0 ? 0 : 1;
+                const int gc = (par == 0 ? 0 : 1) + 4 * gz, gs = (par == 0 ? 1 : 0) + 2 + 4 * gz;
+                const float* f = a.fac + (long long)a.fac_ofs * V + cell;
+                al[par] = make_float2(__ldg(f + 2 * gc * V), __ldg(f + 2 * gs * V));
+                if (MODE == FORWARD) be[par] = make_float2(__ldg(f + (2 * gc + 1) * V), __ldg(f + (2 * gs + 1) * V));
             }
+            if (A == 0) {
+                al0 = __ldg(a.fac + (long long)FAC_U0 * V + cell);
+                be0 = __ldg(a.fac + (long long)(FAC_U0 + 1) * V + cell);
+                ga0 = __ldg(a.fac + (long long)(FAC_U0 + 2) * V + cell);
+            }
+        } else if (MODE == ADJ_SOURCES) {
+            al[0] = al[1] = make_float2(1.f, 1.f);
+            al0 = 1.f;
         }
-        // target column i - 1 of type T is finished in this stage (the same for the whole warp); the
-        // sweep and the finish run on every thread of the tile (a thread past the grid's edge works
-        // on zero-filled or in-tile shared memory), only global memory accesses need an active cell
-        const bool finw = i >= 1 && (T == 0 || i - 1 >= 1);
-
-        if (!__all_sync(0xffffffffu, wait_phase(full0 + 8 * b, ph, a.wait_limit))) {
-            if (lane == 0) atomicOr(a.status, STATUS_TIMEOUT);
-            return false;
-        }
-        const unsigned char* buf = bufs + b * L::BUF;
-
-        if (column_len(N, i, B) > 0) sweep_column<N, A, S, TX, TY, TZ, NB, EQ>(buf, op, T, i, prev, cur, next);
-        if (finw) {
-            const int M = i - 1;
-            const float alpha = (M & 1) ? alO : alE, beta = (M & 1) ? beO : beE;
-            const int q0 = first_l(M, A) / 2;
-            (void)RTPN_SCHECK(offA == colA[M]);
-            S* tp = reinterpret_cast<S*>(a.tgt) + (long long)(cA0 + offA + T * column_len(N, M, A) - q0) * V + cell;
-            finish_column<N, A, S, TX, TY, TZ, NB, EQ, MODE>(buf, tgo, M, T, tp, V, active, alpha, beta, al0, be0,
-                                                             ga0, a.inv_h, prev);
-        }
-        // the stage buffer is free once every lane of the warp is past its reads
-        __syncwarp();
-        if (lane == 0) mbar_arrive(empty0 + 8 * b);
-        if (++b == NB) {
-            b = 0;
-            ph ^= 1u;
-        }
-        // prev is done: it is the next stage's `next`
 #pragma unroll
-        for (int q = 0; q < NLA; ++q) prev[q] = 0.f;
-        if (i >= 1) offA += ntypes(i - 1) * column_len(N, i - 1, A);
-        if (i == NST - 1) offA = 0;  // tile done
-        ++s;
-        i = (i == NST - 1) ? 0 : i + 1;
-        return true;
-    };
-    // the column loop unrolled by three: the window's roles rotate instead of its registers moving
-    while (s < total) {
-        if (!stage(wa, wb, wc) || s >= total) break;
-        if (!stage(wb, wc, wa) || s >= total) break;
-        if (!stage(wc, wa, wb)) break;
+        for (int q = 0; q < NLA; ++q) wa[q] = wb[q] = wc[q] = make_float2(0.f, 0.f);
+        char* const tcell = reinterpret_cast<char*>(a.tgt) + cell * ES;
+        unsigned comp = cA0;  // the first component of target column M in the target array
+
+        // One column: its sub-stages sweep source column i into prev (column i - 1), cur (i) and next
+        // (i + 1) and finish prev slot by slot; then prev is cleared (it is the next column's `next`).
+        auto column = [&](int i, float2 (&prev)[NLA], float2 (&cur)[NLA], float2 (&next)[NLA]) {
+            const int C0 = first_chunk<N, A, NCH>(i), fq = first_source<N, A>(i);
+            const bool sources = i <= N && 2 * fq + B <= N;
+            const ColumnOps cop = column_operands(op, i, L::SRC_T, a.sy);
+            // target column M = i - 1
+            const int M = i - 1, q0 = M >= 0 ? first_source<N, B>(M) : 0, lenA = NLA - q0;
+            (void)RTPN_SCHECK(M < 0 || comp == (unsigned)(cA0 + colA[M]));
+            char* const t0 = tcell + (unsigned long long)(comp - (unsigned)q0) * vb;
+            char* const t1 = t0 + (unsigned long long)(unsigned)lenA * vb;
+            const bool odd = M & 1, sin_t = active && M >= 1;
+            const float2 alpha = odd ? al[1] : al[0];
+            const float2 scale = MODE == ADJ_SOURCES ? make_float2(a.inv_h, a.inv_h)
+                                                     : pair_mul(odd ? be[1] : be[0], make_float2(-a.inv_h, -a.inv_h));
+            static_for<NCH>([&](auto ci) {
+                constexpr int C = decltype(ci)::value;
+                if (C < C0) return;
+                if (!wait_phase(full0 + 8 * b, ph, limit)) {
+                    if (lane == 0) atomicOr(a.status, STATUS_TIMEOUT);
+                    limit = 0;
+                }
+                const unsigned char* buf = bufs + b * (unsigned)L::BUF;
+                // the sweep and the finish run on every thread of the tile (a thread past the grid's edge
+                // works on zero-filled or in-tile shared memory), only global accesses need an active cell
+                if (sources) sweep_pairs<N, A, S, TX, TY, TZ, NB, NCH, C>(buf, op.c, cop, fq, prev, cur, next);
+                if (M >= 0)
+                    finish_pairs<N, A, S, TX, TY, TZ, NB, NCH, MODE, C>(buf, tgo, M, q0, t0, t1, vb, active, sin_t, alpha,
+                                                                        scale, al0, be0 * a.inv_h, ga0, prev);
+                // the stage buffer is free once every lane of the warp is past its reads
+                __syncwarp();
+                if (lane == 0) mbar_arrive(empty0 + 8 * b);
+                if (++b == NB) {
+                    b = 0;
+                    ph ^= 1u;
+                }
+            });
+#pragma unroll
+            for (int q = 0; q < NLA; ++q) prev[q] = make_float2(0.f, 0.f);
+            if (M >= 0) comp += (unsigned)((M >= 1 ? 2 : 1) * lenA);
+        };
+        // unrolled by three: the window's roles rotate instead of its registers moving
+        for (int i = 0; i < NST; i += 3) {
+            column(i, wa, wb, wc);
+            if (NST % 3 == 0 || i + 1 < NST) column(i + 1, wb, wc, wa);
+            if (NST % 3 == 0 || i + 2 < NST) column(i + 2, wc, wa, wb);
+        }
     }
 }
 
