@@ -322,6 +322,8 @@ void release(rtpn_ctx* ctx) {
     if (ctx->scat) cudaFree(ctx->scat);
     ctx->scat = nullptr;
     if (ctx->table_mem) cudaFree(ctx->table_mem);
+    if (ctx->perm) cudaFree(ctx->perm);
+    ctx->perm = nullptr;
     if (ctx->partial) cudaFree(ctx->partial);
     if (ctx->counter) cudaFree(ctx->counter);
     if (ctx->staging) cudaFree(ctx->staging);
@@ -526,6 +528,10 @@ int rtpn_create(rtpn_ctx** out, int N, int nx, int ny, int nz, double h, int bc,
     if (e != cudaSuccess) return bail(fail(ctx, RTPN_ENOMEM, "factor allocation failed"));
     e = cudaMalloc(&ctx->staging, (size_t)V * 8);
     if (e != cudaSuccess) return bail(fail(ctx, RTPN_ENOMEM, "staging allocation failed"));
+    e = cudaMalloc(&ctx->perm, ctx->md.nc * sizeof(int));
+    if (e != cudaSuccess) return bail(fail(ctx, RTPN_ENOMEM, "scratch allocation failed"));
+    e = cudaMemcpy(ctx->perm, ctx->md.internal_of_abi.data(), ctx->md.nc * sizeof(int), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return bail(fail(ctx, RTPN_ECUDA, cudaGetErrorString(e)));
     e = cudaMalloc(&ctx->partial, (SUM_BLOCKS + 1) * sizeof(double));
     if (e != cudaSuccess) return bail(fail(ctx, RTPN_ENOMEM, "scratch allocation failed"));
     e = cudaMalloc(&ctx->counter, sizeof(unsigned long long));
@@ -771,6 +777,18 @@ int rtpn_get_component(rtpn_ctx* ctx, int c, void* field, int dtype, int where) 
 int rtpn_set_moments(rtpn_ctx* ctx, const void* u, int dtype, int where) {
     if (!ctx || !u) return RTPN_EINVAL;
     if (!valid_dtype(dtype) || !valid_where(where)) return fail(ctx, RTPN_EINVAL, "bad dtype/where");
+    if (where == RTPN_DEVICE) {
+        with_storage(ctx->prec, [&](auto tag) {
+            using S = std::remove_pointer_t<decltype(tag)>;
+            if (dtype == RTPN_DTYPE_F64)
+                launch_reorder<double, S>((const double*)u, (S*)ctx->u, ctx->perm, ctx->md.nc, ctx->g.V, true, ctx->stream);
+            else
+                launch_reorder<float, S>((const float*)u, (S*)ctx->u, ctx->perm, ctx->md.nc, ctx->g.V, true, ctx->stream);
+        });
+        CHECK_LAUNCH(ctx);
+        ctx->steps_done = 0;
+        return RTPN_OK;
+    }
     const size_t plane = (size_t)ctx->g.V * dtype_size(dtype);
     for (int c = 0; c < ctx->md.nc; ++c) {
         int rc = put_component(ctx, c, (const char*)u + (size_t)c * plane, dtype, where);
@@ -784,6 +802,17 @@ int rtpn_set_moments(rtpn_ctx* ctx, const void* u, int dtype, int where) {
 int rtpn_get_moments(rtpn_ctx* ctx, void* u, int dtype, int where) {
     if (!ctx || !u) return RTPN_EINVAL;
     if (!valid_dtype(dtype) || !valid_where(where)) return fail(ctx, RTPN_EINVAL, "bad dtype/where");
+    if (where == RTPN_DEVICE) {
+        with_storage(ctx->prec, [&](auto tag) {
+            using S = std::remove_pointer_t<decltype(tag)>;
+            if (dtype == RTPN_DTYPE_F64)
+                launch_reorder<S, double>((const S*)ctx->u, (double*)u, ctx->perm, ctx->md.nc, ctx->g.V, false, ctx->stream);
+            else
+                launch_reorder<S, float>((const S*)ctx->u, (float*)u, ctx->perm, ctx->md.nc, ctx->g.V, false, ctx->stream);
+        });
+        CHECK_LAUNCH(ctx);
+        return RTPN_OK;
+    }
     const size_t plane = (size_t)ctx->g.V * dtype_size(dtype);
     for (int c = 0; c < ctx->md.nc; ++c) {
         int rc = take_component(ctx, c, (char*)u + (size_t)c * plane, dtype, where);

@@ -70,6 +70,10 @@ void launch_media_factors(const double* sa, const double* ss, const double* q, F
                           const Geom& g, double dt, const double* scat, int N, cudaStream_t st);
 template <typename Sin, typename Sout>
 void launch_convert(const Sin* in, Sout* out, long long n, cudaStream_t st);
+// all components between interface order and internal order: out[perm[c]] = in[c] (in_order), else
+// out[c] = in[perm[c]], with conversion; perm (device): internal index by interface index
+template <typename Sin, typename Sout>
+void launch_reorder(const Sin* in, Sout* out, const int* perm, int nc, long long V, bool in_order, cudaStream_t st);
 template <typename S>
 void launch_sum(const S* x, long long n, double* partial, int nblocks, double* out, cudaStream_t st);
 template <typename S>
@@ -158,6 +162,7 @@ struct rtpn_ctx {
     void* table_mem = nullptr;       // device partner tables (both classes)
     rtpn::PartnerTable<double> tab64[2]{};
     rtpn::PartnerTable<float> tab32[2]{};
+    int* perm = nullptr;             // internal component by interface index (device)
     double* partial = nullptr;       // reduction partials [SUM_BLOCKS] + result
     unsigned long long* counter = nullptr;
     void* staging = nullptr;         // one plane of FP64 (conversions, media upload)
