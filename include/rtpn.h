@@ -68,8 +68,9 @@ extern "C" {
 #define RTPN_KERNEL_AUTO    0  /* fastest available for (N, precision)                            */
 #define RTPN_KERNEL_GENERIC 1  /* any N and precision: one thread per cell, partner-table gather   */
 #define RTPN_KERNEL_WINDOW  2  /* FP32/BF16, compiled N: register-window scatter over m-columns  */
-#define RTPN_KERNEL_STAGE   3  /* FP32/BF16, compiled N, nx*elem a multiple of 16 B: column loop
-                                  with TMA-staged shared-memory tiles, persistent CTAs          */
+#define RTPN_KERNEL_STAGE   3  /* FP32/BF16, compiled N, nx*elem a multiple of 16 B (AUTO: any nx, see
+                                  rtpn_set_kernel): column loop with TMA-staged shared-memory
+                                  tiles, persistent CTAs                                        */
 #define RTPN_KERNEL_FUSED   4  /* FP32/BF16, compiled N (1, 3, 5, 7, 9): each (even full step, odd
                                   step) pair of rtpn_step in one z-streaming pass between two
                                   state buffers; single substeps use the window kernel          */
@@ -83,7 +84,7 @@ typedef struct rtpn_info {
     int nx, ny, nz;
     int bc, precision, kernel;
     double h, dt;
-    size_t state_bytes;    /* device bytes of the moment state               */
+    size_t state_bytes;    /* device bytes of the moment state (padding included) */
     size_t factor_bytes;   /* device bytes of the per-cell substep factors   */
     long long steps_done;  /* full steps taken since the last set_moments    */
     int tile[3];           /* CTA tile of the active kernel (0 = not tiled)  */
@@ -159,8 +160,10 @@ int rtpn_set_stream(rtpn_ctx* ctx, void* stream);
  * tile_x and tile_y must be 0 (or 32 and 8); tile_z is the number of z planes a CTA streams through
  * (0 = one wave of resident CTAs).  Selecting it allocates a second state buffer (RTPN_ENOMEM if
  * that fails); RTPN_EUNSUPPORTED for a batch instance.
- * RTPN_KERNEL_AUTO picks STAGE (for N >= 15), then WINDOW, then GENERIC; with non-cubic cells STAGE
- * (any compiled N), else GENERIC; with anisotropic scattering GENERIC.
+ * RTPN_KERNEL_AUTO picks STAGE (for N >= 15; where nx gives no 16-byte rows the state's rows are padded
+ * inside the library, except in a batch), then WINDOW, then GENERIC; with non-cubic cells STAGE (any
+ * compiled N), else GENERIC; with anisotropic scattering GENERIC.  Moving between padded and dense rows
+ * rearranges the state in place.
  * RTPN_EUNSUPPORTED if the kernel is not compiled for (N, precision, nx) or does not take the
  * context's cells or scattering; the previous selection then stays. */
 int rtpn_set_kernel(rtpn_ctx* ctx, int kernel, int tile_x, int tile_y, int tile_z);

@@ -231,6 +231,26 @@ __global__ void k_copy_cast(const A* __restrict__ in, B* __restrict__ out, long 
         out[i] = (B)in[i];
 }
 
+// the same with padded rows of u_0 (nx values, px apart)
+template <typename S>
+__global__ void k_dot_rows(const S* __restrict__ u0, int nx, int px, const double* __restrict__ w, long long n,
+                           double* __restrict__ partial) {
+    double acc = 0.0;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const long long row = i / nx;
+        acc += (double)ldv<S, float>(u0 + row * px + (i - row * nx)) * w[i];
+    }
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    __shared__ double ws[32];
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double s = 0.0;
+        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += ws[i];
+        partial[blockIdx.x] = s;
+    }
+}
+
 unsigned blocks_for(long long V, int threads = 256) { return (unsigned)((V + threads - 1) / threads); }
 
 // out = sum of partial[0 .. count) in a fixed order (one block)
@@ -578,6 +598,16 @@ extern "C" int rtpn_adjoint(rtpn_ctx* ctx, const void* w, int dtype, int where, 
     if (ctx->scat) return afail(ctx, RTPN_EUNSUPPORTED, "adjoint: anisotropic scattering");
     if (!ctx->media_set || !ctx->media) return afail(ctx, RTPN_ESTATE, "adjoint: media not set");
     const long long V = ctx->g.V;
+    // the adjoint's kernels read dense rows; the selected kernel and its padded rows come back at the end
+    struct DenseRows {
+        rtpn_ctx* c;
+        bool padded;
+        ~DenseRows() {
+            if (padded) use_dense_rows(c, false);
+        }
+    } dense{ctx, ctx->padded()};
+    if (dense.padded)
+        if (int rc = use_dense_rows(ctx, true)) return rc;
     // the weights and outputs as FP64 device arrays
     Buf wd, out;
     if (!wd.alloc((size_t)V * sizeof(double)) || !out.alloc((size_t)3 * V * sizeof(double)))
@@ -646,6 +676,10 @@ extern "C" int rtpn_detector(rtpn_ctx* ctx, const void* w, int dtype, int where,
     }
     if (ctx->prec == RTPN_FP64)
         k_dot_u0<double><<<SUM_BLOCKS, 256, 0, st>>>((const double*)ctx->u, wd, V, ctx->partial);
+    else if (ctx->padded() && ctx->prec == RTPN_FP32)
+        k_dot_rows<float><<<SUM_BLOCKS, 256, 0, st>>>((const float*)ctx->u, ctx->g.nx, ctx->px, wd, V, ctx->partial);
+    else if (ctx->padded())
+        k_dot_rows<__nv_bfloat16><<<SUM_BLOCKS, 256, 0, st>>>((const __nv_bfloat16*)ctx->u, ctx->g.nx, ctx->px, wd, V, ctx->partial);
     else if (ctx->prec == RTPN_FP32)
         k_dot_u0<float><<<SUM_BLOCKS, 256, 0, st>>>((const float*)ctx->u, wd, V, ctx->partial);
     else

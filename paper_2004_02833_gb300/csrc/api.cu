@@ -86,13 +86,53 @@ bool same_type(int prec, int dtype) {
 }
 
 void* comp_ptr(rtpn_ctx* ctx, int internal) {
-    return (char*)ctx->u + (size_t)internal * ctx->g.V * ctx->elem;
+    return (char*)ctx->u + (size_t)internal * ctx->sV * ctx->elem;
+}
+
+// rows between a dense array of the caller's type and the (padded) state; one component without a
+// permutation, or all of them
+RowCopy rows_of(const rtpn_ctx* ctx, bool into_state, bool all) {
+    const Geom& g = ctx->g;
+    RowCopy r{g.nx, into_state ? g.nx : ctx->px, into_state ? ctx->px : g.nx, all ? ctx->md.nc : 1,
+              (long long)g.ny * g.nz, into_state ? g.V : ctx->sV, into_state ? ctx->sV : g.V,
+              all ? ctx->perm : nullptr, into_state};
+    return r;
+}
+void rows_in(rtpn_ctx* ctx, const void* in, int dtype, void* state, bool all) {
+    const RowCopy r = rows_of(ctx, true, all);
+    with_storage(ctx->prec, [&](auto tag) {
+        using S = std::remove_pointer_t<decltype(tag)>;
+        if (dtype == RTPN_DTYPE_F64)
+            launch_rows<double, S>((const double*)in, (S*)state, r, ctx->stream);
+        else
+            launch_rows<float, S>((const float*)in, (S*)state, r, ctx->stream);
+    });
+}
+void rows_out(rtpn_ctx* ctx, const void* state, void* out, int dtype, bool all) {
+    const RowCopy r = rows_of(ctx, false, all);
+    with_storage(ctx->prec, [&](auto tag) {
+        using S = std::remove_pointer_t<decltype(tag)>;
+        if (dtype == RTPN_DTYPE_F64)
+            launch_rows<S, double>((const S*)state, (double*)out, r, ctx->stream);
+        else
+            launch_rows<S, float>((const S*)state, (float*)out, r, ctx->stream);
+    });
 }
 
 int put_component(rtpn_ctx* ctx, int abi, const void* src, int dtype, int where) {
     const long long V = ctx->g.V;
     void* dst = comp_ptr(ctx, ctx->md.internal_of_abi[abi]);
     const size_t bytes = (size_t)V * dtype_size(dtype);
+    if (ctx->padded()) {
+        const void* dev = src;
+        if (where == RTPN_HOST) {
+            CUDA_TRY(ctx, cudaMemcpyAsync(ctx->staging, src, bytes, cudaMemcpyHostToDevice, ctx->stream));
+            dev = ctx->staging;
+        }
+        rows_in(ctx, dev, dtype, dst, false);
+        CHECK_LAUNCH(ctx);
+        return RTPN_OK;
+    }
     if (same_type(ctx->prec, dtype)) {
         CUDA_TRY(ctx, cudaMemcpyAsync(dst, src, bytes,
                                       where == RTPN_HOST ? cudaMemcpyHostToDevice
@@ -112,6 +152,13 @@ int take_component(rtpn_ctx* ctx, int abi, void* dst, int dtype, int where) {
     const long long V = ctx->g.V;
     const void* src = comp_ptr(ctx, ctx->md.internal_of_abi[abi]);
     const size_t bytes = (size_t)V * dtype_size(dtype);
+    if (ctx->padded()) {
+        rows_out(ctx, src, where == RTPN_HOST ? ctx->staging : dst, dtype, false);
+        CHECK_LAUNCH(ctx);
+        if (where == RTPN_HOST)
+            CUDA_TRY(ctx, cudaMemcpyAsync(dst, ctx->staging, bytes, cudaMemcpyDeviceToHost, ctx->stream));
+        return RTPN_OK;
+    }
     if (same_type(ctx->prec, dtype)) {
         CUDA_TRY(ctx, cudaMemcpyAsync(dst, src, bytes,
                                       where == RTPN_HOST ? cudaMemcpyDeviceToHost
@@ -346,13 +393,48 @@ void release(rtpn_ctx* ctx) {
     ctx->own = nullptr;
 }
 
-// Automatic selection: the staged kernel where it is compiled for (N, precision), N >= kStageMinN
-// and nx gives 16-byte rows, else the register-window kernel, else the generic one.  Below
-// kStageMinN the unrolled window body is small enough for the instruction cache and the staged
-// kernel's per-column-stage overhead dominates its few components per column (P7 128^3 FP32 on a
-// GB300: 0.41 ms per step with the window kernel, 0.92 with the staged one; P15: 2.16 and 2.02).
+// Automatic selection: the staged kernel where it is compiled for (N, precision) and N >= kStageMinN, on
+// padded rows where nx does not give 16-byte ones, else the register-window kernel, else the generic
+// one.  Padding costs at most three (FP32) or seven (BF16) columns of traffic; the kernels that take any
+// width cost far more there (GB300, FP32, a pass: P15 61 x 77 x 75 0.14 ms against
+// 0.24 on the window kernel, P19 0.18 against 1.09 on the generic one, P39 0.68 against 3.25 on the window
+// kernel).  Below kStageMinN the unrolled window body is
+// small enough for the instruction cache and the staged kernel's barriers and copies per stage weigh more
+// (P7 128^3: 0.40 ms a step with the window kernel, 0.38 with the staged one).
 constexpr bool kStageInAuto = true;
 constexpr int kStageMinN = 15;
+
+// Row pitch of the state: nx, or nx padded to 16-byte rows.  The state is rearranged in place, a component
+// at a time through the staging plane (its buffer holds the padded state if the context can ever need
+// it); the padding holds zeros.
+int set_rows(rtpn_ctx* ctx, bool padded) {
+    const Geom& g = ctx->g;
+    const int grp = stage_row_group(ctx->prec), px = padded ? (g.nx + grp - 1) / grp * grp : g.nx;
+    if (px == ctx->px) return RTPN_OK;
+    const long long sV = (long long)px * g.ny * g.nz, rows = (long long)g.ny * g.nz;
+    drop_graphs(ctx);
+    for (int k = 0; k < ctx->md.nc; ++k) {
+        const int c = px > ctx->px ? ctx->md.nc - 1 - k : k;  // growing: from the last component
+        with_storage(ctx->prec, [&](auto tag) {
+            using S = std::remove_pointer_t<decltype(tag)>;
+            if constexpr (!std::is_same_v<S, double>) {  // FP64 states are never padded
+                const S* from = (const S*)ctx->u + (size_t)c * ctx->sV;
+                S* to = (S*)ctx->u + (size_t)c * sV;
+                launch_rows<S, S>(from, (S*)ctx->staging, RowCopy{g.nx, ctx->px, g.nx, 1, rows, 0, 0, nullptr, true}, ctx->stream);
+                launch_rows<S, S>((const S*)ctx->staging, to, RowCopy{g.nx, g.nx, px, 1, rows, 0, 0, nullptr, true}, ctx->stream);
+            }
+        });
+    }
+    CHECK_LAUNCH(ctx);
+    ctx->px = px;
+    ctx->sV = sV;
+    return RTPN_OK;
+}
+
+// whether the automatic choice may pad the rows for the staged kernel
+bool may_pad(const rtpn_ctx* ctx) {
+    return kStageInAuto && ctx->N >= kStageMinN && !ctx->batch_member && stage_compiled(ctx->N, ctx->prec);
+}
 
 int choose_kernel(rtpn_ctx* ctx) {
     int k = ctx->kernel;
@@ -370,9 +452,12 @@ int choose_kernel(rtpn_ctx* ctx) {
     // kernel takes cubic cells only
     const bool win_ok = window_supported(ctx->N, ctx->prec) && (cubic || window_extended(ctx->N));
     if (k == RTPN_KERNEL_AUTO) {
-        const bool tile_set = ctx->tx || ctx->ty || ctx->tz;
+        const bool tile_set = (ctx->tx || ctx->ty || ctx->tz) && !ctx->tile_from_stage;
+        // other widths than 16-byte rows: padded, unless the caller asks for a tile (then one of the
+        // kernels that take any width)
+        const bool pad = may_pad(ctx) && !ctx->dense_rows && !tile_set;
         if (kStageInAuto && (ctx->N >= kStageMinN || !win_ok) &&
-            stage_supported(ctx->N, ctx->prec, ctx->g.nx) &&
+            (stage_supported(ctx->N, ctx->prec, ctx->g.nx) || pad) &&
             (!tile_set || stage_has_tile(ctx->N, ctx->tx, ctx->ty, ctx->tz, ctx->depth, ctx->prec)))
             k = RTPN_KERNEL_STAGE;
         else
@@ -389,12 +474,19 @@ int choose_kernel(rtpn_ctx* ctx) {
         return fail(ctx, RTPN_EUNSUPPORTED, "the fused kernel takes cubic cells only");
     if (!cubic && k == RTPN_KERNEL_WINDOW && !window_extended(ctx->N))
         return fail(ctx, RTPN_EUNSUPPORTED, "the window kernel takes non-cubic cells up to N = 15 only");
-    if (k == RTPN_KERNEL_STAGE) {
+    // the automatic choice runs the staged kernel on any width of rows, padding them; chosen by name it
+    // takes 16-byte rows only
+    const bool pad = k == RTPN_KERNEL_STAGE && ctx->kernel == RTPN_KERNEL_AUTO &&
+                     !stage_supported(ctx->N, ctx->prec, ctx->g.nx);
+    if (k == RTPN_KERNEL_STAGE && !pad) {
         if (!stage_supported(ctx->N, ctx->prec, ctx->g.nx))
             return fail(ctx, RTPN_EUNSUPPORTED,
                         "staged kernel not compiled for this N/precision or nx*elem not 16-byte rows");
         if (!stage_has_tile(ctx->N, ctx->tx, ctx->ty, ctx->tz, ctx->depth, ctx->prec))
             return fail(ctx, RTPN_EUNSUPPORTED, "no staged kernel compiled for this tile / stage depth");
+    }
+    if (int rc = set_rows(ctx, pad)) return rc;
+    if (k == RTPN_KERNEL_STAGE) {
         int rc = stage_prepare(ctx, ctx->tx, ctx->ty, ctx->tz, ctx->depth);
         if (rc) return fail(ctx, RTPN_ECUDA, std::string("staged kernel set-up: ") +
                                                  cudaGetErrorString((cudaError_t)rc));
@@ -489,6 +581,19 @@ int rtpn_coupling_dense(int N, int axis, double* out) {
 
 int rtpn_create(rtpn_ctx** out, int N, int nx, int ny, int nz, double h, int bc, int precision,
                 double dt) {
+    return rtpn::create_context(out, N, nx, ny, nz, h, bc, precision, dt, false);
+}
+
+}  // extern "C"
+
+int rtpn::use_dense_rows(rtpn_ctx* ctx, bool on) {
+    if (ctx->dense_rows == on) return RTPN_OK;
+    ctx->dense_rows = on;
+    return choose_kernel(ctx);
+}
+
+int rtpn::create_context(rtpn_ctx** out, int N, int nx, int ny, int nz, double h, int bc, int precision, double dt,
+                         bool batch_member) {
     if (!out) return fail(nullptr, RTPN_EINVAL, "out is NULL");
     *out = nullptr;
     if (N < 0 || N > 63) return fail(nullptr, RTPN_EINVAL, "N must be in 0..63");
@@ -509,6 +614,9 @@ int rtpn_create(rtpn_ctx** out, int N, int nx, int ny, int nz, double h, int bc,
     ctx->g = Geom{nx, ny, nz, V, bc, h, h, h};
     ctx->prec = precision;
     ctx->dt = dt;
+    ctx->batch_member = batch_member;
+    ctx->px = nx;
+    ctx->sV = V;
     ctx->elem = precision == RTPN_FP64 ? 8 : (precision == RTPN_FP32 ? 4 : 2);
     const size_t fac_elem = precision == RTPN_FP64 ? 8 : 4;
     auto bail = [&](int rc) {
@@ -521,7 +629,10 @@ int rtpn_create(rtpn_ctx** out, int N, int nx, int ny, int nz, double h, int bc,
     if (cudaStreamCreateWithFlags(&ctx->own, cudaStreamDefault) != cudaSuccess)
         return bail(fail(ctx, RTPN_ECUDA, "stream create failed"));
     ctx->stream = ctx->own;
-    cudaError_t e = cudaMalloc(&ctx->u, (size_t)ctx->md.nc * V * ctx->elem);
+    // room for padded rows where the automatic choice may take them
+    const int grp = may_pad(ctx) ? stage_row_group(precision) : 1;
+    const size_t state_room = (size_t)ctx->md.nc * ((nx + grp - 1) / grp * grp) * ny * nz * ctx->elem;
+    cudaError_t e = cudaMalloc(&ctx->u, state_room);
     if (e != cudaSuccess) return bail(fail(ctx, RTPN_ENOMEM, "state allocation failed"));
     ctx->u_home = ctx->u;
     e = cudaMalloc(&ctx->fac, (size_t)FAC_PLANES * V * fac_elem);
@@ -541,7 +652,7 @@ int rtpn_create(rtpn_ctx** out, int N, int nx, int ny, int nz, double h, int bc,
     e = cudaMemsetAsync(ctx->status, 0, 8 * sizeof(unsigned), ctx->stream);
     if (e != cudaSuccess) return bail(fail(ctx, RTPN_ECUDA, cudaGetErrorString(e)));
     if ((rc = upload_tables(ctx))) return bail(rc);
-    e = cudaMemsetAsync(ctx->u, 0, (size_t)ctx->md.nc * V * ctx->elem, ctx->stream);
+    e = cudaMemsetAsync(ctx->u, 0, state_room, ctx->stream);
     if (e != cudaSuccess) return bail(fail(ctx, RTPN_ECUDA, cudaGetErrorString(e)));
     if ((rc = choose_kernel(ctx))) return bail(rc);
     e = cudaStreamSynchronize(ctx->stream);
@@ -549,6 +660,8 @@ int rtpn_create(rtpn_ctx** out, int N, int nx, int ny, int nz, double h, int bc,
     *out = ctx;
     return RTPN_OK;
 }
+
+extern "C" {
 
 int rtpn_destroy(rtpn_ctx* ctx) {
     if (!ctx) return RTPN_OK;
@@ -777,6 +890,12 @@ int rtpn_get_component(rtpn_ctx* ctx, int c, void* field, int dtype, int where) 
 int rtpn_set_moments(rtpn_ctx* ctx, const void* u, int dtype, int where) {
     if (!ctx || !u) return RTPN_EINVAL;
     if (!valid_dtype(dtype) || !valid_where(where)) return fail(ctx, RTPN_EINVAL, "bad dtype/where");
+    if (where == RTPN_DEVICE && ctx->padded()) {
+        rows_in(ctx, u, dtype, ctx->u, true);
+        CHECK_LAUNCH(ctx);
+        ctx->steps_done = 0;
+        return RTPN_OK;
+    }
     if (where == RTPN_DEVICE) {
         with_storage(ctx->prec, [&](auto tag) {
             using S = std::remove_pointer_t<decltype(tag)>;
@@ -802,6 +921,11 @@ int rtpn_set_moments(rtpn_ctx* ctx, const void* u, int dtype, int where) {
 int rtpn_get_moments(rtpn_ctx* ctx, void* u, int dtype, int where) {
     if (!ctx || !u) return RTPN_EINVAL;
     if (!valid_dtype(dtype) || !valid_where(where)) return fail(ctx, RTPN_EINVAL, "bad dtype/where");
+    if (where == RTPN_DEVICE && ctx->padded()) {
+        rows_out(ctx, ctx->u, u, dtype, true);
+        CHECK_LAUNCH(ctx);
+        return RTPN_OK;
+    }
     if (where == RTPN_DEVICE) {
         with_storage(ctx->prec, [&](auto tag) {
             using S = std::remove_pointer_t<decltype(tag)>;
@@ -824,7 +948,7 @@ int rtpn_get_moments(rtpn_ctx* ctx, void* u, int dtype, int where) {
 
 int rtpn_zero_moments(rtpn_ctx* ctx) {
     if (!ctx) return RTPN_EINVAL;
-    CUDA_TRY(ctx, cudaMemsetAsync(ctx->u, 0, (size_t)ctx->md.nc * ctx->g.V * ctx->elem, ctx->stream));
+    CUDA_TRY(ctx, cudaMemsetAsync(ctx->u, 0, (size_t)ctx->md.nc * ctx->sV * ctx->elem, ctx->stream));
     ctx->steps_done = 0;
     return RTPN_OK;
 }
@@ -872,9 +996,9 @@ int rtpn_copy_planes(rtpn_ctx* dst, int dst_z, rtpn_ctx* src, int src_z, int nz,
     // the components of a class are contiguous in the internal order (class 0 first)
     const int c0 = cls == 1 ? dst->md.ne : 0;
     const int n = cls == -1 ? dst->md.nc : (cls == 0 ? dst->md.ne : dst->md.no);
-    const size_t plane = (size_t)dst->g.nx * dst->g.ny * dst->elem;
-    const char* sp = (const char*)src->u + ((size_t)c0 * src->g.V + (size_t)src_z * dst->g.nx * dst->g.ny) * dst->elem;
-    char* dp = (char*)dst->u + ((size_t)c0 * dst->g.V + (size_t)dst_z * dst->g.nx * dst->g.ny) * dst->elem;
+    auto at = [&](const rtpn_ctx* c, int comp, int z) {
+        return (char*)c->u + ((size_t)comp * c->sV + (size_t)z * c->px * c->g.ny) * c->elem;
+    };
     // the copy runs on dst's stream after src's queued work, and src's later work runs after it
     cudaEvent_t ev = nullptr;
     if (src->stream != dst->stream) {
@@ -882,8 +1006,14 @@ int rtpn_copy_planes(rtpn_ctx* dst, int dst_z, rtpn_ctx* src, int src_z, int nz,
         CUDA_TRY(dst, cudaEventRecord(ev, src->stream));
         CUDA_TRY(dst, cudaStreamWaitEvent(dst->stream, ev, 0));
     }
-    cudaError_t e = cudaMemcpy2DAsync(dp, (size_t)dst->g.V * dst->elem, sp, (size_t)src->g.V * dst->elem,
-                                      (size_t)nz * plane, (size_t)n, cudaMemcpyDeviceToDevice, dst->stream);
+    cudaError_t e = cudaSuccess;
+    if (src->px == dst->px)
+        e = cudaMemcpy2DAsync(at(dst, c0, dst_z), (size_t)dst->sV * dst->elem, at(src, c0, src_z), (size_t)src->sV * src->elem,
+                              (size_t)nz * dst->px * dst->g.ny * dst->elem, (size_t)n, cudaMemcpyDeviceToDevice, dst->stream);
+    else  // one of the states has padded rows
+        for (int c = c0; c < c0 + n && e == cudaSuccess; ++c)
+            e = cudaMemcpy2DAsync(at(dst, c, dst_z), (size_t)dst->px * dst->elem, at(src, c, src_z), (size_t)src->px * src->elem,
+                                  (size_t)dst->g.nx * dst->elem, (size_t)nz * dst->g.ny, cudaMemcpyDeviceToDevice, dst->stream);
     if (ev) {
         if (e == cudaSuccess) e = cudaEventRecord(ev, dst->stream);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(src->stream, ev, 0);
@@ -898,7 +1028,7 @@ int rtpn_sum_u0(rtpn_ctx* ctx, double* out) {
     const void* u0 = comp_ptr(ctx, ctx->md.internal_of_abi[0]);
     with_storage(ctx->prec, [&](auto tag) {
         using S = std::remove_pointer_t<decltype(tag)>;
-        launch_sum<S>((const S*)u0, ctx->g.V, ctx->partial, SUM_BLOCKS, ctx->partial + SUM_BLOCKS,
+        launch_sum<S>((const S*)u0, ctx->sV, ctx->partial, SUM_BLOCKS, ctx->partial + SUM_BLOCKS,
                       ctx->stream);
     });
     CHECK_LAUNCH(ctx);
@@ -912,7 +1042,7 @@ int rtpn_count_nonfinite(rtpn_ctx* ctx, long long* out) {
     if (!ctx || !out) return RTPN_EINVAL;
     with_storage(ctx->prec, [&](auto tag) {
         using S = std::remove_pointer_t<decltype(tag)>;
-        launch_count_nonfinite<S>((const S*)ctx->u, (long long)ctx->md.nc * ctx->g.V, ctx->counter,
+        launch_count_nonfinite<S>((const S*)ctx->u, (long long)ctx->md.nc * ctx->sV, ctx->counter,
                                   ctx->stream);
     });
     CHECK_LAUNCH(ctx);
@@ -967,7 +1097,7 @@ int rtpn_get_info(const rtpn_ctx* ctx, rtpn_info* out) {
     out->hy = ctx->g.hy;
     out->hz = ctx->g.hz;
     out->dt = ctx->dt;
-    out->state_bytes = (size_t)ctx->md.nc * ctx->g.V * ctx->elem;
+    out->state_bytes = (size_t)ctx->md.nc * ctx->sV * ctx->elem;
     out->factor_bytes = (size_t)ctx->fac_planes * ctx->g.V * (ctx->prec == RTPN_FP64 ? 8 : 4);
     out->steps_done = ctx->steps_done;
     out->tile[0] = ctx->tx;

@@ -131,12 +131,14 @@ int rtpn_autotune(rtpn_ctx* ctx, int reps, int tile[3], double* ms_per_step) {
     if (kernel == RTPN_KERNEL_STAGE) {
         int v[4 * 64];
         const int n = rtpn::stage_variants_of(ctx->N, ctx->prec, v, 64);
-        for (int i = 0; i < n; ++i) cands.push_back({v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]});
+        // padded rows belong to the automatic choice: its tile is timed, none is set by name
+        for (int i = 0; i < n && !ctx->padded(); ++i) cands.push_back({v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]});
+        if (ctx->padded()) cands.push_back(best);
     } else {
         for (const Tile& t : kCandidates) cands.push_back(t);
     }
     if (best_ms < 0) {
-        const size_t bytes = (size_t)ctx->md.nc * ctx->g.V * ctx->elem;
+        const size_t bytes = (size_t)ctx->md.nc * ctx->sV * ctx->elem;
         void* snap = nullptr;
         if (cudaMalloc(&snap, bytes) != cudaSuccess) {
             cudaGetLastError();
@@ -147,7 +149,7 @@ int rtpn_autotune(rtpn_ctx* ctx, int reps, int tile[3], double* ms_per_step) {
         const int otx = ctx->tx, oty = ctx->ty, otz = ctx->tz, oc = ctx->depth;
         int rc = sweep(
             ctx->stream, reps, cands,
-            [&](Tile t) { return rtpn_set_kernel_ex(ctx, kernel, t.x, t.y, t.z, t.c); },
+            [&](Tile t) { return ctx->padded() ? RTPN_OK : rtpn_set_kernel_ex(ctx, kernel, t.x, t.y, t.z, t.c); },
             [&](cudaStream_t) {
                 int r = rtpn_substep(ctx, 0, 0);
                 return r ? r : rtpn_substep(ctx, 1, 0);
@@ -157,14 +159,14 @@ int rtpn_autotune(rtpn_ctx* ctx, int reps, int tile[3], double* ms_per_step) {
         cudaStreamSynchronize(ctx->stream);
         cudaFree(snap);
         if (rc) {
-            rtpn_set_kernel_ex(ctx, kernel, otx, oty, otz, oc);
+            if (!ctx->padded()) rtpn_set_kernel_ex(ctx, kernel, otx, oty, otz, oc);
             return rc;
         }
         std::lock_guard<std::mutex> lock(g_mu);
         g_cache[key] = {best, best_ms};
         store_file(key, best, best_ms);
     }
-    int rc = rtpn_set_kernel_ex(ctx, kernel, best.x, best.y, best.z, best.c);
+    int rc = ctx->padded() ? RTPN_OK : rtpn_set_kernel_ex(ctx, kernel, best.x, best.y, best.z, best.c);
     if (rc) return rc;
     if (tile) {
         tile[0] = best.x;

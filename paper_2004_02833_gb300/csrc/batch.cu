@@ -333,13 +333,12 @@ int rtpn_batch_create(rtpn_batch** out, int count, const int* N, const int* nx, 
     b->prec = precision;
     for (int i = 0; i < count; ++i) {
         rtpn_ctx* c = nullptr;
-        int rc = rtpn_create(&c, N[i], nx[i], ny[i], nz[i], h[i], bc[i], precision, dt ? dt[i] : 0.0);
+        int rc = create_context(&c, N[i], nx[i], ny[i], nz[i], h[i], bc[i], precision, dt ? dt[i] : 0.0, true);
         if (rc) {
             release(b);
             delete b;
             return rc;
         }
-        c->batch_member = true;
         b->ctx.push_back(c);
         rc = bat::upload_constants(c->md);
         if (rc) {

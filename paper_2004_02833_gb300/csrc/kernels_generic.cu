@@ -206,6 +206,10 @@ __device__ __forceinline__ double conv<__nv_bfloat16, double>(__nv_bfloat16 v) {
     return (double)__bfloat162float(v);
 }
 template <>
+__device__ __forceinline__ __nv_bfloat16 conv<__nv_bfloat16, __nv_bfloat16>(__nv_bfloat16 v) {
+    return v;
+}
+template <>
 __device__ __forceinline__ float conv<__nv_bfloat16, float>(__nv_bfloat16 v) {
     return __bfloat162float(v);
 }
@@ -298,6 +302,32 @@ RTPN_REORDER(float, __nv_bfloat16)
 RTPN_REORDER(__nv_bfloat16, double)
 RTPN_REORDER(__nv_bfloat16, float)
 #undef RTPN_REORDER
+
+// The same for arrays with padded rows: a warp per row.
+template <typename A, typename B>
+__global__ void __launch_bounds__(256) k_rows(const A* __restrict__ in, B* __restrict__ out, RowCopy r) {
+    const long long row = (long long)blockIdx.x * 8 + threadIdx.y;
+    if (row >= r.rows) return;
+    const int c = blockIdx.y, p = r.perm ? r.perm[c] : c;
+    const A* src = in + (r.in_order ? c : p) * r.is + row * r.ip;
+    B* dst = out + (r.in_order ? p : c) * r.os + row * r.op;
+    for (int x = threadIdx.x; x < r.op; x += 32) dst[x] = x < r.nx ? conv<A, B>(src[x]) : conv<float, B>(0.f);
+}
+template <typename A, typename B>
+void launch_rows(const A* in, B* out, const RowCopy& r, cudaStream_t stream) {
+    k_rows<A, B><<<dim3((unsigned)((r.rows + 7) / 8), (unsigned)r.nc), dim3(32, 8), 0, stream>>>(in, out, r);
+}
+#define RTPN_ROWS(A, B) template void launch_rows<A, B>(const A*, B*, const RowCopy&, cudaStream_t);
+RTPN_ROWS(float, float)
+RTPN_ROWS(float, double)
+RTPN_ROWS(float, __nv_bfloat16)
+RTPN_ROWS(double, float)
+RTPN_ROWS(double, __nv_bfloat16)
+RTPN_ROWS(double, double)
+RTPN_ROWS(__nv_bfloat16, __nv_bfloat16)
+RTPN_ROWS(__nv_bfloat16, float)
+RTPN_ROWS(__nv_bfloat16, double)
+#undef RTPN_ROWS
 
 // ------------------------------------------------------------------ FP64 reductions
 template <typename S>

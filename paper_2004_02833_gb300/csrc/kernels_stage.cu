@@ -56,13 +56,14 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     return fn;
 }
 
-static bool make_map(CUtensorMap* m, void* base, int precision, const rtpn::Geom& g, int nc, int bx, int by,
-                     int bz, int bc) {
+// px, sV: row pitch and component stride of the array
+static bool make_map(CUtensorMap* m, void* base, int precision, const rtpn::Geom& g, int px, long long sV, int nc,
+                     int bx, int by, int bz, int bc) {
     auto fn = encode_fn();
     if (!fn) return false;
     const cuuint64_t es = precision == RTPN_BF16 ? 2 : 4;
     const cuuint64_t dims[4] = {(cuuint64_t)g.nx, (cuuint64_t)g.ny, (cuuint64_t)g.nz, (cuuint64_t)nc};
-    const cuuint64_t strides[3] = {g.nx * es, (cuuint64_t)g.nx * g.ny * es, (cuuint64_t)g.V * es};
+    const cuuint64_t strides[3] = {px * es, (cuuint64_t)px * g.ny * es, (cuuint64_t)sV * es};
     const cuuint32_t box[4] = {(cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)bz, (cuuint32_t)bc};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     CUresult r = fn(m, precision == RTPN_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
@@ -74,16 +75,16 @@ static bool make_map(CUtensorMap* m, void* base, int precision, const rtpn::Geom
 // The tensor maps of one array for a variant (kinds MAP_PLANE, MAP_YROW, MAP_XGRP, each for box
 // lengths E = 1, 2, ..., nmap; see stage_impl.cuh) into out[0 .. kinds * nmap); kinds = 1 builds the
 // plane maps only (target arrays).
-static bool make_maps(CUtensorMap* out, void* base, int precision, const rtpn::Geom& g, int nc, const Variant& v,
-                      int kinds) {
+static bool make_maps(CUtensorMap* out, void* base, int precision, const rtpn::Geom& g, int px, long long sV, int nc,
+                      const Variant& v, int kinds) {
     int geo[4];
     v.geom(precision, geo);
     const int nmap = geo[0], xw = geo[2], ry = geo[3];
     for (int j = 0; j < nmap; ++j) {
         const int e = j + 1;
-        if (!make_map(&out[MAP_PLANE * nmap + j], base, precision, g, nc, v.tx, v.ty, 1, e)) return false;
-        if (kinds > 1 && (!make_map(&out[MAP_YROW * nmap + j], base, precision, g, nc, v.tx, 1, v.tz, e) ||
-                          !make_map(&out[MAP_XGRP * nmap + j], base, precision, g, nc, xw, ry, v.tz, e)))
+        if (!make_map(&out[MAP_PLANE * nmap + j], base, precision, g, px, sV, nc, v.tx, v.ty, 1, e)) return false;
+        if (kinds > 1 && (!make_map(&out[MAP_YROW * nmap + j], base, precision, g, px, sV, nc, v.tx, 1, v.tz, e) ||
+                          !make_map(&out[MAP_XGRP * nmap + j], base, precision, g, px, sV, nc, xw, ry, v.tz, e)))
             return false;
     }
     return true;
@@ -97,7 +98,7 @@ static bool make_maps(CUtensorMap* out, void* base, int precision, const rtpn::G
 // 256-cell and 0.195 with 512-cell tiles, P39 120^3 69 us a round with 192 cells and 82 with 320.  Rows
 // that do not start on 128-byte lines touch one more line each: P39 82 us a round of 32x3x3 tiles at 96^3
 // (aligned), 113 at 120^3 (GB300, FP32).
-static const Variant* best_variant(int N, int precision, int depth, const rtpn::Geom& g, int sms) {
+static const Variant* best_variant(int N, int precision, int depth, const rtpn::Geom& g, int px, int sms) {
     const Variant* best = nullptr;
     double best_cost = 0;
     const int es = precision == RTPN_BF16 ? 2 : 4;
@@ -112,7 +113,7 @@ static const Variant* best_variant(int N, int precision, int depth, const rtpn::
         // a grid of less than a round leaves SMs with fewer CTAs than they hold
         const long long per_sm = rounds > 1 ? geo[1] : (tiles + sms - 1) / sms;
         const int row = v.tx * es;
-        const double lines = row % 128 == 0 && g.nx * es % 128 == 0 ? 1.0 : 1.0 + 48.0 / row;
+        const double lines = row % 128 == 0 && px * es % 128 == 0 ? 1.0 : 1.0 + 48.0 / row;
         const double cost = rounds * (per_sm * v.tx * v.ty * v.tz * lines + fixed);
         if (!best || cost < best_cost) {
             best = &v;
@@ -133,10 +134,12 @@ static int nmaps_of(const Variant& v, int precision) {
 // device tensor-map slots of a context: forward (all kinds), adjoint w (all kinds), adjoint lam (plane)
 static constexpr int stage_maps_capacity = (2 * stg::MAP_KINDS + 1) * stg::kMaxSlots;
 
+bool stage_compiled(int N, int precision) {
+    return precision != RTPN_FP64 && stg::find(N, 0, 0, 0, 0, precision) != nullptr;
+}
+
 bool stage_supported(int N, int precision, int nx) {
-    if (precision == RTPN_FP64 || !stg::find(N, 0, 0, 0, 0, precision)) return false;
-    const int hx = precision == RTPN_BF16 ? 8 : 4;  // 16-byte rows for the tensor maps
-    return nx % hx == 0;
+    return stage_compiled(N, precision) && nx % stage_row_group(precision) == 0;
 }
 
 bool stage_has_tile(int N, int tx, int ty, int tz, int depth, int precision) {
@@ -150,14 +153,14 @@ int stage_prepare(rtpn_ctx* ctx, int tx, int ty, int tz, int depth) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, dev);
     if (tx == 0)
-        if (const stg::Variant* w = stg::best_variant(ctx->N, ctx->prec, depth, ctx->g, ctx->sms)) v = w;
+        if (const stg::Variant* w = stg::best_variant(ctx->N, ctx->prec, depth, ctx->g, ctx->px, ctx->sms)) v = w;
     const int N = ctx->N;
     // the tensor maps live in device global memory (64-byte aligned) and the kernel reads them from
     // there: tile planes / z halo plane, y halo row and x halo group, each for every box length
     const int nmap = stg::nmaps_of(*v, ctx->prec);
     if (nmap <= 0 || nmap > stg::kMaxSlots) return (int)cudaErrorInvalidValue;
     std::vector<CUtensorMap> maps((size_t)stg::MAP_KINDS * nmap);
-    if (!stg::make_maps(maps.data(), ctx->u, ctx->prec, ctx->g, ctx->md.nc, *v, stg::MAP_KINDS))
+    if (!stg::make_maps(maps.data(), ctx->u, ctx->prec, ctx->g, ctx->px, ctx->sV, ctx->md.nc, *v, stg::MAP_KINDS))
         return (int)cudaErrorInvalidValue;
     if (!ctx->stage_maps_dev) {
         // the forward's maps, then room for the adjoint's (all kinds over w, plane maps over lam)
@@ -228,12 +231,14 @@ static bool base_args(const rtpn_ctx* ctx, const stg::Variant& v, int coef_cls, 
     a.ntz = (a.nz + v.tz - 1) / v.tz;
     a.tiles = (long long)a.ntx * a.nty * a.ntz;
     // 32-bit stage counts and 32-bit byte strides of a component
-    if (a.tiles * (ctx->N + 2) * 4 >= (1ll << 31) || ctx->g.V * (long long)ctx->elem >= (1ll << 32)) return false;
+    if (a.tiles * (ctx->N + 2) * 4 >= (1ll << 31) || ctx->sV * (long long)ctx->elem >= (1ll << 32)) return false;
     // z chunk of the tile walk: the ~one tile per SM at work at a time then spans about as many
     // tile rows in y as layers in z, across the whole x extent
     const double side = std::sqrt((double)(ctx->sms > 0 ? ctx->sms : 1) / a.ntx);
     const int kz = (int)(side + 0.5);
     a.kz = kz < 1 ? 1 : (kz > a.ntz ? a.ntz : kz);
+    a.px = a.nx;
+    a.sV = a.V;
     a.nc = ctx->md.nc;
     a.status = ctx->status;
     a.wait_limit = (unsigned)STAGE_WAIT_LIMIT;
@@ -243,15 +248,18 @@ static bool base_args(const rtpn_ctx* ctx, const stg::Variant& v, int coef_cls, 
 }
 
 // a forward pass on class cls: sources through src_maps, old targets through the plane maps
-// tgt_maps, new targets stored into out (all three may be the context's state)
+// tgt_maps, new targets stored into out, whose rows are px and components sV apart (all three may be the
+// context's state)
 static int launch_pass(rtpn_ctx* ctx, int cls, int fac_ofs, const CUtensorMap* src_maps,
-                       const CUtensorMap* tgt_maps, void* out, cudaStream_t st, long long skip_stage,
-                       long long wait_limit) {
+                       const CUtensorMap* tgt_maps, void* out, int px, long long sV, cudaStream_t st,
+                       long long skip_stage, long long wait_limit) {
     if (ctx->stage_variant < 0) return (int)cudaErrorNotSupported;
     const stg::Variant& v = stg::kVariants[ctx->stage_variant];
     stg::Args a;
     if (!base_args(ctx, v, cls, &a)) return (int)cudaErrorInvalidValue;
     a.tgt = out;
+    a.px = px;
+    a.sV = sV;
     a.fac = (const float*)ctx->fac;
     a.fac_ofs = fac_ofs;
     a.maps = src_maps;
@@ -265,14 +273,14 @@ static int launch_pass(rtpn_ctx* ctx, int cls, int fac_ofs, const CUtensorMap* s
 int launch_stage(rtpn_ctx* ctx, int cls, int fac_ofs, cudaStream_t st, long long skip_stage,
                  long long wait_limit) {
     const CUtensorMap* maps = (const CUtensorMap*)ctx->stage_maps_dev;  // sources and targets: the state
-    return launch_pass(ctx, cls, fac_ofs, maps, maps, ctx->u, st, skip_stage, wait_limit);
+    return launch_pass(ctx, cls, fac_ofs, maps, maps, ctx->u, ctx->px, ctx->sV, st, skip_stage, wait_limit);
 }
 
 int launch_stage_between(rtpn_ctx* ctx, int cls, int fac_ofs, const void* src_maps, const void* tgt_maps,
                          void* out, cudaStream_t st) {
     if (ctx->prec != RTPN_FP32) return (int)cudaErrorNotSupported;
-    return launch_pass(ctx, cls, fac_ofs, (const CUtensorMap*)src_maps, (const CUtensorMap*)tgt_maps, out, st,
-                       -1, STAGE_WAIT_LIMIT);
+    return launch_pass(ctx, cls, fac_ofs, (const CUtensorMap*)src_maps, (const CUtensorMap*)tgt_maps, out,
+                       ctx->g.nx, ctx->g.V, st, -1, STAGE_WAIT_LIMIT);
 }
 
 size_t stage_maps_bytes(const rtpn_ctx* ctx) {
@@ -282,10 +290,10 @@ size_t stage_maps_bytes(const rtpn_ctx* ctx) {
 }
 
 int stage_maps_for(rtpn_ctx* ctx, const void* state, void* maps_dev) {
-    if (ctx->stage_variant < 0 || ctx->prec != RTPN_FP32) return (int)cudaErrorNotSupported;
+    if (ctx->stage_variant < 0 || ctx->prec != RTPN_FP32 || ctx->padded()) return (int)cudaErrorNotSupported;
     const stg::Variant& v = stg::kVariants[ctx->stage_variant];
     std::vector<CUtensorMap> maps((size_t)stg::MAP_KINDS * stg::nmaps_of(v, RTPN_FP32));
-    if (!stg::make_maps(maps.data(), const_cast<void*>(state), RTPN_FP32, ctx->g, ctx->md.nc, v, stg::MAP_KINDS))
+    if (!stg::make_maps(maps.data(), const_cast<void*>(state), RTPN_FP32, ctx->g, ctx->g.nx, ctx->g.V, ctx->md.nc, v, stg::MAP_KINDS))
         return (int)cudaErrorInvalidValue;
     return (int)cudaMemcpy(maps_dev, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice);
 }
@@ -300,8 +308,8 @@ int launch_stage_adjoint_sources(rtpn_ctx* ctx, int tgt_cls, float* lam, const f
     CUtensorMap* dev = (CUtensorMap*)ctx->stage_maps_dev + stg::MAP_KINDS * nmap;
     if (ctx->stage_adj_lam != lam || ctx->stage_adj_w != w) {
         std::vector<CUtensorMap> maps((size_t)(stg::MAP_KINDS + 1) * nmap);
-        if (!stg::make_maps(maps.data(), const_cast<float*>(w), RTPN_FP32, ctx->g, w_planes, v, stg::MAP_KINDS) ||
-            !stg::make_maps(maps.data() + stg::MAP_KINDS * nmap, lam, RTPN_FP32, ctx->g, ctx->md.nc, v, 1))
+        if (!stg::make_maps(maps.data(), const_cast<float*>(w), RTPN_FP32, ctx->g, ctx->g.nx, ctx->g.V, w_planes, v, stg::MAP_KINDS) ||
+            !stg::make_maps(maps.data() + stg::MAP_KINDS * nmap, lam, RTPN_FP32, ctx->g, ctx->g.nx, ctx->g.V, ctx->md.nc, v, 1))
             return (int)cudaErrorInvalidValue;
         cudaError_t err = cudaMemcpy(dev, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice);
         if (err != cudaSuccess) return (int)err;

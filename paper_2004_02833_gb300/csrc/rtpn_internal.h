@@ -74,6 +74,17 @@ void launch_convert(const Sin* in, Sout* out, long long n, cudaStream_t st);
 // out[c] = in[perm[c]], with conversion; perm (device): internal index by interface index
 template <typename Sin, typename Sout>
 void launch_reorder(const Sin* in, Sout* out, const int* perm, int nc, long long V, bool in_order, cudaStream_t st);
+// Rows of nx values between two arrays of nc components with their own row pitches (ip, op) and component
+// strides (is, os), with conversion; perm / in_order as in launch_reorder (perm may be null), the
+// padding of the output's rows set to zero.
+struct RowCopy {
+    int nx, ip, op, nc;
+    long long rows, is, os;
+    const int* perm;
+    bool in_order;
+};
+template <typename Sin, typename Sout>
+void launch_rows(const Sin* in, Sout* out, const RowCopy& r, cudaStream_t st);
 template <typename S>
 void launch_sum(const S* x, long long n, double* partial, int nblocks, double* out, cudaStream_t st);
 template <typename S>
@@ -113,11 +124,19 @@ bool fused_supported(int N, int precision);
 int fused_prepare(const Model& md, int precision);
 int launch_fused(int N, int precision, const FusedLaunch& f, cudaStream_t st);
 
+// rtpn_create; batch_member contexts keep dense rows (the grouped kernels read their states)
+int create_context(rtpn_ctx** out, int N, int nx, int ny, int nz, double h, int bc, int precision, double dt,
+                   bool batch_member);
+// Dense rows and a kernel that takes them (on), or the kernel and row pitch of the selection again (off).
+int use_dense_rows(rtpn_ctx* ctx, bool on);
+
 // transposed partner table (adjoint.cu): targets of class clsB, sources of the other class
 HostTable transposed_table(const Model& md, int clsB, const Geom& g);
 
 // ---- TMA-staged kernels (kernels_stage.cu, stage.cu) ----
-// nx must give 16-byte rows for the tensor maps
+// compiled for (N, precision); rows must be 16-byte groups for the tensor maps (stage_row_group values)
+bool stage_compiled(int N, int precision);
+inline int stage_row_group(int precision) { return precision == RTPN_BF16 ? 8 : 4; }
 bool stage_supported(int N, int precision, int nx);
 bool stage_has_tile(int N, int tx, int ty, int tz, int depth, int precision);
 // builds the tensor maps (tile 0,0,0 = default; depth 0 = any) and the coupling tables;
@@ -170,11 +189,17 @@ struct rtpn_ctx {
     cudaStream_t stream = nullptr;   // work stream (user's or own)
     cudaStream_t own = nullptr;      // private stream (capture, default work stream)
     bool media_set = false;
+    // row pitch of the state and stride of its components: nx and V, but with rows padded to 16-byte
+    // groups while the automatic choice runs the staged kernel on a grid of other widths (padding: zeros)
+    int px = 0;
+    long long sV = 0;
+    bool dense_rows = false;         // no padded rows now (use_dense_rows)
     bool batch_member = false;       // created by rtpn_batch_create (its kernels take cubic cells)
     double* scat = nullptr;          // f_l (l = 0..N) of anisotropic scattering on the device, or null
     int fac_planes = rtpn::FAC_PLANES;  // factor planes allocated
     long long steps_done = 0;
     std::map<int, cudaGraphExec_t> graphs;  // pair-sequence graphs keyed by pair count
+    bool padded() const { return px != g.nx; }
     std::string err;
     unsigned* status = nullptr;      // device status words: [0] bounded-wait / check bits, [1..7] record
     void* stage_mem = nullptr;       // staged kernels: coupling tables of both classes + column starts

@@ -100,7 +100,7 @@ struct Args {
     const float* fac;
     const float* coefcol;   // [column 0..N][type][slot q 0..N/2][CPAD] of the source class (0 for l < M)
     const int* colstart;    // [2][N+2]: first local index of column M in class 0 / class 1
-    long long V;
+    long long V;            // cells: stride of the factor planes (dense rows)
     int nx, ny, nz, bc;
     int fac_ofs;
     float inv_h;
@@ -114,6 +114,8 @@ struct Args {
     unsigned* status;       // device status word (STATUS_TIMEOUT on a wait that ran out)
     unsigned wait_limit;    // try_wait polls (each up to WAIT_HINT_NS) before giving up
     long long skip_stage;   // stage index never issued (a wait that must run out); -1 normally
+    int px = 0;             // row pitch of the target array and stride of its components
+    long long sV = 0;
     float sy = 1.f;         // h / h_y: scale of the y differences (non-cubic cells)
 };
 
@@ -922,7 +924,7 @@ __device__ __forceinline__ void stage_kernel_body(const Args& a, unsigned char* 
     // the three live target columns; their roles (prev, cur, next) rotate by one per stage
     float2 wa[NLA], wb[NLA], wc[NLA];
 
-    const unsigned vb = (unsigned)(V * ES);  // bytes of a component
+    const unsigned vb = (unsigned)(a.sV * ES);  // bytes of a component of the target array
     unsigned limit = a.wait_limit;           // 0 once a wait has run out: the rest of the pass is not waited for
     unsigned tile = blockIdx.x;
     unsigned b = 0, ph = 0;                  // stage buffer, phase parity of its current use
@@ -954,7 +956,8 @@ __device__ __forceinline__ void stage_kernel_body(const Args& a, unsigned char* 
         }
 #pragma unroll
         for (int q = 0; q < NLA; ++q) wa[q] = wb[q] = wc[q] = make_float2(0.f, 0.f);
-        char* const tcell = reinterpret_cast<char*>(a.tgt) + cell * ES;
+        char* const tcell = reinterpret_cast<char*>(a.tgt) +
+                            (((long long)(g.z0 + lz) * a.ny + (g.y0 + ly)) * a.px + (g.x0 + lx)) * ES;
         unsigned comp = cA0;  // the first component of target column M in the target array
 
         // One column: its sub-stages sweep source column i into prev (column i - 1), cur (i) and next
