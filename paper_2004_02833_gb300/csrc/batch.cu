@@ -85,6 +85,8 @@ __global__ void __launch_bounds__(256) k_batch(const Inst* __restrict__ inst, in
         a.ntx = I.ntx;
         a.nty = I.nty;
         a.ntz = I.ntz;
+        if constexpr (win::prefetches(N))
+            win::prefetch_tile<N, A, S, false>(a, (int)(it - I.block0), threadIdx.x, blockDim.x);
         int x, y, z;
         if (win::cell_of(a, (int)(it - I.block0), threadIdx.x, &x, &y, &z))
             win::substep_cell<N, A, S>(a, coef_of<N, A>(), x, y, z);

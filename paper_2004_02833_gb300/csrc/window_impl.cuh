@@ -176,6 +176,47 @@ RTPN_HD bool cell_of(const Args& a, int blk, int tid, int* x, int* y, int* z) {
     return *x < a.nx && *y < a.ny && *z < a.nz;
 }
 
+// Orders whose tiles ask L2 for their rows first (prefetch_tile).  The sweep's loads wait for memory with
+// few of them in flight (a thread's registers hold its accumulators), so a tile's rows are requested
+// at once, without registers, and the sweep then finds them in L2 or on the way.  GB300, FP32, even /
+// odd pass without -> with: P5 128^3 0.115 / 0.133 -> 0.104 / 0.111 ms, P7 128^3 0.207 / 0.199 -> 0.180 /
+// 0.183, P9 96^3 0.156 / 0.164 -> 0.141 / 0.131; P3 gains nothing (0.059 / 0.054; its few rows are in
+// flight anyway, and a 32^3 grid loses 1 us), P15 loses (0.41 -> 0.45: its rows leave L1 and L2 again
+// before the sweep comes to them).  Asking for a tile that runs later is slower the later it runs
+// (P7: 0.195 ms for the tile 114 blocks ahead, 0.253 for 760).
+__host__ __device__ constexpr bool prefetches(int N) { return N >= 5 && N <= 9; }
+
+// Ask L2 for every row of tile blk: the sources of class 1 - A, then the targets, then with per-order
+// factors (ANISO) the factor rows of the targets.
+template <int N, int A, typename S, bool ANISO>
+__device__ __forceinline__ void prefetch_tile(const Args& a, int blk, int tid, int threads) {
+    constexpr int nc = (N + 1) * (N + 1), first = A == 1 ? 0 : class_size(N, 0);  // first source
+    constexpr int nl = (N - A) / 2 + 1;                                           // orders of class A
+    const int rows = a.ty * a.tz;
+    const int bz = blk % a.ntz, bx = (blk / a.ntz) % a.ntx, by = blk / a.ntz / a.ntx;
+    const int x0 = bx * a.tx, y0 = by * a.ty, z0 = bz * a.tz;
+    auto ask = [&](const char* base, int es, int r) {  // row r of the tile in the plane at base
+        const int y = y0 + r % a.ty, z = z0 + r / a.ty;
+        if (y >= a.ny || z >= a.nz) return;
+        const char* p = base + (((long long)z * a.ny + y) * a.nx + x0) * es;
+        const int bytes = (a.nx - x0 < a.tx ? a.nx - x0 : a.tx) * es;
+        for (int o = 0; o < bytes; o += 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + o));
+    };
+    for (int k = tid; k < nc * rows; k += threads) {
+        int c = k / rows + first;
+        if (c >= nc) c -= nc;
+        ask(reinterpret_cast<const char*>(a.u) + c * a.V * (long long)sizeof(S), (int)sizeof(S), k % rows);
+    }
+    if constexpr (ANISO)
+        for (int k = tid; k < 8 * nl * rows; k += threads) {
+            const int f = k / rows, g3 = f / (2 * nl), l = A + 2 * ((f >> 1) % nl);
+            // the four slot codes of class A: (x, y) free, z by the parity of the 2-slots
+            const int g = g3 + 4 * ((A + g3 + (g3 >> 1)) & 1);
+            const int plane = a.fac_ofs + aniso_plane(N, g, l) + (f & 1);
+            ask(reinterpret_cast<const char*>(a.fac + plane * a.V), 4, k % rows);
+        }
+}
+
 // SCALED: non-cubic cells (Section 2.1 divides each difference by its own axis' cell size); the
 // y and z differences are scaled by h / h_y and h / h_z, and 1/h (of x) is applied per target.
 // ANISO: anisotropic scattering (Section 2, Sigma_tl = Sigma_a + Sigma_s0 - Sigma_sl): every target
