@@ -8,6 +8,8 @@
 //  * conversions, the FP64 sum of u_0 and the non-finite count.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "rtpn_internal.h"
 
 namespace rtpn {
@@ -48,7 +50,7 @@ __device__ __forceinline__ bool neighbour(const Geom& g, int x, int y, int z, in
 // ------------------------------------------------------------------ substep (generic gather)
 template <typename S, typename F>
 __global__ void k_substep_generic(S* __restrict__ u, const F* __restrict__ fac,
-                                  PartnerTable<F> tab, Geom g, int fac_ofs) {
+                                  PartnerTable<F> tab, Geom g, int fac_ofs, int chunk) {
     const long long cell = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (cell >= g.V) return;
     const int x = (int)(cell % g.nx);
@@ -61,7 +63,8 @@ __global__ void k_substep_generic(S* __restrict__ u, const F* __restrict__ fac,
         ok[code] = neighbour(g, x, y, z, code >> 1, (code & 1) ? 1 : -1, &nb[code]);
         if (!ok[code]) nb[code] = cell;
     }
-    for (int t = 0; t < tab.na; ++t) {
+    const int t0 = blockIdx.y * chunk, t1 = min(t0 + chunk, tab.na);
+    for (int t = t0; t < t1; ++t) {
         F r = F(0);
         for (int p = tab.row[t]; p < tab.row[t + 1]; ++p) {
             const S* ub = u + (long long)tab.src[p] * g.V;
@@ -92,9 +95,17 @@ __global__ void k_substep_generic(S* __restrict__ u, const F* __restrict__ fac,
 template <typename S, typename F>
 void launch_substep_generic(S* u, const F* fac, const PartnerTable<F>& tab, const Geom& g,
                             int fac_ofs, cudaStream_t stream) {
+    // A thread walks `chunk` targets of its cell, one after another.  A small grid splits the targets over
+    // blockIdx.y until kBlocks blocks are in the launch (eight 256-thread blocks per SM): a target only
+    // reads the other class, so the split needs no order.  A large grid keeps them together, because
+    // targets of a cell share their sources through L1.
     const int bs = 256;
     const long long nb = (g.V + bs - 1) / bs;
-    k_substep_generic<S, F><<<(unsigned)nb, bs, 0, stream>>>(u, fac, tab, g, fac_ofs);
+    constexpr long long kBlocks = 152 * 8;
+    const int split = (int)std::max(1ll, std::min((long long)tab.na, (kBlocks + nb - 1) / nb));
+    const int chunk = std::max(1, (tab.na + split - 1) / split);
+    const dim3 grid((unsigned)nb, (unsigned)std::max(1, (tab.na + chunk - 1) / chunk));
+    k_substep_generic<S, F><<<grid, bs, 0, stream>>>(u, fac, tab, g, fac_ofs, chunk);
 }
 
 template void launch_substep_generic<double, double>(double*, const double*,
