@@ -268,6 +268,8 @@ struct alignas(sizeof(T) * W > 16 ? 16 : sizeof(T) * W) IoVec {
 template <typename A, typename B, int W, bool IN_ORDER>
 __global__ void __launch_bounds__(kIoThreads) k_reorder(const A* __restrict__ in, B* __restrict__ out,
                                                         const int* __restrict__ perm, long long V) {
+    pdl_trigger();
+    pdl_wait();
     const int c = blockIdx.y, p = perm[c];
     const IoVec<A, W>* src = reinterpret_cast<const IoVec<A, W>*>(in + (long long)(IN_ORDER ? c : p) * V);
     IoVec<B, W>* dst = reinterpret_cast<IoVec<B, W>*>(out + (long long)(IN_ORDER ? p : c) * V);
@@ -294,13 +296,13 @@ void launch_reorder(const A* in, B* out, const int* perm, int nc, long long V, b
     const long long n = wide ? V / 4 : V;
     const dim3 grid((unsigned)((n + kIoThreads * kIoGroups - 1) / (kIoThreads * kIoGroups)), (unsigned)nc);
     if (wide && in_order)
-        k_reorder<A, B, 4, true><<<grid, kIoThreads, 0, stream>>>(in, out, perm, V);
+        launch_pdl(k_reorder<A, B, 4, true>, grid, kIoThreads, 0, stream, in, out, perm, V);
     else if (wide)
-        k_reorder<A, B, 4, false><<<grid, kIoThreads, 0, stream>>>(in, out, perm, V);
+        launch_pdl(k_reorder<A, B, 4, false>, grid, kIoThreads, 0, stream, in, out, perm, V);
     else if (in_order)
-        k_reorder<A, B, 1, true><<<grid, kIoThreads, 0, stream>>>(in, out, perm, V);
+        launch_pdl(k_reorder<A, B, 1, true>, grid, kIoThreads, 0, stream, in, out, perm, V);
     else
-        k_reorder<A, B, 1, false><<<grid, kIoThreads, 0, stream>>>(in, out, perm, V);
+        launch_pdl(k_reorder<A, B, 1, false>, grid, kIoThreads, 0, stream, in, out, perm, V);
 }
 #define RTPN_REORDER(A, B) \
     template void launch_reorder<A, B>(const A*, B*, const int*, int, long long, bool, cudaStream_t);

@@ -28,6 +28,8 @@ __constant__ float c_coef[kSources * 10];
 
 template <typename S, bool SCALED, bool ANISO>
 __global__ void __launch_bounds__(256) k_window(Args a) {
+    pdl_trigger();
+    pdl_wait();
     if constexpr (prefetches(kN)) prefetch_tile<kN, kA, S, ANISO>(a, blockIdx.x, threadIdx.x, blockDim.x);
     int x, y, z;
     if (!cell_of(a, blockIdx.x, threadIdx.x, &x, &y, &z)) return;
@@ -38,11 +40,8 @@ template <bool SCALED, bool ANISO>
 int launch_form(int precision, const Args& a, cudaStream_t st) {
     const int threads = a.tx * a.ty * a.tz;
     const unsigned blocks = (unsigned)a.ntx * a.nty * a.ntz;
-    if (precision == RTPN_BF16)
-        k_window<__nv_bfloat16, SCALED, ANISO><<<blocks, threads, 0, st>>>(a);
-    else
-        k_window<float, SCALED, ANISO><<<blocks, threads, 0, st>>>(a);
-    return (int)cudaGetLastError();
+    if (precision == RTPN_BF16) return (int)launch_pdl(k_window<__nv_bfloat16, SCALED, ANISO>, blocks, threads, 0, st, a);
+    return (int)launch_pdl(k_window<float, SCALED, ANISO>, blocks, threads, 0, st, a);
 }
 
 // the form a launch needs; the non-cubic and anisotropic forms exist up to kExtendedMaxN (a
