@@ -174,6 +174,11 @@ int take_component(rtpn_ctx* ctx, int abi, void* dst, int dtype, int where) {
 }
 
 // ------------------------------------------------------------------ step schedule
+// whether the generic kernel has a compiled form for this FP64 context
+bool generic_compiled(const rtpn_ctx* ctx) {
+    return ctx->prec == RTPN_FP64 && !ctx->scat && cubic_cells(ctx->g) && window64_supported(ctx->N);
+}
+
 int run_pass(rtpn_ctx* ctx, int cls, int fac_ofs, cudaStream_t st) {
     if (ctx->active_kernel == RTPN_KERNEL_STAGE) {
         int rc = launch_stage(ctx, cls, fac_ofs, st, -1, STAGE_WAIT_LIMIT);
@@ -194,6 +199,9 @@ int run_pass(rtpn_ctx* ctx, int cls, int fac_ofs, cudaStream_t st) {
         int rc = launch_window(ctx->N, ctx->prec, w, st);
         if (rc) return fail(ctx, RTPN_ECUDA, std::string("window kernel: ") +
                                                  cudaGetErrorString((cudaError_t)rc));
+    } else if (ctx->prec == RTPN_FP64 && generic_compiled(ctx)) {
+        int rc = launch_window64(ctx->N, (double*)ctx->u, (const double*)ctx->fac, ctx->g, cls, fac_ofs, st);
+        if (rc) return fail(ctx, RTPN_ECUDA, std::string("generic kernel: ") + cudaGetErrorString((cudaError_t)rc));
     } else if (ctx->prec == RTPN_FP64) {
         if (ctx->scat && fac_ofs == FAC_HALF) fac_ofs = aniso_half_ofs(ctx->N);
         launch_substep_generic<double, double>((double*)ctx->u, (const double*)ctx->fac,
@@ -490,6 +498,10 @@ int choose_kernel(rtpn_ctx* ctx) {
         int rc = stage_prepare(ctx, ctx->tx, ctx->ty, ctx->tz, ctx->depth);
         if (rc) return fail(ctx, RTPN_ECUDA, std::string("staged kernel set-up: ") +
                                                  cudaGetErrorString((cudaError_t)rc));
+    }
+    if (k == RTPN_KERNEL_GENERIC && generic_compiled(ctx)) {
+        int rc = window64_prepare(ctx->md);
+        if (rc) return fail(ctx, RTPN_ECUDA, std::string("generic kernel constants: ") + cudaGetErrorString((cudaError_t)rc));
     }
     if (k == RTPN_KERNEL_WINDOW) {
         if (!window_supported(ctx->N, ctx->prec))

@@ -133,6 +133,11 @@ bool window_extended(int N);  // the window kernel's non-cubic and anisotropic f
 int window_prepare(const Model& md, double h, int precision);
 int launch_window(int N, int precision, const WindowLaunch& w, cudaStream_t st);
 
+// ---- the generic kernel's compiled FP64 form (window64.cu): cubic cells, isotropic scattering
+bool window64_supported(int N);
+int window64_prepare(const Model& md);  // uploads the constants of order N (idempotent); returns cudaError_t
+int launch_window64(int N, double* u, const double* fac, const Geom& g, int cls, int fac_ofs, cudaStream_t st);
+
 // ---- fused step kernels (kernels_fused.cu, fused.cu) ----
 // One pass of the even full step and the odd step after it, from state x into state y (another
 // buffer of the same layout).

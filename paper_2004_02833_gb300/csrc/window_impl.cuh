@@ -135,6 +135,24 @@ RTPN_HD float load_nc<__nv_bfloat16>(const __nv_bfloat16* p) {
     return __bfloat162float(*p);
 #endif
 }
+// loads of a stored value and of a factor in the arithmetic type F (double: FP64 storage only)
+RTPN_HD double ro(const double* p) {
+    RTPN_CHECK_PTR(p);
+#ifdef __CUDA_ARCH__
+    return __ldg(p);
+#else
+    return *p;
+#endif
+}
+template <typename F, typename S>
+RTPN_HD F load_as(const S* p) {
+    if constexpr (std::is_same_v<F, double>)
+        return ro(p);
+    else
+        return load_nc<S>(p);
+}
+RTPN_HD float fma_f(float a, float b, float c) { return fmaf(a, b, c); }
+RTPN_HD double fma_f(double a, double b, double c) { return fma(a, b, c); }
 template <typename S>
 RTPN_HD void store(S* p, float v);
 template <>
@@ -148,6 +166,16 @@ RTPN_HD void store<__nv_bfloat16>(__nv_bfloat16* p, float v) {
     *p = __float2bfloat16_rn(v);
 }
 
+template <typename F, typename S>
+RTPN_HD void store_as(S* p, F v) {
+    if constexpr (std::is_same_v<F, double>) {
+        RTPN_CHECK_PTR(p);
+        *p = v;
+    } else {
+        store<S>(p, v);
+    }
+}
+
 struct Args {
     void* u;
     const float* fac;
@@ -159,6 +187,7 @@ struct Args {
     int ntx, nty, ntz;  // tiles per axis
     float sy = 1.f, sz = 1.f;  // h / h_y, h / h_z: the y and z differences' scale (non-cubic cells)
     int aniso = 0;             // factors per (sub-grid, order l): anisotropic scattering
+    double inv_h64 = 0;        // 1 / h of the FP64 arithmetic
 };
 
 // coef[j * 10 + k]: source j (local index in class B), relation k: M_d[a][b] * dir, where dir = +1 if
@@ -225,8 +254,11 @@ __device__ __forceinline__ void prefetch_tile(const Args& a, int blk, int tid, i
 // Both forms are compiled up to order kExtendedMaxN: P39 runs non-cubic cells on the staged
 // kernel, and its window body is the slowest to compile.
 constexpr int kExtendedMaxN = 15;
-template <int N, int A, typename S, bool SCALED = false, bool ANISO = false>
-RTPN_HD void substep_cell(const Args& a, const float* __restrict__ coef, int x, int y, int z) {
+// F: arithmetic type, float or (FP64 storage, factors and constants) double.
+template <int N, int A, typename S, bool SCALED = false, bool ANISO = false, typename F = float>
+RTPN_HD void substep_cell(const Args& a, const F* __restrict__ coef, int x, int y, int z) {
+    const F* const fac = reinterpret_cast<const F*>(a.fac);
+    const F inv_h = std::is_same_v<F, double> ? (F)a.inv_h64 : (F)a.inv_h;
     constexpr int B = 1 - A;
     constexpr int NL = N / 2 + 1;
     const long long V = a.V;
@@ -251,35 +283,35 @@ RTPN_HD void substep_cell(const Args& a, const float* __restrict__ coef, int x, 
     S* tgtbase = u + (long long)(A == 0 ? 0 : class_size(N, 0)) * V + cell;
 
     // ---- factors of the four target sub-grids (and u_0)
-    float al[8], be[8];
+    F al[8], be[8];
 #pragma unroll
     for (int g = 0; g < 8; ++g) {
-        al[g] = 0.f;
-        be[g] = 0.f;
+        al[g] = F(0);
+        be[g] = F(0);
     }
     // be holds beta / h: the accumulators carry sum coef * (u(neighbour) - u(i)) without 1/h
     static_for<8>([&](auto gi) {
         constexpr int g = decltype(gi)::value;
         constexpr int twos = (g & 1) + ((g >> 1) & 1) + ((g >> 2) & 1);
         if constexpr (twos % 2 == A && !ANISO) {
-            al[g] = ro(a.fac + (long long)(a.fac_ofs + 2 * g) * V + cell);
-            be[g] = ro(a.fac + (long long)(a.fac_ofs + 2 * g + 1) * V + cell) * a.inv_h;
+            al[g] = ro(fac + (long long)(a.fac_ofs + 2 * g) * V + cell);
+            be[g] = ro(fac + (long long)(a.fac_ofs + 2 * g + 1) * V + cell) * inv_h;
         }
     });
-    float al0 = 0.f, be0 = 0.f, ga0 = 0.f;
+    F al0 = F(0), be0 = F(0), ga0 = F(0);
     if constexpr (A == 0) {
-        al0 = ro(a.fac + (long long)FAC_U0 * V + cell);
-        be0 = ro(a.fac + (long long)(FAC_U0 + 1) * V + cell) * a.inv_h;
-        ga0 = ro(a.fac + (long long)(FAC_U0 + 2) * V + cell);
+        al0 = ro(fac + (long long)FAC_U0 * V + cell);
+        be0 = ro(fac + (long long)(FAC_U0 + 1) * V + cell) * inv_h;
+        ga0 = ro(fac + (long long)(FAC_U0 + 2) * V + cell);
     }
 
-    float acc[3][2][NL];
+    F acc[3][2][NL];
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int t = 0; t < 2; ++t)
 #pragma unroll
-            for (int j = 0; j < NL; ++j) acc[i][t][j] = 0.f;
+            for (int j = 0; j < NL; ++j) acc[i][t][j] = F(0);
 
     // finalize target column M (every contribution is in)
     auto finalize = [&](auto Mi) {
@@ -293,22 +325,22 @@ RTPN_HD void substep_cell(const Args& a, const float* __restrict__ coef, int x, 
                     if constexpr (l <= N) {
                         constexpr int idx = local_index(N, A, l, M, t);
                         S* p = tgtbase + (long long)idx * V;
-                        const float old = load_nc<S>(p);
-                        const float r = acc[M % 3][t][j];
-                        acc[M % 3][t][j] = 0.f;
-                        float nv;
+                        const F old = load_as<F, S>(p);
+                        const F r = acc[M % 3][t][j];
+                        acc[M % 3][t][j] = F(0);
+                        F nv;
                         if constexpr (A == 0 && l == 0) {
-                            nv = fmaf(al0, old, fmaf(-be0, r, ga0));
+                            nv = fma_f(al0, old, fma_f(-be0, r, ga0));
                         } else if constexpr (ANISO) {
                             constexpr int pl = aniso_plane(N, slot_code(l, M, t), l);
-                            const float alv = ro(a.fac + (long long)(a.fac_ofs + pl) * V + cell);
-                            const float bev = ro(a.fac + (long long)(a.fac_ofs + pl + 1) * V + cell) * a.inv_h;
-                            nv = fmaf(alv, old, -bev * r);
+                            const F alv = ro(fac + (long long)(a.fac_ofs + pl) * V + cell);
+                            const F bev = ro(fac + (long long)(a.fac_ofs + pl + 1) * V + cell) * inv_h;
+                            nv = fma_f(alv, old, -bev * r);
                         } else {
                             constexpr int g = slot_code(l, M, t);
-                            nv = fmaf(al[g], old, -be[g] * r);
+                            nv = fma_f(al[g], old, -be[g] * r);
                         }
-                        store<S>(p, nv);
+                        store_as<F, S>(p, nv);
                     }
                 });
             }
@@ -326,14 +358,14 @@ RTPN_HD void substep_cell(const Args& a, const float* __restrict__ coef, int x, 
                     if constexpr (ls <= N) {
                         constexpr int sidx = local_index(N, B, ls, Ms, ts);
                         const S* p = srcbase + (long long)sidx * V;
-                        const float c = load_nc<S>(p);
-                        float d[3] = {0.f, 0.f, 0.f};
+                        const F c = load_as<F, S>(p);
+                        F d[3] = {F(0), F(0), F(0)};
                         constexpr int sl[3] = {slot_x(Ms, ts), slot_y(ts), slot_z(ls, Ms)};
                         static_for<3>([&](auto di) {
                             constexpr int ax = decltype(di)::value;
                             if constexpr (needs_axis(N, ls, Ms, ts, ax)) {
                                 constexpr int side = sl[ax] == 1 ? 1 : 0;
-                                const float nb = ok[ax][side] ? load_nc<S>(p + off[ax][side]) : 0.f;
+                                const F nb = ok[ax][side] ? load_as<F, S>(p + off[ax][side]) : F(0);
                                 d[ax] = nb - c;
                                 if constexpr (SCALED && ax > 0) d[ax] *= ax == 1 ? a.sy : a.sz;
                             }
@@ -344,7 +376,7 @@ RTPN_HD void substep_cell(const Args& a, const float* __restrict__ coef, int x, 
                             if constexpr (T.ok) {
                                 constexpr int jt = (T.l - first_l(T.M, A)) / 2;
                                 acc[T.M % 3][T.t][jt] =
-                                    fmaf(coef[sidx * 10 + k], d[T.axis], acc[T.M % 3][T.t][jt]);
+                                    fma_f(coef[sidx * 10 + k], d[T.axis], acc[T.M % 3][T.t][jt]);
                             }
                         });
                     }
@@ -360,7 +392,8 @@ RTPN_HD void substep_cell(const Args& a, const float* __restrict__ coef, int x, 
 // Coefficient table of target class A: for every source j of class 1 - A (internal order) and
 // relation k, M_d[a][b] * dir.  Cross-checks the compile-time relations against the model's
 // nonzeros; returns false on any mismatch.
-inline bool coef_table(const Model& md, int A, std::vector<float>* out) {
+template <typename F>
+bool coef_table(const Model& md, int A, std::vector<F>* out) {
     const int N = md.N, B = 1 - A;
     const int base = B == 0 ? 0 : md.ne;
     const int nS = class_size(N, B);
@@ -371,7 +404,7 @@ inline bool coef_table(const Model& md, int A, std::vector<float>* out) {
         nz[(long long)e.a * md.nc + e.b] = {e.axis, e.v};
         if (md.comp[e.b].cls == B) ++expected;
     }
-    out->assign((size_t)nS * 10, 0.f);
+    out->assign((size_t)nS * 10, F(0));
     long long found = 0;
     for (int j = 0; j < nS; ++j) {
         const int b = md.abi_of_internal[base + j];
@@ -384,7 +417,7 @@ inline bool coef_table(const Model& md, int A, std::vector<float>* out) {
             auto it = nz.find((long long)a * md.nc + b);
             if (it == nz.end() || it->second.first != T.axis) return false;
             const double dir = c.slot[T.axis] == 1 ? 1.0 : -1.0;
-            (*out)[(size_t)j * 10 + k] = (float)(it->second.second * dir);
+            (*out)[(size_t)j * 10 + k] = (F)(it->second.second * dir);
             ++found;
         }
     }
