@@ -659,9 +659,10 @@ int rtpn::create_context(rtpn_ctx** out, int N, int nx, int ny, int nz, double h
     if (e != cudaSuccess) return bail(fail(ctx, RTPN_ENOMEM, "scratch allocation failed"));
     e = cudaMalloc(&ctx->counter, sizeof(unsigned long long));
     if (e != cudaSuccess) return bail(fail(ctx, RTPN_ENOMEM, "scratch allocation failed"));
-    e = cudaMalloc(&ctx->status, 8 * sizeof(unsigned));
+    e = cudaMalloc(&ctx->status, 10 * sizeof(unsigned));
     if (e != cudaSuccess) return bail(fail(ctx, RTPN_ENOMEM, "status allocation failed"));
-    e = cudaMemsetAsync(ctx->status, 0, 8 * sizeof(unsigned), ctx->stream);
+    ctx->tickets = ctx->status + 8;
+    e = cudaMemsetAsync(ctx->status, 0, 10 * sizeof(unsigned), ctx->stream);
     if (e != cudaSuccess) return bail(fail(ctx, RTPN_ECUDA, cudaGetErrorString(e)));
     if ((rc = upload_tables(ctx))) return bail(rc);
     e = cudaMemsetAsync(ctx->u, 0, state_room, ctx->stream);

@@ -241,6 +241,7 @@ static bool base_args(const rtpn_ctx* ctx, const stg::Variant& v, int coef_cls, 
     a.sV = a.V;
     a.nc = ctx->md.nc;
     a.status = ctx->status;
+    a.tickets = ctx->tickets;
     a.wait_limit = (unsigned)STAGE_WAIT_LIMIT;
     a.skip_stage = -1;
     *out = a;

@@ -231,6 +231,7 @@ struct rtpn_ctx {
     std::map<int, cudaGraphExec_t> graphs;  // pair-sequence graphs keyed by pair count
     bool padded() const { return px != g.nx; }
     std::string err;
+    unsigned* tickets = nullptr;     // staged kernels: tiles handed out, CTAs done (zero between passes)
     unsigned* status = nullptr;      // device status words: [0] bounded-wait / check bits, [1..7] record
     void* stage_mem = nullptr;       // staged kernels: coupling tables of both classes + column starts
     size_t stage_tab_bytes[2] = {0, 0};

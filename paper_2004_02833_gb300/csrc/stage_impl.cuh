@@ -39,9 +39,12 @@
 // accumulators); P19 96 x 96 x 128 0.54 ms (5.2 TB/s); P15 96^3 0.41 -> 0.27 ms (5.1 TB/s, 77 %); P7 128^3
 // 0.46 -> 0.19 ms (4.3 TB/s): barriers and copies per stage.
 //
-// CTAs are persistent (one or two per SM) and walk tiles in z-chunked order (z fastest inside a chunk of kz
-// tile layers, then x, then y), so the CTAs at work at any time cover a compact block and read one
-// another's halos from L2.  Every mbarrier wait is bounded: one that runs out sets a status bit;
+// CTAs are persistent (one or two per SM) and take tiles by ticket (an atomic counter) in z-chunked order (z
+// fastest inside a chunk of kz tile layers, then x, then y), so the CTAs at work at any time cover a compact
+// block and read one another's halos from L2.  With fixed shares instead, a pass waited for the CTAs that
+// started late because another stream's kernel held their SMs (three P39 160^3 contexts in turn, two
+// steps and the state out each: 54.2 ms against 42.4 with tickets; one pass alone 7.4 -> 7.1 ms).
+// Every mbarrier wait is bounded: one that runs out sets a status bit;
 // a consumer then stops waiting (the rest of its pass is undefined, as the caller is told), a
 // producer leaves after a bounded wait for the copies it issued.
 #pragma once
@@ -113,6 +116,7 @@ struct Args {
     int nc;                   // components (bound of the 4th tensor coordinate)
     unsigned* status;       // device status word (STATUS_TIMEOUT on a wait that ran out)
     unsigned wait_limit;    // try_wait polls (each up to WAIT_HINT_NS) before giving up
+    unsigned* tickets;      // [0] tiles handed out past the first round, [1] CTAs that are done (both 0 between passes)
     long long skip_stage;   // stage index never issued (a wait that must run out); -1 normally
     int px = 0;             // row pitch of the target array and stride of its components
     long long sV = 0;
@@ -120,6 +124,9 @@ struct Args {
 };
 
 __host__ __device__ constexpr int pad128(int bytes) { return (bytes + 127) / 128 * 128; }
+
+// Tile indices handed from the producer that draws them to the other warps of the CTA.
+constexpr int kNextRing = 4;
 
 // Width XW of the x halo box: the widest group of 16-byte aligned columns that divides TX and
 // leaves RY = TX / XW >= TY rows (so the box volume per component is TZ * TX = U when TY == TZ).
@@ -164,7 +171,8 @@ struct Layout {
     static constexpr int COEFO = SRCO + 2 * SRC_T;
     static constexpr int BUF = COEFO + pad128(COEF_COL);  // one stage buffer
     static constexpr int BARS = pad128(2 * NB * 8);
-    static constexpr int BYTES = NB * BUF + BARS + 128;   // ring, mbarriers, base alignment slack
+    static constexpr int NEXT = 128;                      // the next tiles' indices (kNextRing)
+    static constexpr int BYTES = NB * BUF + BARS + NEXT + 128;  // ring, mbarriers, tiles, alignment slack
     static_assert(TY == TZ, "every box kind has the volume TY * TX per component only if TY == TZ");
     static_assert(TX % G == 0, "tile width must be a multiple of the 16-byte group");
     static_assert(CELLS % 32 == 0, "the tile's cells must fill whole warps");
@@ -545,7 +553,7 @@ RTPN_HD unsigned stage_bytes(const StageRuns& r, int C = 0) {
 // of this CTA's sequence into the ring.  One lane issues; everything else is the same for the warp.
 template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH>
 __device__ __forceinline__ void stage_producer(const Args& a, unsigned char* bufs, unsigned full0,
-                                               unsigned empty0, int total, int t) {
+                                               unsigned empty0, volatile unsigned* next, int t) {
     using L = Layout<N, A, S, TX, TY, TZ, NB, NCH>;
     constexpr int B = 1 - A;
     constexpr int NST = N + 2;
@@ -560,17 +568,34 @@ __device__ __forceinline__ void stage_producer(const Args& a, unsigned char* buf
     for (int k = 0; k < L::NMAP; ++k)
         asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(a.tmap + k) : "memory");
 
+    constexpr int TS = tile_stages<N, A, NCH>();
+    static_assert(TS >= NB + 2, "a tile's second stage is consumed before the next tile is issued");
     int s = 0;
     bool failed = false;
-    int b = 0, i = 0, C = first_chunk<N, A, NCH>(0);
+    int b = 0;
     unsigned ph = 0;  // phase parity of buffer b's current use (flips when b wraps)
-    unsigned tile = blockIdx.x;
-    TileGeo g = tile_geo<TX, TY, TZ, L::G>(a, tile);
-    for (; s < total; ++s) {
+    unsigned tile = blockIdx.x, ticket = 0;
+    for (unsigned k = 0;; ++k) {
+      TileGeo g{};
+      int i = 0, C = first_chunk<N, A, NCH>(0);
+      int j = 0;
+      for (; j < TS; ++j, ++s) {
         const unsigned full = full0 + 8 * b;
         if (s >= NB && !wait_phase(empty0 + 8 * b, ph ^ 1u, a.wait_limit)) {
             failed = true;  // the consumers did not release the buffer's previous stage
             break;
+        }
+        // The next tile: producer 0 draws it while the tile's first stage is issued and hands it on before
+        // the arrival of the second; the consumers have it with that stage, producer 1 with their release.
+        if (j == 0) {
+            if (k > 0) tile = next[k % kNextRing];
+            if (tile >= (unsigned long long)a.tiles) break;
+            g = tile_geo<TX, TY, TZ, L::G>(a, tile);
+            offA = offB = 0;
+            if (t == 0 && lane == 0) ticket = atomicAdd(a.tickets, 1u);
+        } else if (j == 1 && t == 0) {
+            if (lane == 0) next[(k + 1) % kNextRing] = gridDim.x + ticket;
+            __syncwarp();
         }
         const unsigned buf = smem_addr(bufs + b * L::BUF);
         const StageRuns r = stage_runs<N, A, NCH>(i, C);
@@ -605,23 +630,28 @@ __device__ __forceinline__ void stage_producer(const Args& a, unsigned char* buf
             b = 0;
             ph ^= 1u;
         }
-        // the next sub-stage: of this column, the next column, or the next tile
+        // the next sub-stage: of this column or the next
         if (++C == NCH) {
             offB += ntypes(i) * column_len(N, i, B);
             if (i >= 1) offA += ntypes(i - 1) * column_len(N, i - 1, A);
-            if (++i == NST) {
-                i = offA = offB = 0;
-                tile += gridDim.x;
-                if (s + 1 < total) g = tile_geo<TX, TY, TZ, L::G>(a, tile);
-            }
-            C = first_chunk<N, A, NCH>(i);
+            if (++i < NST) C = first_chunk<N, A, NCH>(i);
         }
+      }
+      if (j < TS) break;  // no tile left, or a wait ran out
     }
     if (failed && lane == 0) atomicOr(a.status, STATUS_TIMEOUT);
     // before the CTA ends, the copies of the last stages issued must have landed
     const int first = s > NB ? s - NB : 0;
     for (int q = first; q < s; ++q)
         if (q != a.skip_stage) wait_phase(full0 + 8 * (q % NB), (unsigned)((q / NB) & 1), a.wait_limit);
+    // the last CTA to draw its last ticket clears the counters for the next pass
+    if (t == 0 && lane == 0) {
+        __threadfence();
+        if (atomicAdd(a.tickets + 1, 1u) == gridDim.x - 1) {
+            a.tickets[0] = 0;
+            a.tickets[1] = 0;
+        }
+    }
 }
 
 // ---------------------------------------------------------------- the consumers' column work
@@ -901,6 +931,8 @@ __device__ __forceinline__ void stage_kernel_body(const Args& a, unsigned char* 
     unsigned char* bufs = smem;
     unsigned long long* bars = reinterpret_cast<unsigned long long*>(bufs + NB * L::BUF);
     const unsigned full0 = smem_addr(&bars[0]), empty0 = smem_addr(&bars[NB]);
+    volatile unsigned* next = reinterpret_cast<unsigned*>(bufs + NB * L::BUF + L::BARS);
+    if (tid < kNextRing) next[tid] = 0xffffffffu;  // no tile
     if (tid == 0) {
         for (int b = 0; b < NB; ++b) {
             mbar_init(full0 + 8 * b, kProducers);  // each producer's arrive.expect_tx
@@ -910,10 +942,8 @@ __device__ __forceinline__ void stage_kernel_body(const Args& a, unsigned char* 
     }
     __syncthreads();
 
-    const int my_tiles = a.tiles > blockIdx.x ? (int)((a.tiles - 1 - blockIdx.x) / gridDim.x) + 1 : 0;
-    const int total = my_tiles * tile_stages<N, A, NCH>();
     if (warp >= L::CONSUMER_WARPS) {
-        stage_producer<N, A, S, TX, TY, TZ, NB, NCH>(a, bufs, full0, empty0, total, warp - L::CONSUMER_WARPS);
+        stage_producer<N, A, S, TX, TY, TZ, NB, NCH>(a, bufs, full0, empty0, next, warp - L::CONSUMER_WARPS);
         return;
     }
 
@@ -928,7 +958,10 @@ __device__ __forceinline__ void stage_kernel_body(const Args& a, unsigned char* 
     unsigned limit = a.wait_limit;           // 0 once a wait has run out: the rest of the pass is not waited for
     unsigned tile = blockIdx.x;
     unsigned b = 0, ph = 0;                  // stage buffer, phase parity of its current use
-    for (int k = 0; k < my_tiles; ++k, tile += gridDim.x) {
+    // tile after tile until none is left (a consumer whose wait ran out leaves after the tile it is on)
+    for (unsigned k = 0; k == 0 || limit != 0; ++k) {
+        if (k > 0) tile = next[k % kNextRing];
+        if (tile >= (unsigned long long)a.tiles) break;
         const TileGeo g = tile_geo<TX, TY, TZ, L::G>(a, tile);
         const bool active = lx < g.wx && ly < g.wy && lz < g.wz;
         const long long cell = ((long long)(g.z0 + lz) * a.ny + (g.y0 + ly)) * a.nx + (g.x0 + lx);
