@@ -406,9 +406,9 @@ void release(rtpn_ctx* ctx) {
 // one.  Padding costs at most three (FP32) or seven (BF16) columns of traffic; the kernels that take any
 // width cost far more there (GB300, FP32, a pass: P15 61 x 77 x 75 0.14 ms against
 // 0.24 on the window kernel, P19 0.18 against 1.09 on the generic one, P39 0.68 against 3.25 on the window
-// kernel).  Below kStageMinN the unrolled window body is
-// small enough for the instruction cache and the staged kernel's barriers and copies per stage weigh more
-// (P7 128^3: 0.40 ms a step with the window kernel, 0.38 with the staged one).
+// kernel).  Below kStageMinN the unrolled window body is small enough for the instruction cache and the
+// staged kernel's barriers and copies per stage weigh more (P7 128^3: 0.36 ms a step with the window
+// kernel, 0.38 with the staged one).
 constexpr bool kStageInAuto = true;
 constexpr int kStageMinN = 15;
 

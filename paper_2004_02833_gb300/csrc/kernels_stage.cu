@@ -3,6 +3,7 @@
 
 #include <cmath>
 #include <mutex>
+#include <numeric>
 #include <vector>
 
 #include "stage_impl.cuh"
@@ -92,17 +93,16 @@ static bool make_maps(CUtensorMap* out, void* base, int precision, const rtpn::G
 
 // The default variant for a grid: the one whose tiles cover it at the least cost, rounds of the persistent
 // CTAs times the cost of a round.  Padding at the grid's edges and an emptier last round cost as much as
-// full tiles.  A round costs its cells per SM plus a fixed part (the barriers and the issue of the copies
-// of every stage; above order 30, where one window fills the registers, the latency of a warp's own
-// instructions), in cells: P15 96^3 0.300 ms with 288-cell tiles and 0.276 with 384, P7 128^3 0.246 ms with
-// 256-cell and 0.195 with 512-cell tiles, P39 120^3 69 us a round with 192 cells and 82 with 320.  Rows
-// that do not start on 128-byte lines touch one more line each: P39 82 us a round of 32x3x3 tiles at 96^3
-// (aligned), 113 at 120^3 (GB300, FP32).
+// full tiles.  A round costs its cells per SM plus a fixed part in cells: the issue of a stage's boxes and its
+// barriers (90 with the seven boxes a type of a two-plane tile), above order 30 also the latency of a warp's
+// own instructions (400 in all).  Rows off the 128-byte lines touch more lines than they fill; half of that
+// excess is felt.  GB300, FP32, a round: P15 96^3 13.2 us with two CTAs of 32x2x2, 17.1 with one of 96x2x2,
+// 23.8 with one of 32x4x4 (0.303, 0.274 and 0.286 ms a pass; P19 80^3 0.246 ms with 80x2x2, 0.289 with two CTAs
+// of 40x2x2); P39 69 us with 192 cells, 82 with 320, and 32x3x3 tiles 82 us at 96^3 (aligned), 113 at 120^3.
 static const Variant* best_variant(int N, int precision, int depth, const rtpn::Geom& g, int px, int sms) {
     const Variant* best = nullptr;
     double best_cost = 0;
     const int es = precision == RTPN_BF16 ? 2 : 4;
-    const double fixed = N > 30 ? 400 : 180;
     for (const auto& v : kVariants) {
         if (v.N != N || (depth != 0 && v.depth != depth) || !fits(v, precision)) continue;
         int geo[4];
@@ -112,8 +112,9 @@ static const Variant* best_variant(int N, int precision, int depth, const rtpn::
         const long long rounds = (tiles + slots - 1) / slots;
         // a grid of less than a round leaves SMs with fewer CTAs than they hold
         const long long per_sm = rounds > 1 ? geo[1] : (tiles + sms - 1) / sms;
-        const int row = v.tx * es;
-        const double lines = row % 128 == 0 && px * es % 128 == 0 ? 1.0 : 1.0 + 48.0 / row;
+        const double fixed = (N > 30 ? 400.0 : 90.0) * (2 * v.tz + 3) / 7;
+        const int row = v.tx * es, align = std::gcd(std::gcd(row, px * es), 128);
+        const double lines = 1.0 + 0.5 * (128 - align) / row;  // row / 128 lines filled, (128 - align) / 128 more touched
         const double cost = rounds * (per_sm * v.tx * v.ty * v.tz * lines + fixed);
         if (!best || cost < best_cost) {
             best = &v;

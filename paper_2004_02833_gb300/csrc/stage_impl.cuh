@@ -11,7 +11,7 @@
 //    from sources of the other type (Eq. 3's Mx and Mz keep the type, My swaps it), so the two lanes
 //    run the same code and share one coupling constant for x and y.  Each thread keeps three columns
 //    of N/2 + 1 accumulator pairs.  (Two threads per cell, one per type, took twice the instructions
-//    for the same cells: P39 160^3 FP32, 11.0 ms a pass against 7.4 ms now.)
+//    for the same cells: P39 160^3 FP32, 11.0 ms a pass against 7.1 ms now.)
 //  * The column sweep is a runtime loop whose body handles one column for every l slot; the three
 //    live target columns are register arrays that change roles from column to column (the loop is
 //    unrolled by three), so the body is the same for every column and fits the instruction cache.
@@ -34,8 +34,8 @@
 //    (uniform registers) instead of by one lane.  NB stage buffers form a ring with a full / empty
 //    mbarrier pair each, so up to NB - 1 stages are in flight while one is computed.
 //
-// What bounds it (GB300, FP32, a pass, before -> now, of the 6697 GB/s copy): P39 160^3 11.0 -> 7.4 ms
-// (5.3 TB/s, 79 %): the latency of a warp's own instructions, 10 consumer warps with 168 registers (120
+// What bounds it (GB300, FP32, a pass, before -> now, of the 6697 GB/s copy): P39 160^3 11.0 -> 7.1 ms
+// (5.6 TB/s, 83 %): the latency of a warp's own instructions, 10 consumer warps with 168 registers (120
 // accumulators); P19 96 x 96 x 128 0.54 ms (5.2 TB/s); P15 96^3 0.41 -> 0.27 ms (5.1 TB/s, 77 %); P7 128^3
 // 0.46 -> 0.19 ms (4.3 TB/s): barriers and copies per stage.
 //

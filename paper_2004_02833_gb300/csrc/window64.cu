@@ -4,8 +4,9 @@
 // An FP64 pass is bound by the FP64 rate (about 0.6 T fused multiply-adds a second on a GB300).  The
 // partner-table kernel takes a difference and a product for every (target, partner) pair, about 17
 // operations a source; the window body takes each source's three differences once and at most ten
-// products, 12 on average, with no index loads.  GB300, without -> with: P3 32^3, forty steps
-// with the state out, 534 -> 419 us, P7 64^3 0.29 / 0.31 -> 0.20 / 0.20 ms a pass.  Orders up to 9, cubic cells, isotropic scattering; the table kernel takes the rest.
+// products, 12 on average, with no index loads.  GB300, without -> with: P3 32^3, forty steps with the state
+// out, 534 -> 419 us; P7 64^3 0.29 / 0.31 -> 0.20 / 0.20 ms an even / odd pass.  Orders up to 9, cubic cells,
+// isotropic scattering; the table kernel takes the rest.
 #include <mutex>
 #include <set>
 #include <utility>
