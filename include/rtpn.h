@@ -160,7 +160,7 @@ int rtpn_set_stream(rtpn_ctx* ctx, void* stream);
  * tile_x and tile_y must be 0 (or 32 and 8); tile_z is the number of z planes a CTA streams through
  * (0 = one wave of resident CTAs).  Selecting it allocates a second state buffer (RTPN_ENOMEM if
  * that fails); RTPN_EUNSUPPORTED for a batch instance.
- * RTPN_KERNEL_AUTO picks STAGE (for N >= 15; where nx gives no 16-byte rows the state's rows are padded
+ * RTPN_KERNEL_AUTO picks STAGE (for N >= 15; where nx >= 8 gives no 16-byte rows the state's rows are padded
  * inside the library, except in a batch), then WINDOW, then GENERIC; with non-cubic cells STAGE (any
  * compiled N), else GENERIC; with anisotropic scattering GENERIC.  Moving between padded and dense rows
  * rearranges the state in place.

@@ -411,6 +411,10 @@ void release(rtpn_ctx* ctx) {
 // kernel, 0.38 with the staged one).
 constexpr bool kStageInAuto = true;
 constexpr int kStageMinN = 15;
+// Rows of fewer than 8 cells are not padded: up to three cells in four would be padding, and the staged tiles
+// are at least 32 cells wide (P19 64 x 64 x nx FP32, a pass, staged against the generic kernel: nx = 5 0.080 and
+// 0.057 ms, 7 0.079 and 0.077, 9 0.099 and 0.095; 75 0.18 and 1.09 at 61 x 77).
+constexpr int kPadMinNx = 8;
 
 // Row pitch of the state: nx, or nx padded to 16-byte rows.  The state is rearranged in place, a component
 // at a time through the staging plane (its buffer holds the padded state if the context can ever need
@@ -441,7 +445,8 @@ int set_rows(rtpn_ctx* ctx, bool padded) {
 
 // whether the automatic choice may pad the rows for the staged kernel
 bool may_pad(const rtpn_ctx* ctx) {
-    return kStageInAuto && ctx->N >= kStageMinN && !ctx->batch_member && stage_compiled(ctx->N, ctx->prec);
+    return kStageInAuto && ctx->N >= kStageMinN && !ctx->batch_member && ctx->g.nx >= kPadMinNx &&
+           stage_compiled(ctx->N, ctx->prec);
 }
 
 int choose_kernel(rtpn_ctx* ctx) {
@@ -667,6 +672,9 @@ int rtpn::create_context(rtpn_ctx** out, int N, int nx, int ny, int nz, double h
     if ((rc = upload_tables(ctx))) return bail(rc);
     e = cudaMemsetAsync(ctx->u, 0, state_room, ctx->stream);
     if (e != cudaSuccess) return bail(fail(ctx, RTPN_ECUDA, cudaGetErrorString(e)));
+    // a state of zeros needs no rearranging: padded from the start where the choice below pads it
+    ctx->px = (nx + grp - 1) / grp * grp;
+    ctx->sV = (long long)ctx->px * ny * nz;
     if ((rc = choose_kernel(ctx))) return bail(rc);
     e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return bail(fail(ctx, RTPN_ECUDA, cudaGetErrorString(e)));

@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 CASES = [
     # N, shape (nz, ny, nx), bc
     (15, (5, 6, 75), "periodic"),
-    (15, (4, 3, 1), "vacuum"),
+    (15, (4, 3, 9), "vacuum"),
     (15, (3, 4, 66), "vacuum"),
     (19, (4, 5, 35), "periodic"),
     (29, (3, 2, 9), "vacuum"),
