@@ -45,8 +45,9 @@
 // started late because another stream's kernel held their SMs (three P39 160^3 contexts in turn, two
 // steps and the state out each: 54.2 ms against 42.4 with tickets; one pass alone 7.4 -> 7.1 ms).
 // Every mbarrier wait is bounded: one that runs out sets a status bit;
-// a consumer then stops waiting (the rest of its pass is undefined, as the caller is told), a
-// producer leaves after a bounded wait for the copies it issued.
+// a consumer then neither waits nor hands a buffer back for the rest of its tile (whose results are
+// undefined, as the caller is told), so that the producers run out of buffers instead of reusing one
+// whose copies are in flight; a producer leaves after a bounded wait for the copies it issued.
 #pragma once
 
 #include <cuda.h>
@@ -549,6 +550,16 @@ RTPN_HD unsigned stage_bytes(const StageRuns& r, int C = 0) {
     return type_bytes<N, A, S, TX, TY, TZ, NB, NCH>(r, C, 0) + type_bytes<N, A, S, TX, TY, TZ, NB, NCH>(r, C, 1);
 }
 
+// What the ring rests on when a wait runs out (also run by a host model of its barriers).  Stage s uses
+// buffer s % nb; phase s / nb of the buffer's full barrier is the one its copies complete.
+// A consumer warp whose wait ran out (its limit is then 0) hands no buffer back: the buffer may have copies in
+// flight, or none issued, and a producer given it would arrive on a phase that is not complete.
+RTPN_HD constexpr bool hands_back(unsigned limit) { return limit != 0; }
+// A producer that issued the stages below s waits for those from here on before its CTA ends: the earlier
+// ones were handed back.
+RTPN_HD constexpr int drain_first(int s, int nb) { return s > nb ? s - nb : 0; }
+RTPN_HD constexpr unsigned full_parity(int s, int nb) { return (unsigned)(s / nb) & 1u; }
+
 // Producer warp t: issues the copies of type t (and for t = 0 the coupling constants) of every sub-stage
 // of this CTA's sequence into the ring.  One lane issues; everything else is the same for the warp.
 template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH>
@@ -641,9 +652,8 @@ __device__ __forceinline__ void stage_producer(const Args& a, unsigned char* buf
     }
     if (failed && lane == 0) atomicOr(a.status, STATUS_TIMEOUT);
     // before the CTA ends, the copies of the last stages issued must have landed
-    const int first = s > NB ? s - NB : 0;
-    for (int q = first; q < s; ++q)
-        if (q != a.skip_stage) wait_phase(full0 + 8 * (q % NB), (unsigned)((q / NB) & 1), a.wait_limit);
+    for (int q = drain_first(s, NB); q < s; ++q)
+        if (q != a.skip_stage) wait_phase(full0 + 8 * (q % NB), full_parity(q, NB), a.wait_limit);
     // the last CTA to draw its last ticket clears the counters for the next pass
     if (t == 0 && lane == 0) {
         __threadfence();
@@ -1024,7 +1034,7 @@ __device__ __forceinline__ void stage_kernel_body(const Args& a, unsigned char* 
                                                                         scale, al0, be0 * a.inv_h, ga0, prev);
                 // the stage buffer is free once every lane of the warp is past its reads
                 __syncwarp();
-                if (lane == 0) mbar_arrive(empty0 + 8 * b);
+                if (lane == 0 && hands_back(limit)) mbar_arrive(empty0 + 8 * b);
                 if (++b == NB) {
                     b = 0;
                     ph ^= 1u;
