@@ -189,7 +189,10 @@ int rtpn_set_kernel_ex(rtpn_ctx* ctx, int kernel, int tile_x, int tile_y, int ti
 int rtpn_set_media(rtpn_ctx* ctx, const void* sigma_a, const void* sigma_s, const void* q,
                    int dtype, int where);
 
-/* Full state [c][z][y][x] in interface order, converted to the storage precision. */
+/* Full state [c][z][y][x] in interface order, converted to the storage precision.  RTPN_DEVICE here and in the
+ * three calls below: memory of the context's GPU, aligned for its type, is read or written by one kernel;
+ * any other pointer the runtime can copy from or to (another GPU's memory, page-locked host memory, odd
+ * addresses) component by component through cudaMemcpyAsync. */
 int rtpn_set_moments(rtpn_ctx* ctx, const void* u, int dtype, int where);
 /* Copy the full state out ([c][z][y][x], interface order) into a caller-owned buffer. */
 int rtpn_get_moments(rtpn_ctx* ctx, void* u, int dtype, int where);

@@ -119,57 +119,59 @@ void rows_out(rtpn_ctx* ctx, const void* state, void* out, int dtype, bool all) 
     });
 }
 
+// Whether kernels of the context may dereference the caller's device pointer: memory of the context's GPU
+// (or managed), aligned for its type, with that GPU current.  Anything else (another GPU's memory, with
+// or without peer access, page-locked host memory, odd addresses) goes through the runtime's copies.
+bool direct(const rtpn_ctx* ctx, const void* p, int dtype) {
+    cudaPointerAttributes at{};
+    int dev = -1;
+    if (reinterpret_cast<uintptr_t>(p) % dtype_size(dtype) != 0) return false;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (dev != ctx->device) return false;
+    return at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == ctx->device);
+}
+
 int put_component(rtpn_ctx* ctx, int abi, const void* src, int dtype, int where) {
     const long long V = ctx->g.V;
     void* dst = comp_ptr(ctx, ctx->md.internal_of_abi[abi]);
     const size_t bytes = (size_t)V * dtype_size(dtype);
-    if (ctx->padded()) {
-        const void* dev = src;
-        if (where == RTPN_HOST) {
-            CUDA_TRY(ctx, cudaMemcpyAsync(ctx->staging, src, bytes, cudaMemcpyHostToDevice, ctx->stream));
-            dev = ctx->staging;
-        }
-        rows_in(ctx, dev, dtype, dst, false);
-        CHECK_LAUNCH(ctx);
+    const cudaMemcpyKind kind = where == RTPN_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
+    if (same_type(ctx->prec, dtype) && !ctx->padded()) {
+        CUDA_TRY(ctx, cudaMemcpyAsync(dst, src, bytes, kind, ctx->stream));
         return RTPN_OK;
     }
-    if (same_type(ctx->prec, dtype)) {
-        CUDA_TRY(ctx, cudaMemcpyAsync(dst, src, bytes,
-                                      where == RTPN_HOST ? cudaMemcpyHostToDevice
-                                                         : cudaMemcpyDeviceToDevice,
-                                      ctx->stream));
-        return RTPN_OK;
+    const void* dev = src;
+    if (where == RTPN_HOST || !direct(ctx, src, dtype)) {
+        CUDA_TRY(ctx, cudaMemcpyAsync(ctx->staging, src, bytes, kind, ctx->stream));
+        dev = ctx->staging;
     }
-    const void* dev_src = src;
-    if (where == RTPN_HOST) {
-        CUDA_TRY(ctx, cudaMemcpyAsync(ctx->staging, src, bytes, cudaMemcpyHostToDevice, ctx->stream));
-        dev_src = ctx->staging;
-    }
-    return convert_in(ctx, dev_src, dtype, dst, V);
+    if (!ctx->padded()) return convert_in(ctx, dev, dtype, dst, V);
+    rows_in(ctx, dev, dtype, dst, false);
+    CHECK_LAUNCH(ctx);
+    return RTPN_OK;
 }
 
 int take_component(rtpn_ctx* ctx, int abi, void* dst, int dtype, int where) {
     const long long V = ctx->g.V;
     const void* src = comp_ptr(ctx, ctx->md.internal_of_abi[abi]);
     const size_t bytes = (size_t)V * dtype_size(dtype);
+    const cudaMemcpyKind kind = where == RTPN_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
+    if (same_type(ctx->prec, dtype) && !ctx->padded()) {
+        CUDA_TRY(ctx, cudaMemcpyAsync(dst, src, bytes, kind, ctx->stream));
+        return RTPN_OK;
+    }
+    const bool staged = where == RTPN_HOST || !direct(ctx, dst, dtype);
+    void* dev = staged ? ctx->staging : dst;
     if (ctx->padded()) {
-        rows_out(ctx, src, where == RTPN_HOST ? ctx->staging : dst, dtype, false);
+        rows_out(ctx, src, dev, dtype, false);
         CHECK_LAUNCH(ctx);
-        if (where == RTPN_HOST)
-            CUDA_TRY(ctx, cudaMemcpyAsync(dst, ctx->staging, bytes, cudaMemcpyDeviceToHost, ctx->stream));
-        return RTPN_OK;
+    } else if (int rc = convert_out(ctx, src, dev, dtype, V)) {
+        return rc;
     }
-    if (same_type(ctx->prec, dtype)) {
-        CUDA_TRY(ctx, cudaMemcpyAsync(dst, src, bytes,
-                                      where == RTPN_HOST ? cudaMemcpyDeviceToHost
-                                                         : cudaMemcpyDeviceToDevice,
-                                      ctx->stream));
-        return RTPN_OK;
-    }
-    if (where == RTPN_DEVICE) return convert_out(ctx, src, dst, dtype, V);
-    int rc = convert_out(ctx, src, ctx->staging, dtype, V);
-    if (rc) return rc;
-    CUDA_TRY(ctx, cudaMemcpyAsync(dst, ctx->staging, bytes, cudaMemcpyDeviceToHost, ctx->stream));
+    if (staged) CUDA_TRY(ctx, cudaMemcpyAsync(dst, dev, bytes, kind, ctx->stream));
     return RTPN_OK;
 }
 
@@ -643,6 +645,7 @@ int rtpn::create_context(rtpn_ctx** out, int N, int nx, int ny, int nz, double h
         return rc;
     };
     int rc;
+    if (cudaGetDevice(&ctx->device) != cudaSuccess) return bail(fail(ctx, RTPN_ECUDA, "no CUDA device"));
     if (cudaStreamCreateWithFlags(&ctx->own, cudaStreamDefault) != cudaSuccess)
         return bail(fail(ctx, RTPN_ECUDA, "stream create failed"));
     ctx->stream = ctx->own;
@@ -911,13 +914,14 @@ int rtpn_get_component(rtpn_ctx* ctx, int c, void* field, int dtype, int where) 
 int rtpn_set_moments(rtpn_ctx* ctx, const void* u, int dtype, int where) {
     if (!ctx || !u) return RTPN_EINVAL;
     if (!valid_dtype(dtype) || !valid_where(where)) return fail(ctx, RTPN_EINVAL, "bad dtype/where");
-    if (where == RTPN_DEVICE && ctx->padded()) {
+    const bool near = where == RTPN_DEVICE && direct(ctx, u, dtype);
+    if (near && ctx->padded()) {
         rows_in(ctx, u, dtype, ctx->u, true);
         CHECK_LAUNCH(ctx);
         ctx->steps_done = 0;
         return RTPN_OK;
     }
-    if (where == RTPN_DEVICE) {
+    if (near) {
         with_storage(ctx->prec, [&](auto tag) {
             using S = std::remove_pointer_t<decltype(tag)>;
             if (dtype == RTPN_DTYPE_F64)
@@ -942,12 +946,13 @@ int rtpn_set_moments(rtpn_ctx* ctx, const void* u, int dtype, int where) {
 int rtpn_get_moments(rtpn_ctx* ctx, void* u, int dtype, int where) {
     if (!ctx || !u) return RTPN_EINVAL;
     if (!valid_dtype(dtype) || !valid_where(where)) return fail(ctx, RTPN_EINVAL, "bad dtype/where");
-    if (where == RTPN_DEVICE && ctx->padded()) {
+    const bool near = where == RTPN_DEVICE && direct(ctx, u, dtype);
+    if (near && ctx->padded()) {
         rows_out(ctx, ctx->u, u, dtype, true);
         CHECK_LAUNCH(ctx);
         return RTPN_OK;
     }
-    if (where == RTPN_DEVICE) {
+    if (near) {
         with_storage(ctx->prec, [&](auto tag) {
             using S = std::remove_pointer_t<decltype(tag)>;
             if (dtype == RTPN_DTYPE_F64)

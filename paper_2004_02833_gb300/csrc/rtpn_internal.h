@@ -217,6 +217,7 @@ struct rtpn_ctx {
     void* staging = nullptr;         // one plane of FP64 (conversions, media upload)
     double* media = nullptr;         // FP64 sigma_a, sigma_s, q as last set (3 planes)
     cudaStream_t stream = nullptr;   // work stream (user's or own)
+    int device = 0;                  // the GPU the context was created on
     cudaStream_t own = nullptr;      // private stream (capture, default work stream)
     bool media_set = false;
     // row pitch of the state and stride of its components: nx and V, but with rows padded to 16-byte
