@@ -588,28 +588,10 @@ int adjoint_staged(rtpn_ctx* ctx, const double* w_dev, int k, int ckpt, double* 
     return RTPN_OK;
 }
 
-}  // namespace
-
-extern "C" int rtpn_adjoint(rtpn_ctx* ctx, const void* w, int dtype, int where, int k, int ckpt_every,
-                            double* g_sa, double* g_ss, double* g_q, int out_where, double* J) {
-    if (!ctx || !w || !g_sa || !g_ss || !g_q || !J || k < 0 || ckpt_every < 1) return RTPN_EINVAL;
-    if ((dtype != RTPN_DTYPE_F64 && dtype != RTPN_DTYPE_F32) || (where != RTPN_HOST && where != RTPN_DEVICE) ||
-        (out_where != RTPN_HOST && out_where != RTPN_DEVICE))
-        return afail(ctx, RTPN_EINVAL, "adjoint: bad dtype/where");
-    if (ctx->prec == RTPN_BF16) return afail(ctx, RTPN_EUNSUPPORTED, "adjoint: BF16 storage");
-    if (ctx->scat) return afail(ctx, RTPN_EUNSUPPORTED, "adjoint: anisotropic scattering");
-    if (!ctx->media_set || !ctx->media) return afail(ctx, RTPN_ESTATE, "adjoint: media not set");
+// rtpn_adjoint on a state with dense rows
+int adjoint_dense(rtpn_ctx* ctx, const void* w, int dtype, int where, int k, int ckpt_every, double* g_sa, double* g_ss,
+                  double* g_q, int out_where, double* J) {
     const long long V = ctx->g.V;
-    // the adjoint's kernels read dense rows; the selected kernel and its padded rows come back at the end
-    struct DenseRows {
-        rtpn_ctx* c;
-        bool padded;
-        ~DenseRows() {
-            if (padded) use_dense_rows(c, false);
-        }
-    } dense{ctx, ctx->padded()};
-    if (dense.padded)
-        if (int rc = use_dense_rows(ctx, true)) return rc;
     // the weights and outputs as FP64 device arrays
     Buf wd, out;
     if (!wd.alloc((size_t)V * sizeof(double)) || !out.alloc((size_t)3 * V * sizeof(double)))
@@ -638,6 +620,36 @@ extern "C" int rtpn_adjoint(rtpn_ctx* ctx, const void* w, int dtype, int where, 
     cudaError_t e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return afail(ctx, RTPN_ECUDA, cudaGetErrorString(e));
     return RTPN_OK;
+}
+
+}  // namespace
+
+extern "C" int rtpn_adjoint(rtpn_ctx* ctx, const void* w, int dtype, int where, int k, int ckpt_every,
+                            double* g_sa, double* g_ss, double* g_q, int out_where, double* J) {
+    if (!ctx || !w || !g_sa || !g_ss || !g_q || !J || k < 0 || ckpt_every < 1) return RTPN_EINVAL;
+    if ((dtype != RTPN_DTYPE_F64 && dtype != RTPN_DTYPE_F32) || (where != RTPN_HOST && where != RTPN_DEVICE) ||
+        (out_where != RTPN_HOST && out_where != RTPN_DEVICE))
+        return afail(ctx, RTPN_EINVAL, "adjoint: bad dtype/where");
+    if (ctx->prec == RTPN_BF16) return afail(ctx, RTPN_EUNSUPPORTED, "adjoint: BF16 storage");
+    if (ctx->scat) return afail(ctx, RTPN_EUNSUPPORTED, "adjoint: anisotropic scattering");
+    if (!ctx->media_set || !ctx->media) return afail(ctx, RTPN_ESTATE, "adjoint: media not set");
+    // the adjoint's kernels read dense rows; the selected kernel and its padded rows come back at the end,
+    // also after an error, and before the call returns
+    const bool padded = ctx->padded();
+    if (padded)
+        if (int rc = use_dense_rows(ctx, true)) return rc;
+    int rc = adjoint_dense(ctx, w, dtype, where, k, ckpt_every, g_sa, g_ss, g_q, out_where, J);
+    if (padded) {
+        const std::string msg = ctx->err;
+        int back = use_dense_rows(ctx, false);
+        const cudaError_t e = cudaStreamSynchronize(ctx->stream);
+        if (!back && e != cudaSuccess) back = afail(ctx, RTPN_ECUDA, cudaGetErrorString(e));
+        if (rc)
+            ctx->err = msg;
+        else
+            rc = back;
+    }
+    return rc;
 }
 
 extern "C" int rtpn_adjoint_release(rtpn_ctx* ctx) {

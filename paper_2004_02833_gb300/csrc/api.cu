@@ -418,12 +418,15 @@ constexpr int kStageMinN = 15;
 // 0.057 ms, 7 0.079 and 0.077, 9 0.099 and 0.095; 75 0.18 and 1.09 at 61 x 77).
 constexpr int kPadMinNx = 8;
 
-// Row pitch of the state: nx, or nx padded to 16-byte rows.  The state is rearranged in place, a component
+// Row pitch of the state: nx, or nx padded to 16-byte rows.  set_rows rearranges the state in place, a component
 // at a time through the staging plane (its buffer holds the padded state if the context can ever need
 // it); the padding holds zeros.
-int set_rows(rtpn_ctx* ctx, bool padded) {
+int padded_pitch(const rtpn_ctx* ctx) {
+    const int grp = stage_row_group(ctx->prec);
+    return (ctx->g.nx + grp - 1) / grp * grp;
+}
+int set_rows(rtpn_ctx* ctx, int px) {
     const Geom& g = ctx->g;
-    const int grp = stage_row_group(ctx->prec), px = padded ? (g.nx + grp - 1) / grp * grp : g.nx;
     if (px == ctx->px) return RTPN_OK;
     const long long sV = (long long)px * g.ny * g.nz, rows = (long long)g.ny * g.nz;
     drop_graphs(ctx);
@@ -439,9 +442,9 @@ int set_rows(rtpn_ctx* ctx, bool padded) {
             }
         });
     }
-    CHECK_LAUNCH(ctx);
     ctx->px = px;
     ctx->sV = sV;
+    CHECK_LAUNCH(ctx);
     return RTPN_OK;
 }
 
@@ -451,8 +454,12 @@ bool may_pad(const rtpn_ctx* ctx) {
            stage_compiled(ctx->N, ctx->prec);
 }
 
+// The kernel for the context's selection, with what it needs.  Whatever can fail comes first; the kernel, its
+// tile and the rows of the state then change together, so a failure leaves the context as it was.
 int choose_kernel(rtpn_ctx* ctx) {
     int k = ctx->kernel;
+    int tx = ctx->tx, ty = ctx->ty, tz = ctx->tz, depth = ctx->depth;
+    bool from_stage = ctx->tile_from_stage;
     const bool cubic = cubic_cells(ctx->g);
     if (ctx->scat) {
         // per-order factors: the generic kernel's per-target plane table, or the window kernel's
@@ -467,23 +474,22 @@ int choose_kernel(rtpn_ctx* ctx) {
     // kernel takes cubic cells only
     const bool win_ok = window_supported(ctx->N, ctx->prec) && (cubic || window_extended(ctx->N));
     if (k == RTPN_KERNEL_AUTO) {
-        const bool tile_set = (ctx->tx || ctx->ty || ctx->tz) && !ctx->tile_from_stage;
+        const bool tile_set = (tx || ty || tz) && !from_stage;
         // other widths than 16-byte rows: padded, unless the caller asks for a tile (then one of the
         // kernels that take any width)
         const bool pad = may_pad(ctx) && !ctx->dense_rows && !tile_set;
         if (kStageInAuto && (ctx->N >= kStageMinN || !win_ok) &&
             (stage_supported(ctx->N, ctx->prec, ctx->g.nx) || pad) &&
-            (!tile_set || stage_has_tile(ctx->N, ctx->tx, ctx->ty, ctx->tz, ctx->depth, ctx->prec)))
+            (!tile_set || stage_has_tile(ctx->N, tx, ty, tz, depth, ctx->prec)))
             k = RTPN_KERNEL_STAGE;
         else
             k = win_ok ? RTPN_KERNEL_WINDOW : RTPN_KERNEL_GENERIC;
     }
     // a tile the staged kernel chose is no request for another kernel (its shape need not even be a
     // valid window tile): the other kernels start from their defaults
-    if (k != RTPN_KERNEL_STAGE && ctx->tile_from_stage) {
-        ctx->tx = ctx->ty = ctx->tz = 0;
-        ctx->depth = 0;
-        ctx->tile_from_stage = false;
+    if (k != RTPN_KERNEL_STAGE && from_stage) {
+        tx = ty = tz = depth = 0;
+        from_stage = false;
     }
     if (!cubic && k == RTPN_KERNEL_FUSED)
         return fail(ctx, RTPN_EUNSUPPORTED, "the fused kernel takes cubic cells only");
@@ -497,25 +503,23 @@ int choose_kernel(rtpn_ctx* ctx) {
         if (!stage_supported(ctx->N, ctx->prec, ctx->g.nx))
             return fail(ctx, RTPN_EUNSUPPORTED,
                         "staged kernel not compiled for this N/precision or nx*elem not 16-byte rows");
-        if (!stage_has_tile(ctx->N, ctx->tx, ctx->ty, ctx->tz, ctx->depth, ctx->prec))
+        if (!stage_has_tile(ctx->N, tx, ty, tz, depth, ctx->prec))
             return fail(ctx, RTPN_EUNSUPPORTED, "no staged kernel compiled for this tile / stage depth");
     }
-    if (int rc = set_rows(ctx, pad)) return rc;
-    if (k == RTPN_KERNEL_STAGE) {
-        int rc = stage_prepare(ctx, ctx->tx, ctx->ty, ctx->tz, ctx->depth);
-        if (rc) return fail(ctx, RTPN_ECUDA, std::string("staged kernel set-up: ") +
-                                                 cudaGetErrorString((cudaError_t)rc));
-    }
+    auto unprepared = [&](const char* what, int rc) {
+        cudaGetLastError();  // reported here; the next launch check is not to see it
+        return fail(ctx, RTPN_ECUDA, std::string(what) + ": " + cudaGetErrorString((cudaError_t)rc));
+    };
+    const int px = pad ? padded_pitch(ctx) : ctx->g.nx;
     if (k == RTPN_KERNEL_GENERIC && generic_compiled(ctx)) {
         int rc = window64_prepare(ctx->md);
-        if (rc) return fail(ctx, RTPN_ECUDA, std::string("generic kernel constants: ") + cudaGetErrorString((cudaError_t)rc));
+        if (rc) return unprepared("generic kernel constants", rc);
     }
     if (k == RTPN_KERNEL_WINDOW) {
         if (!window_supported(ctx->N, ctx->prec))
             return fail(ctx, RTPN_EUNSUPPORTED, "window kernel not compiled for this N/precision");
         int rc = window_prepare(ctx->md, ctx->g.h, ctx->prec);
-        if (rc) return fail(ctx, RTPN_ECUDA, std::string("window constants: ") +
-                                                 cudaGetErrorString((cudaError_t)rc));
+        if (rc) return unprepared("window constants", rc);
     }
     if (k == RTPN_KERNEL_FUSED) {
         // a batch keeps each instance's state pointer in its launch items; the fused kernel moves it
@@ -525,8 +529,7 @@ int choose_kernel(rtpn_ctx* ctx) {
             return fail(ctx, RTPN_EUNSUPPORTED, "fused kernel not compiled for this N/precision");
         int rc = fused_prepare(ctx->md, ctx->prec);
         if (!rc) rc = window_prepare(ctx->md, ctx->g.h, ctx->prec);
-        if (rc) return fail(ctx, RTPN_ECUDA, std::string("fused kernel constants: ") +
-                                                 cudaGetErrorString((cudaError_t)rc));
+        if (rc) return unprepared("fused kernel constants", rc);
         if (!ctx->u_alt) {
             cudaError_t e = cudaMalloc(&ctx->u_alt, (size_t)ctx->md.nc * ctx->g.V * ctx->elem);
             if (e != cudaSuccess) {
@@ -536,9 +539,19 @@ int choose_kernel(rtpn_ctx* ctx) {
             }
         }
     }
+    if (k == RTPN_KERNEL_STAGE) {
+        int rc = stage_prepare(ctx, tx, ty, tz, depth, px);  // sets the tile
+        if (rc) return unprepared("staged kernel set-up", rc);
+    } else {
+        ctx->tx = tx;
+        ctx->ty = ty;
+        ctx->tz = tz;
+        ctx->depth = depth;
+        ctx->tile_from_stage = from_stage;
+    }
     if (k != ctx->active_kernel) drop_graphs(ctx);
     ctx->active_kernel = k;
-    return RTPN_OK;
+    return set_rows(ctx, px);
 }
 
 }  // namespace
@@ -608,7 +621,9 @@ int rtpn_create(rtpn_ctx** out, int N, int nx, int ny, int nz, double h, int bc,
 int rtpn::use_dense_rows(rtpn_ctx* ctx, bool on) {
     if (ctx->dense_rows == on) return RTPN_OK;
     ctx->dense_rows = on;
-    return choose_kernel(ctx);
+    const int rc = choose_kernel(ctx);
+    if (rc) ctx->dense_rows = !on;
+    return rc;
 }
 
 int rtpn::create_context(rtpn_ctx** out, int N, int nx, int ny, int nz, double h, int bc, int precision, double dt,
@@ -830,16 +845,13 @@ int rtpn_set_kernel_ex(rtpn_ctx* ctx, int kernel, int tile_x, int tile_y, int ti
     ctx->tile_from_stage = false;
     ctx->depth = kernel == RTPN_KERNEL_STAGE || kernel == RTPN_KERNEL_AUTO ? depth : 0;
     int rc = choose_kernel(ctx);
-    if (rc) {
-        const std::string msg = ctx->err;
+    if (rc) {  // nothing has changed but the selection
         ctx->kernel = old;
         ctx->tx = ox;
         ctx->ty = oy;
         ctx->tz = oz;
         ctx->depth = oc;
         ctx->tile_from_stage = ofs;
-        choose_kernel(ctx);
-        ctx->err = msg;
     }
     return rc;
 }

@@ -147,32 +147,27 @@ bool stage_has_tile(int N, int tx, int ty, int tz, int depth, int precision) {
     return stg::find(N, tx, ty, tz, depth, precision) != nullptr;
 }
 
-int stage_prepare(rtpn_ctx* ctx, int tx, int ty, int tz, int depth) {
+int stage_prepare(rtpn_ctx* ctx, int tx, int ty, int tz, int depth, int px) {
     const stg::Variant* v = stg::find(ctx->N, tx, ty, tz, depth, ctx->prec);
     if (!v) return (int)cudaErrorNotSupported;
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, dev);
     if (tx == 0)
-        if (const stg::Variant* w = stg::best_variant(ctx->N, ctx->prec, depth, ctx->g, ctx->px, ctx->sms)) v = w;
+        if (const stg::Variant* w = stg::best_variant(ctx->N, ctx->prec, depth, ctx->g, px, ctx->sms)) v = w;
     const int N = ctx->N;
     // the tensor maps live in device global memory (64-byte aligned) and the kernel reads them from
     // there: tile planes / z halo plane, y halo row and x halo group, each for every box length
     const int nmap = stg::nmaps_of(*v, ctx->prec);
     if (nmap <= 0 || nmap > stg::kMaxSlots) return (int)cudaErrorInvalidValue;
     std::vector<CUtensorMap> maps((size_t)stg::MAP_KINDS * nmap);
-    if (!stg::make_maps(maps.data(), ctx->u, ctx->prec, ctx->g, ctx->px, ctx->sV, ctx->md.nc, *v, stg::MAP_KINDS))
+    if (!stg::make_maps(maps.data(), ctx->u, ctx->prec, ctx->g, px, (long long)px * ctx->g.ny * ctx->g.nz, ctx->md.nc, *v,
+                        stg::MAP_KINDS))
         return (int)cudaErrorInvalidValue;
     if (!ctx->stage_maps_dev) {
         // the forward's maps, then room for the adjoint's (all kinds over w, plane maps over lam)
         cudaError_t err = cudaMalloc(&ctx->stage_maps_dev, stage_maps_capacity * sizeof(CUtensorMap));
         if (err != cudaSuccess) return (int)err;
-    }
-    {
-        cudaError_t err = cudaMemcpy(ctx->stage_maps_dev, maps.data(), maps.size() * sizeof(CUtensorMap),
-                                     cudaMemcpyHostToDevice);
-        if (err != cudaSuccess) return (int)err;
-        ctx->stage_adj_lam = ctx->stage_adj_w = nullptr;  // the adjoint's maps follow the tile
     }
     if (!ctx->stage_mem) {
         std::vector<int> col;
@@ -180,16 +175,23 @@ int stage_prepare(rtpn_ctx* ctx, int tx, int ty, int tz, int depth) {
         if (!stg::coupling_tables(ctx->md, ctx->g.h / ctx->g.hy, ctx->g.h / ctx->g.hz, tab, &col))
             return (int)cudaErrorInvalidValue;
         const size_t b0 = tab[0].size() * 4, b1 = tab[1].size() * 4, b2 = col.size() * 4;
-        cudaError_t err = cudaMalloc(&ctx->stage_mem, b0 + b1 + b2);
-        if (err != cudaSuccess) return (int)err;
-        char* m = (char*)ctx->stage_mem;
-        cudaMemcpy(m, tab[0].data(), b0, cudaMemcpyHostToDevice);
-        cudaMemcpy(m + b0, tab[1].data(), b1, cudaMemcpyHostToDevice);
-        err = cudaMemcpy(m + b0 + b1, col.data(), b2, cudaMemcpyHostToDevice);
-        if (err != cudaSuccess) return (int)err;
+        char* m = nullptr;
+        cudaError_t err = cudaMalloc(&m, b0 + b1 + b2);
+        if (err == cudaSuccess) err = cudaMemcpy(m, tab[0].data(), b0, cudaMemcpyHostToDevice);
+        if (err == cudaSuccess) err = cudaMemcpy(m + b0, tab[1].data(), b1, cudaMemcpyHostToDevice);
+        if (err == cudaSuccess) err = cudaMemcpy(m + b0 + b1, col.data(), b2, cudaMemcpyHostToDevice);
+        if (err != cudaSuccess) {
+            if (m) cudaFree(m);
+            return (int)err;
+        }
+        ctx->stage_mem = m;
         ctx->stage_tab_bytes[0] = b0;
         ctx->stage_tab_bytes[1] = b1;
     }
+    // last, because the active kernel may be running on the maps in place
+    cudaError_t err = cudaMemcpy(ctx->stage_maps_dev, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice);
+    if (err != cudaSuccess) return (int)err;
+    ctx->stage_adj_lam = ctx->stage_adj_w = nullptr;  // the adjoint's maps follow the tile
     ctx->stage_variant = (int)(v - stg::kVariants);
     ctx->tx = v->tx;
     ctx->ty = v->ty;

@@ -171,7 +171,7 @@ bool stage_supported(int N, int precision, int nx);
 bool stage_has_tile(int N, int tx, int ty, int tz, int depth, int precision);
 // builds the tensor maps (tile 0,0,0 = default; depth 0 = any) and the coupling tables;
 // returns cudaError_t
-int stage_prepare(rtpn_ctx* ctx, int tx, int ty, int tz, int depth);
+int stage_prepare(rtpn_ctx* ctx, int tx, int ty, int tz, int depth, int px);
 // compiled (tx, ty, tz, depth) of order N that fit for this precision into tiles[4*i..];
 // returns the count
 int stage_variants_of(int N, int precision, int* tiles, int max);

@@ -1,0 +1,94 @@
+"""Kernel selection, row pitch and allocation against failures of the calls they make, with a stand-in for the
+CUDA runtime (no GPU): whatever fails, the kernel in use and the rows of the state go together, and the
+error is reported."""
+import pytest
+
+import fake_runtime
+
+
+@pytest.fixture(scope="module")
+def so(tmp_path_factory, rtpn_lib):
+    return fake_runtime.build(tmp_path_factory.mktemp("fake"))
+
+
+COMMON = """
+shape = (3, 4, 75)
+V = 3 * 4 * 75
+dense, padded = 256 * V * 4, 256 * 3 * 4 * 76 * 4
+def layout(ctx):
+    i = ctx.info()
+    return i.kernel, i.state_bytes
+def fits(ctx):
+    return layout(ctx) in ((1, dense), (2, dense), (3, padded))
+def context(media=True):
+    ctx = rtpn.Context(15, shape, 0.1)
+    assert layout(ctx) == (3, padded)
+    if media:
+        m = np.full(shape, 0.5)
+        ctx.set_media(m, m, m)
+    log()
+    return ctx
+"""
+
+
+def test_a_failed_selection_leaves_kernel_and_rows(so):
+    fake_runtime.run(so, COMMON + """
+ctx = context()
+tile = tuple(ctx.info().tile)
+ctx.set_kernel("window", (32, 4, 1))
+for api, after in (("cudaMemcpy", 0),):
+    fail(api, after, 719)
+    log()
+    assert code(ctx.set_kernel, "auto") == rtpn.ECUDA
+    assert layout(ctx) == (2, dense) and tuple(ctx.info().tile) == (32, 4, 1)
+    assert kernels(log(), "k_rows") == 0  # the state was not touched
+ctx.set_kernel("auto")
+assert layout(ctx) == (3, padded) and tuple(ctx.info().tile) == tile
+# from the staged kernel to one that cannot be had: the staged kernel and its rows stay
+log()
+assert code(ctx.set_kernel, "fused") == rtpn.EUNSUPPORTED
+assert layout(ctx) == (3, padded) and tuple(ctx.info().tile) == tile
+assert kernels(log(), "k_rows") == 0
+""")
+
+
+def test_set_up_that_fails_for_want_of_memory(so):
+    fake_runtime.run(so, COMMON + """
+ctx = context()
+ctx.set_kernel("window")
+ctx.set_spacing(0.1, 0.1, 0.1)  # drops the staged kernel's tables
+fail("cudaMalloc", 0, 2)
+log()
+assert code(ctx.set_kernel, "auto") != rtpn.OK
+assert layout(ctx) == (2, dense)
+assert kernels(log(), "k_rows") == 0
+ctx.set_kernel("auto")
+assert layout(ctx) == (3, padded)
+""")
+
+
+def test_adjoint_on_padded_rows_returns_what_its_way_back_met(so):
+    fake_runtime.run(so, COMMON + """
+ctx = context()
+w = np.ones(shape)
+ctx.adjoint(w, 2, ckpt_every=2)
+assert layout(ctx) == (3, padded)
+lines = log()
+# the way back to padded rows is queued before the last wait, so that its errors are the call's
+rows = max(i for i, l in enumerate(lines) if l.startswith("K ") and "k_rows" in l)
+assert rows < max(i for i, l in enumerate(lines) if l == "S")
+copies = sum(l.startswith("C cudaMemcpy ") for l in lines)
+assert copies > 0
+# the last of them sets up the staged kernel again
+fail("cudaMemcpy", copies - 1, 719)
+assert code(ctx.adjoint, w, 2, 2) == rtpn.ECUDA
+assert fits(ctx), layout(ctx)
+ctx.set_kernel("auto")
+ctx.step(1)
+assert fits(ctx)
+# an error inside: reported as itself, with the rows padded again
+ctx = context()
+fail("cudaMalloc", 2, 2)
+assert code(ctx.adjoint, w, 2, 2) == rtpn.ENOMEM
+assert layout(ctx) == (3, padded)
+""")
