@@ -257,7 +257,9 @@ RTPN_CONV(__nv_bfloat16, float)
 // out[perm[c]] = in[c] (true), V values each.  Bound by memory; one launch for all components, because a
 // copy per component is bound by the host's issue of them (P15 64^3: 256 copies took 1.0 ms of host
 // time for 0.08 ms of traffic).  Four values per access where V and the pointers allow 16-byte rows,
-// kIoGroups accesses in flight per thread.
+// kIoGroups accesses in flight per thread.  The kernel may start while the one before it still writes `in`
+// (launch_pdl), so `in` is read by ordinary loads: neither __ldg nor const __restrict__, which promise
+// that nothing writes it while the kernel runs.
 constexpr int kIoThreads = 256, kIoGroups = 4;
 
 template <typename T, int W>
@@ -266,8 +268,8 @@ struct alignas(sizeof(T) * W > 16 ? 16 : sizeof(T) * W) IoVec {
 };
 
 template <typename A, typename B, int W, bool IN_ORDER>
-__global__ void __launch_bounds__(kIoThreads) k_reorder(const A* __restrict__ in, B* __restrict__ out,
-                                                        const int* __restrict__ perm, long long V) {
+__global__ void __launch_bounds__(kIoThreads) k_reorder(const A* in, B* out, const int* __restrict__ perm,
+                                                        long long V) {
     pdl_trigger();
     pdl_wait();
     const int c = blockIdx.y, p = perm[c];

@@ -57,11 +57,12 @@ struct HostTable {
     int a0 = 0, na = 0;
 };
 
-// For the short kernels of small problems (window passes, moments in and out: a P3 32^3 step and its state
-// out 10.3 -> 9.3 us): launch with programmatic stream serialisation: the kernel may be set up while the
-// one before it on the stream drains, and waits for its end (with everything it wrote) in pdl_wait, which every thread
-// calls before it touches anything an earlier kernel could have written or could still read.  The staged
-// and generic passes gain nothing from it (P15 96^3 within 0.3 %, the P15 64^3 adjoint 2 % slower).
+// For the moments in and out: launch with programmatic stream serialisation: the kernel may be set up while
+// the one before it on the stream drains, and waits for its end (with everything it wrote) in pdl_wait, which every
+// thread calls before it touches anything an earlier kernel could have written or could still read.  Such a
+// kernel runs beside the writes of the one before, so it loads what that may write by ordinary loads, not
+// by __ldg or through const __restrict__, which promise memory that nothing writes while the kernel runs.
+// (A P3 32^3 step and its state out 10.3 -> 9.8 us; the step kernels are launched in stream order.)
 template <typename... K, typename... A>
 cudaError_t launch_pdl(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
     cudaLaunchAttribute at{};

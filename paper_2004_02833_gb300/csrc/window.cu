@@ -26,10 +26,13 @@ static_assert(kSources * 10 * 4 <= 64 * 1024 - 1024, "coefficient table exceeds 
 // coefficient of source j (class 1 - kA, local index) for relation k: M_d[a][b] * dir
 __constant__ float c_coef[kSources * 10];
 
+// Launched in stream order, with no early start: the body reads the state and the factors by the read-only
+// path, which holds only while no other kernel writes them.  (An early start with ordinary loads is slower on
+// all but the smallest grids, because the compiler then keeps loads behind the stores to the same state: GB300,
+// FP32, ten steps, P7 128^3 4.05 ms against 3.50, ragged 67 x 90 x 101 1.45 against 1.22, per-order factors 96^3 2.72 against
+// 1.85; a P3 32^3 step with the state out 9.3 us against 9.8.)
 template <typename S, bool SCALED, bool ANISO>
 __global__ void __launch_bounds__(256) k_window(Args a) {
-    pdl_trigger();
-    pdl_wait();
     if constexpr (prefetches(kN)) prefetch_tile<kN, kA, S, ANISO>(a, blockIdx.x, threadIdx.x, blockDim.x);
     int x, y, z;
     if (!cell_of(a, blockIdx.x, threadIdx.x, &x, &y, &z)) return;
@@ -40,8 +43,11 @@ template <bool SCALED, bool ANISO>
 int launch_form(int precision, const Args& a, cudaStream_t st) {
     const int threads = a.tx * a.ty * a.tz;
     const unsigned blocks = (unsigned)a.ntx * a.nty * a.ntz;
-    if (precision == RTPN_BF16) return (int)launch_pdl(k_window<__nv_bfloat16, SCALED, ANISO>, blocks, threads, 0, st, a);
-    return (int)launch_pdl(k_window<float, SCALED, ANISO>, blocks, threads, 0, st, a);
+    if (precision == RTPN_BF16)
+        k_window<__nv_bfloat16, SCALED, ANISO><<<blocks, threads, 0, st>>>(a);
+    else
+        k_window<float, SCALED, ANISO><<<blocks, threads, 0, st>>>(a);
+    return (int)cudaGetLastError();
 }
 
 // the form a launch needs; the non-cubic and anisotropic forms exist up to kExtendedMaxN (a
