@@ -475,9 +475,10 @@ int choose_kernel(rtpn_ctx* ctx) {
     const bool win_ok = window_supported(ctx->N, ctx->prec) && (cubic || window_extended(ctx->N));
     if (k == RTPN_KERNEL_AUTO) {
         const bool tile_set = (tx || ty || tz) && !from_stage;
-        // other widths than 16-byte rows: padded, unless the caller asks for a tile (then one of the
-        // kernels that take any width)
-        const bool pad = may_pad(ctx) && !ctx->dense_rows && !tile_set;
+        // other widths than 16-byte rows: padded, unless the caller asks for a tile, or for a stage depth that
+        // no variant has (then one of the kernels that take any width)
+        const bool pad = may_pad(ctx) && !ctx->dense_rows && !tile_set &&
+                         stage_has_tile(ctx->N, tx, ty, tz, depth, ctx->prec);
         if (kStageInAuto && (ctx->N >= kStageMinN || !win_ok) &&
             (stage_supported(ctx->N, ctx->prec, ctx->g.nx) || pad) &&
             (!tile_set || stage_has_tile(ctx->N, tx, ty, tz, depth, ctx->prec)))

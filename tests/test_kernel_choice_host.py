@@ -92,3 +92,23 @@ fail("cudaMalloc", 2, 2)
 assert code(ctx.adjoint, w, 2, 2) == rtpn.ENOMEM
 assert layout(ctx) == (3, padded)
 """)
+
+
+def test_auto_with_a_depth_on_rows_that_are_no_16_byte_groups(so):
+    # a depth that a variant has runs staged; one that none has leaves the kernels that take any width
+    fake_runtime.run(so, """
+for precision in ("fp32", "bf16"):
+    for N, any_width in ((15, 2), (19, 1), (29, 1), (39, 2)):
+        ctx = rtpn.Context(N, (2, 3, 75), 0.1, "periodic", precision)
+        assert ctx.info().kernel == 3
+        for depth in range(9):
+            assert code(ctx.set_kernel, "auto", (0, 0, 0), depth) == rtpn.OK, (N, depth)
+            i = ctx.info()
+            assert i.kernel in (3, any_width) and (i.kernel != 3 or depth in (0, i.depth)), (N, depth)
+            dense = (N + 1) ** 2 * 2 * 3 * 75 * (4 if precision == "fp32" else 2)
+            assert (i.state_bytes != dense) == (i.kernel == 3)
+        # on 16-byte rows such a depth is refused, as by name, and the selection stays
+        even = rtpn.Context(N, (2, 3, 72), 0.1, "periodic", precision)
+        assert code(even.set_kernel, "auto", (0, 0, 0), 8) == rtpn.EUNSUPPORTED
+        assert even.info().kernel == 3
+""")
