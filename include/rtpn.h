@@ -118,7 +118,10 @@ int rtpn_coupling_dense(int N, int axis, double* out);
 /*
  * Create a context for order N on nx*ny*nz cells of size h, boundary bc, storage precision, time
  * step dt (dt <= 0 selects 0.3 h).  Allocates the state (zeroed) and the factor tables on the
- * current CUDA device and uses the legacy default stream until rtpn_set_stream.
+ * current CUDA device and uses the legacy default stream until rtpn_set_stream.  Where RTPN_KERNEL_AUTO may
+ * pad the state's rows (see rtpn_set_kernel) the state is allocated with room for it, which stays when
+ * another kernel is selected; if that does not fit the device, the state is created dense and AUTO does
+ * not pad.
  * Errors: RTPN_EINVAL (N < 0 or N > 63, dims < 1, h <= 0, bad bc/precision, out == NULL),
  * RTPN_ECFL (dt >= h/3, Section 2.1), RTPN_ENOMEM, RTPN_ECUDA.  *out is NULL on failure.
  */

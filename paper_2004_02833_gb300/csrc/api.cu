@@ -450,7 +450,7 @@ int set_rows(rtpn_ctx* ctx, int px) {
 
 // whether the automatic choice may pad the rows for the staged kernel
 bool may_pad(const rtpn_ctx* ctx) {
-    return kStageInAuto && ctx->N >= kStageMinN && !ctx->batch_member && ctx->g.nx >= kPadMinNx &&
+    return kStageInAuto && ctx->N >= kStageMinN && !ctx->batch_member && !ctx->no_padding && ctx->g.nx >= kPadMinNx &&
            stage_compiled(ctx->N, ctx->prec);
 }
 
@@ -509,7 +509,8 @@ int choose_kernel(rtpn_ctx* ctx) {
     }
     auto unprepared = [&](const char* what, int rc) {
         cudaGetLastError();  // reported here; the next launch check is not to see it
-        return fail(ctx, RTPN_ECUDA, std::string(what) + ": " + cudaGetErrorString((cudaError_t)rc));
+        return fail(ctx, rc == (int)cudaErrorMemoryAllocation ? RTPN_ENOMEM : RTPN_ECUDA,
+                    std::string(what) + ": " + cudaGetErrorString((cudaError_t)rc));
     };
     const int px = pad ? padded_pitch(ctx) : ctx->g.nx;
     if (k == RTPN_KERNEL_GENERIC && generic_compiled(ctx)) {
@@ -627,8 +628,10 @@ int rtpn::use_dense_rows(rtpn_ctx* ctx, bool on) {
     return rc;
 }
 
-int rtpn::create_context(rtpn_ctx** out, int N, int nx, int ny, int nz, double h, int bc, int precision, double dt,
-                         bool batch_member) {
+namespace {
+// create_context with or without room for padded rows
+int create_with(rtpn_ctx** out, int N, int nx, int ny, int nz, double h, int bc, int precision, double dt, bool batch_member,
+                bool pad, bool* padded) {
     if (!out) return fail(nullptr, RTPN_EINVAL, "out is NULL");
     *out = nullptr;
     if (N < 0 || N > 63) return fail(nullptr, RTPN_EINVAL, "N must be in 0..63");
@@ -650,6 +653,7 @@ int rtpn::create_context(rtpn_ctx** out, int N, int nx, int ny, int nz, double h
     ctx->prec = precision;
     ctx->dt = dt;
     ctx->batch_member = batch_member;
+    ctx->no_padding = !pad;
     ctx->px = nx;
     ctx->sV = V;
     ctx->elem = precision == RTPN_FP64 ? 8 : (precision == RTPN_FP32 ? 4 : 2);
@@ -666,8 +670,9 @@ int rtpn::create_context(rtpn_ctx** out, int N, int nx, int ny, int nz, double h
         return bail(fail(ctx, RTPN_ECUDA, "stream create failed"));
     ctx->stream = ctx->own;
     // room for padded rows where the automatic choice may take them
-    const int grp = may_pad(ctx) ? stage_row_group(precision) : 1;
-    const size_t state_room = (size_t)ctx->md.nc * ((nx + grp - 1) / grp * grp) * ny * nz * ctx->elem;
+    const int room_px = may_pad(ctx) ? padded_pitch(ctx) : nx;
+    *padded = room_px != nx;
+    const size_t state_room = (size_t)ctx->md.nc * room_px * ny * nz * ctx->elem;
     cudaError_t e = cudaMalloc(&ctx->u, state_room);
     if (e != cudaSuccess) return bail(fail(ctx, RTPN_ENOMEM, "state allocation failed"));
     ctx->u_home = ctx->u;
@@ -692,13 +697,25 @@ int rtpn::create_context(rtpn_ctx** out, int N, int nx, int ny, int nz, double h
     e = cudaMemsetAsync(ctx->u, 0, state_room, ctx->stream);
     if (e != cudaSuccess) return bail(fail(ctx, RTPN_ECUDA, cudaGetErrorString(e)));
     // a state of zeros needs no rearranging: padded from the start where the choice below pads it
-    ctx->px = (nx + grp - 1) / grp * grp;
-    ctx->sV = (long long)ctx->px * ny * nz;
+    ctx->px = room_px;
+    ctx->sV = (long long)room_px * ny * nz;
     if ((rc = choose_kernel(ctx))) return bail(rc);
     e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return bail(fail(ctx, RTPN_ECUDA, cudaGetErrorString(e)));
     *out = ctx;
     return RTPN_OK;
+}
+}  // namespace
+
+int rtpn::create_context(rtpn_ctx** out, int N, int nx, int ny, int nz, double h, int bc, int precision, double dt,
+                         bool batch_member) {
+    bool padded = false;
+    int rc = create_with(out, N, nx, ny, nz, h, bc, precision, dt, batch_member, true, &padded);
+    if (rc == RTPN_ENOMEM && padded) {  // the padding must not be what keeps a problem off the device
+        cudaGetLastError();
+        rc = create_with(out, N, nx, ny, nz, h, bc, precision, dt, batch_member, false, &padded);
+    }
+    return rc;
 }
 
 extern "C" {

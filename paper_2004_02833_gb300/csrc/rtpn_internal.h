@@ -226,6 +226,7 @@ struct rtpn_ctx {
     int px = 0;
     long long sV = 0;
     bool dense_rows = false;         // no padded rows now (use_dense_rows)
+    bool no_padding = false;         // created without room for padded rows
     bool batch_member = false;       // created by rtpn_batch_create (its kernels take cubic cells)
     double* scat = nullptr;          // f_l (l = 0..N) of anisotropic scattering on the device, or null
     int fac_planes = rtpn::FAC_PLANES;  // factor planes allocated

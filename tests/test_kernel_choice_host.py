@@ -112,3 +112,36 @@ for precision in ("fp32", "bf16"):
         assert code(even.set_kernel, "auto", (0, 0, 0), 8) == rtpn.EUNSUPPORTED
         assert even.info().kernel == 3
 """)
+
+
+def test_padding_is_not_what_keeps_a_problem_off_the_device(so):
+    # nx = 9 in BF16 pads to 16: the state alone needs 16/9 of the dense one
+    fake_runtime.run(so, """
+shape = (40, 40, 9)
+def used(kernel):
+    ctx = rtpn.Context(15, shape, 0.1, "periodic", "bf16")
+    if kernel:
+        ctx.set_kernel(kernel)
+    b = fake.fake_used(), ctx.info().state_bytes, ctx.info().kernel
+    ctx.close()
+    return b
+room, padded, kernel = used(None)
+dense = 256 * 40 * 40 * 9 * 2
+assert kernel == 3 and padded == dense * 16 // 9 and fake.fake_used() == 0
+least = room - (padded - dense)  # what the dense form of the same context takes (the tables included)
+for limit in range(least, room, (padded - dense) // 7):
+    fake.fake_limit(limit)
+    ctx = rtpn.Context(15, shape, 0.1, "periodic", "bf16")
+    assert ctx.info().kernel == 2 and ctx.info().state_bytes == dense
+    m = np.full(shape, 0.5)
+    ctx.set_kernel("generic")
+    ctx.set_kernel("auto")
+    assert ctx.info().kernel == 2 and ctx.info().state_bytes == dense
+    ctx.close()
+    assert fake.fake_used() == 0
+fake.fake_limit(room)
+assert used(None) == (room, padded, 3)
+fake.fake_limit(dense)
+assert code(rtpn.Context, 15, shape, 0.1, "periodic", "bf16") == rtpn.ENOMEM
+assert fake.fake_used() == 0
+""")
