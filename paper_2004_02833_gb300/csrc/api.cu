@@ -620,11 +620,38 @@ int rtpn_create(rtpn_ctx** out, int N, int nx, int ny, int nz, double h, int bc,
 
 }  // extern "C"
 
+int rtpn::use_staged_tile(rtpn_ctx* ctx, int tx, int ty, int tz, int depth) {
+    if (!ctx->padded() || !stage_has_tile(ctx->N, tx, ty, tz, depth, ctx->prec))
+        return fail(ctx, RTPN_EUNSUPPORTED, "no staged kernel compiled for this tile / stage depth");
+    const int ox = ctx->tx, oy = ctx->ty, oz = ctx->tz, oc = ctx->depth;
+    drop_graphs(ctx);
+    ctx->tx = tx;
+    ctx->ty = ty;
+    ctx->tz = tz;
+    ctx->depth = depth;
+    const int rc = choose_kernel(ctx);  // the selection is AUTO and tile_from_stage stays set
+    if (rc) {
+        ctx->tx = ox;
+        ctx->ty = oy;
+        ctx->tz = oz;
+        ctx->depth = oc;
+    }
+    return rc;
+}
+
 int rtpn::use_dense_rows(rtpn_ctx* ctx, bool on) {
     if (ctx->dense_rows == on) return RTPN_OK;
+    const int tile[4] = {ctx->tx, ctx->ty, ctx->tz, ctx->depth};
     ctx->dense_rows = on;
-    const int rc = choose_kernel(ctx);
-    if (rc) ctx->dense_rows = !on;
+    int rc = choose_kernel(ctx);
+    if (rc) {
+        ctx->dense_rows = !on;
+        return rc;
+    }
+    if (on)
+        std::copy(tile, tile + 4, ctx->padded_tile);
+    else if (ctx->padded())
+        rc = use_staged_tile(ctx, ctx->padded_tile[0], ctx->padded_tile[1], ctx->padded_tile[2], ctx->padded_tile[3]);
     return rc;
 }
 

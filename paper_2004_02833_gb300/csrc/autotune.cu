@@ -127,13 +127,16 @@ int rtpn_autotune(rtpn_ctx* ctx, int reps, int tile[3], double* ms_per_step) {
             best_ms = it->second.second;
         }
     }
+    // on padded rows the staged kernel is the automatic choice's and stays so, with another tile
+    const bool padded = ctx->padded();
+    auto use = [&](const Tile& t) {
+        return padded ? rtpn::use_staged_tile(ctx, t.x, t.y, t.z, t.c) : rtpn_set_kernel_ex(ctx, kernel, t.x, t.y, t.z, t.c);
+    };
     std::vector<Tile> cands;
     if (kernel == RTPN_KERNEL_STAGE) {
         int v[4 * 64];
         const int n = rtpn::stage_variants_of(ctx->N, ctx->prec, v, 64);
-        // padded rows belong to the automatic choice: its tile is timed, none is set by name
-        for (int i = 0; i < n && !ctx->padded(); ++i) cands.push_back({v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]});
-        if (ctx->padded()) cands.push_back(best);
+        for (int i = 0; i < n; ++i) cands.push_back({v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]});
     } else {
         for (const Tile& t : kCandidates) cands.push_back(t);
     }
@@ -146,10 +149,9 @@ int rtpn_autotune(rtpn_ctx* ctx, int reps, int tile[3], double* ms_per_step) {
             return RTPN_ENOMEM;
         }
         cudaMemcpyAsync(snap, ctx->u, bytes, cudaMemcpyDeviceToDevice, ctx->stream);
-        const int otx = ctx->tx, oty = ctx->ty, otz = ctx->tz, oc = ctx->depth;
+        const Tile old{ctx->tx, ctx->ty, ctx->tz, ctx->depth};
         int rc = sweep(
-            ctx->stream, reps, cands,
-            [&](Tile t) { return ctx->padded() ? RTPN_OK : rtpn_set_kernel_ex(ctx, kernel, t.x, t.y, t.z, t.c); },
+            ctx->stream, reps, cands, use,
             [&](cudaStream_t) {
                 int r = rtpn_substep(ctx, 0, 0);
                 return r ? r : rtpn_substep(ctx, 1, 0);
@@ -159,14 +161,14 @@ int rtpn_autotune(rtpn_ctx* ctx, int reps, int tile[3], double* ms_per_step) {
         cudaStreamSynchronize(ctx->stream);
         cudaFree(snap);
         if (rc) {
-            if (!ctx->padded()) rtpn_set_kernel_ex(ctx, kernel, otx, oty, otz, oc);
+            use(old);
             return rc;
         }
         std::lock_guard<std::mutex> lock(g_mu);
         g_cache[key] = {best, best_ms};
         store_file(key, best, best_ms);
     }
-    int rc = ctx->padded() ? RTPN_OK : rtpn_set_kernel_ex(ctx, kernel, best.x, best.y, best.z, best.c);
+    int rc = use(best);
     if (rc) return rc;
     if (tile) {
         tile[0] = best.x;

@@ -158,8 +158,11 @@ int launch_fused(int N, int precision, const FusedLaunch& f, cudaStream_t st);
 // rtpn_create; batch_member contexts keep dense rows (the grouped kernels read their states)
 int create_context(rtpn_ctx** out, int N, int nx, int ny, int nz, double h, int bc, int precision, double dt,
                    bool batch_member);
-// Dense rows and a kernel that takes them (on), or the kernel and row pitch of the selection again (off).
+// Dense rows and a kernel that takes them (on), or the kernel, tile and row pitch of the selection again (off).
 int use_dense_rows(rtpn_ctx* ctx, bool on);
+// Another staged variant on padded rows, which belong to the automatic choice: by name a caller gets the staged
+// kernel on 16-byte rows only, so the tuner chooses among its tiles here.
+int use_staged_tile(rtpn_ctx* ctx, int tx, int ty, int tz, int depth);
 
 // transposed partner table (adjoint.cu): targets of class clsB, sources of the other class
 HostTable transposed_table(const Model& md, int clsB, const Geom& g);
@@ -226,6 +229,7 @@ struct rtpn_ctx {
     int px = 0;
     long long sV = 0;
     bool dense_rows = false;         // no padded rows now (use_dense_rows)
+    int padded_tile[4] = {0, 0, 0, 0};  // the staged tile and depth to come back to from there
     bool no_padding = false;         // created without room for padded rows
     bool batch_member = false;       // created by rtpn_batch_create (its kernels take cubic cells)
     double* scat = nullptr;          // f_l (l = 0..N) of anisotropic scattering on the device, or null

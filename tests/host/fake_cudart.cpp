@@ -28,6 +28,7 @@ auto& g_log = *new std::string;
 auto& g_out = *new std::string;
 size_t g_used = 0, g_limit = (size_t)1 << 60;
 cudaError_t g_last = cudaSuccess;
+float g_ms = 0, g_ms_step = 1;  // the next elapsed time, and how the ones after it change
 
 cudaError_t check(const char* api) {
     auto it = g_fail.find(api);
@@ -57,6 +58,10 @@ extern "C" {
 void fake_fail(const char* api, int after, int code) { g_fail[api] = {after, code}; }
 void fake_limit(size_t bytes) { g_limit = bytes; }
 size_t fake_used() { return g_used; }
+void fake_elapsed(float first, float step) {
+    g_ms = first;
+    g_ms_step = step;
+}
 void fake_clear() { g_log.clear(); }
 const char* fake_log() {
     g_out = g_log;
@@ -188,9 +193,7 @@ cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) {
-    // a timed run takes as long as the kernels launched so far: later candidates are slower
-    static float t = 0;
-    *ms = t += 1.f;
+    *ms = g_ms += g_ms_step;
     return cudaSuccess;
 }
 

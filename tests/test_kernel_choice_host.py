@@ -145,3 +145,36 @@ fake.fake_limit(dense)
 assert code(rtpn.Context, 15, shape, 0.1, "periodic", "bf16") == rtpn.ENOMEM
 assert fake.fake_used() == 0
 """)
+
+
+def test_tuner_on_padded_rows_tries_every_staged_tile(so):
+    fake_runtime.run(so, """
+import re
+text = open({root!r} + "/paper_2004_02833_gb300/csrc/stage_variants.h").read()
+tiles = [tuple(map(int, m)) for m in re.findall(r"X\\(15,\\s*(\\d+),\\s*(\\d+),\\s*(\\d+),\\s*(\\d+),", text)]
+assert len(tiles) > 4
+shape = (3, 4, 75)
+m = np.full(shape, 0.5)
+def use(i):
+    return tuple(i.tile) + (i.depth,)
+fake.fake_elapsed.argtypes = [ctypes.c_float, ctypes.c_float]
+for first, step, best in ((100.0, 1.0, tiles[0]), (1000.0, -1.0, tiles[-1])):
+    ctx = rtpn.Context(15, shape, 0.1, "periodic" if step > 0 else "vacuum")
+    ctx.set_media(m, m, m)
+    fake.fake_elapsed(first, step)
+    log()
+    tile, ms = ctx.autotune(reps=1)
+    assert len({{l for l in log() if "k_stage" in l}}) == len(tiles) * 2  # both classes of every variant
+    info = ctx.info()
+    assert (info.kernel, use(info), tile) == (3, best, best[:3])
+    # the adjoint's way over dense rows, and other cells, keep the tuned tile
+    ctx.adjoint(m, 1, ckpt_every=1)
+    assert (ctx.info().kernel, use(ctx.info())) == (3, best)
+    # a second context of the same problem takes it from the tuner's memory
+    other = rtpn.Context(15, shape, 0.1, "periodic" if step > 0 else "vacuum")
+    other.set_media(m, m, m)
+    assert other.autotune(reps=1)[0] == best[:3] and use(other.info()) == best
+    # a tile that fails to be set leaves the one in use
+    fail("cudaMemcpy", 0, 719)
+    assert code(other.autotune, 1) == rtpn.ECUDA and use(other.info()) == best and other.info().kernel == 3
+""".format(root=fake_runtime.ROOT))
