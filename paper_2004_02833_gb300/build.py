@@ -32,7 +32,7 @@ def _nvcc() -> str:
 
 
 VARIANT_SRC = "window.cu"  # compiled once per (order, class) listed in window_variants.h
-STAGE_SRC = "stage.cu"     # compiled once per (order, tile, depth, box size) listed in stage_variants.h
+STAGE_SRC = "stage.cu"     # compiled per entry of stage_variants.h, for cells with h_y = h_x and without
 FUSED_SRC = "fused.cu"     # compiled once per order listed in fused_variants.h
 
 
@@ -69,10 +69,11 @@ def units() -> list[tuple[str, list[str], str]]:
     for n in fused_orders():
         out.append((os.path.join(CSRC, FUSED_SRC), [f"-DRTPN_FN={n}"], f"fused_N{n}.o"))
     for n, tx, ty, tz, nb, em in stage_variants():
-        out.append((os.path.join(CSRC, STAGE_SRC),
-                    [f"-DRTPN_SN={n}", f"-DRTPN_STX={tx}", f"-DRTPN_STY={ty}", f"-DRTPN_STZ={tz}",
-                     f"-DRTPN_SNB={nb}", f"-DRTPN_SEM={em}"],
-                    f"stage_N{n}_{tx}x{ty}x{tz}_b{nb}_e{em}.o"))
+        for sc in (0, 1):
+            out.append((os.path.join(CSRC, STAGE_SRC),
+                        [f"-DRTPN_SN={n}", f"-DRTPN_STX={tx}", f"-DRTPN_STY={ty}", f"-DRTPN_STZ={tz}",
+                         f"-DRTPN_SNB={nb}", f"-DRTPN_SEM={em}", f"-DRTPN_SSC={sc}"],
+                        f"stage_N{n}_{tx}x{ty}x{tz}_b{nb}_e{em}_s{sc}.o"))
     return out
 
 

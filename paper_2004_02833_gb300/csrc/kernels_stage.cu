@@ -12,26 +12,34 @@
 namespace rtpn {
 namespace stg {
 
-#define RTPN_SDECL(n, x, y, z, b, e)                                                                 \
-    int stage_launch_##n##_##x##_##y##_##z##_##b##_##e(int, int, int, const Args&, int, cudaStream_t);  \
-    int stage_smem_##n##_##x##_##y##_##z##_##b##_##e(int, int);                                          \
-    void stage_geom_##n##_##x##_##y##_##z##_##b##_##e(int, int*);
+#define RTPN_SDECL1(n, x, y, z, b, e, f)                                                                     \
+    int stage_launch_##n##_##x##_##y##_##z##_##b##_##e##_##f(int, int, int, const Args&, int, cudaStream_t);  \
+    int stage_smem_##n##_##x##_##y##_##z##_##b##_##e##_##f(int, int);                                          \
+    void stage_geom_##n##_##x##_##y##_##z##_##b##_##e##_##f(int, int*);
+#define RTPN_SDECL(n, x, y, z, b, e) RTPN_SDECL1(n, x, y, z, b, e, 0) RTPN_SDECL1(n, x, y, z, b, e, 1)
 RTPN_STAGE_VARIANTS(RTPN_SDECL)
 #undef RTPN_SDECL
+#undef RTPN_SDECL1
 
 struct Variant {
     int N, tx, ty, tz, depth;
-    int (*launch)(int, int, int, const Args&, int, cudaStream_t);  // (cls, precision, mode, ...)
+    // by form: 0 plain, 1 SC (h_y != h_x)
+    int (*launch[2])(int, int, int, const Args&, int, cudaStream_t);  // (cls, precision, mode, ...)
     int (*smem)(int, int);
-    void (*geom)(int, int*);  // (precision, {maps per kind, CTAs per SM, x group width, x group rows})
+    void (*geom[2])(int, int*);  // (precision, {maps per kind, CTAs per SM, x group width, x group rows})
 };
-#define RTPN_SENTRY(n, x, y, z, b, e)                                                                \
-    Variant{n, x, y, z, b, stage_launch_##n##_##x##_##y##_##z##_##b##_##e,                           \
-            stage_smem_##n##_##x##_##y##_##z##_##b##_##e, stage_geom_##n##_##x##_##y##_##z##_##b##_##e},
+#define RTPN_SNAME(a, n, x, y, z, b, e, f) a##_##n##_##x##_##y##_##z##_##b##_##e##_##f
+#define RTPN_SENTRY(n, x, y, z, b, e)                                                                                 \
+    Variant{n, x, y, z, b, {RTPN_SNAME(stage_launch, n, x, y, z, b, e, 0), RTPN_SNAME(stage_launch, n, x, y, z, b, e, 1)}, \
+            RTPN_SNAME(stage_smem, n, x, y, z, b, e, 0),                                                              \
+            {RTPN_SNAME(stage_geom, n, x, y, z, b, e, 0), RTPN_SNAME(stage_geom, n, x, y, z, b, e, 1)}},
 static const Variant kVariants[] = {RTPN_STAGE_VARIANTS(RTPN_SENTRY)};
 #undef RTPN_SENTRY
+#undef RTPN_SNAME
 
-// a variant is usable for a storage precision if its stage ring fits shared memory
+static int form_of(const rtpn::Geom& g) { return g.hy != g.h ? 1 : 0; }
+
+// a variant is usable for a storage precision if its stage ring fits shared memory (of both forms or of neither)
 static bool fits(const Variant& v, int precision) { return v.smem(0, precision) > 0 && v.smem(1, precision) > 0; }
 
 // first compiled variant of order N with this tile (0 = any) and depth (0 = any) that fits
@@ -79,7 +87,7 @@ static bool make_map(CUtensorMap* m, void* base, int precision, const rtpn::Geom
 static bool make_maps(CUtensorMap* out, void* base, int precision, const rtpn::Geom& g, int px, long long sV, int nc,
                       const Variant& v, int kinds) {
     int geo[4];
-    v.geom(precision, geo);
+    v.geom[0](precision, geo);
     const int nmap = geo[0], xw = geo[2], ry = geo[3];
     for (int j = 0; j < nmap; ++j) {
         const int e = j + 1;
@@ -106,7 +114,7 @@ static const Variant* best_variant(int N, int precision, int depth, const rtpn::
     for (const auto& v : kVariants) {
         if (v.N != N || (depth != 0 && v.depth != depth) || !fits(v, precision)) continue;
         int geo[4];
-        v.geom(precision, geo);
+        v.geom[form_of(g)](precision, geo);
         const long long tiles = (long long)((g.nx + v.tx - 1) / v.tx) * ((g.ny + v.ty - 1) / v.ty) * ((g.nz + v.tz - 1) / v.tz);
         const long long slots = (long long)sms * geo[1];
         const long long rounds = (tiles + slots - 1) / slots;
@@ -126,7 +134,7 @@ static const Variant* best_variant(int N, int precision, int depth, const rtpn::
 
 static int nmaps_of(const Variant& v, int precision) {
     int geo[4];
-    v.geom(precision, geo);
+    v.geom[0](precision, geo);
     return geo[0];
 }
 
@@ -172,7 +180,7 @@ int stage_prepare(rtpn_ctx* ctx, int tx, int ty, int tz, int depth, int px) {
     if (!ctx->stage_mem) {
         std::vector<int> col;
         std::vector<float> tab[2];
-        if (!stg::coupling_tables(ctx->md, ctx->g.h / ctx->g.hy, ctx->g.h / ctx->g.hz, tab, &col))
+        if (!stg::coupling_tables(ctx->md, ctx->g.h / ctx->g.hy, ctx->g.h / ctx->g.hz, tab, &col, stg::form_of(ctx->g) != 0))
             return (int)cudaErrorInvalidValue;
         const size_t b0 = tab[0].size() * 4, b1 = tab[1].size() * 4, b2 = col.size() * 4;
         char* m = nullptr;
@@ -228,7 +236,6 @@ static bool base_args(const rtpn_ctx* ctx, const stg::Variant& v, int coef_cls, 
     a.nz = ctx->g.nz;
     a.bc = ctx->g.bc;
     a.inv_h = (float)(1.0 / ctx->g.h);
-    a.sy = (float)(ctx->g.h / ctx->g.hy);  // exactly 1 for cubic cells
     a.ntx = (a.nx + v.tx - 1) / v.tx;
     a.nty = (a.ny + v.ty - 1) / v.ty;
     a.ntz = (a.nz + v.tz - 1) / v.tz;
@@ -271,7 +278,7 @@ static int launch_pass(rtpn_ctx* ctx, int cls, int fac_ofs, const CUtensorMap* s
     a.src_c0 = cls == 1 ? 0 : ctx->md.ne;  // the source class is the other one
     a.wait_limit = (unsigned)(wait_limit > 0xffffffffll ? 0xffffffffll : wait_limit);
     a.skip_stage = skip_stage;
-    return v.launch(cls, ctx->prec, stg::FORWARD, a, ctx->sms, st);
+    return v.launch[stg::form_of(ctx->g)](cls, ctx->prec, stg::FORWARD, a, ctx->sms, st);
 }
 
 int launch_stage(rtpn_ctx* ctx, int cls, int fac_ofs, cudaStream_t st, long long skip_stage,
@@ -330,7 +337,7 @@ int launch_stage_adjoint_sources(rtpn_ctx* ctx, int tgt_cls, float* lam, const f
     a.tmap = dev + stg::MAP_KINDS * nmap;
     a.src_c0 = 0;  // w holds only the source class, in its local order
     a.nc = w_planes;
-    return v.launch(tgt_cls, RTPN_FP32, stg::ADJ_SOURCES, a, ctx->sms, st);
+    return v.launch[stg::form_of(ctx->g)](tgt_cls, RTPN_FP32, stg::ADJ_SOURCES, a, ctx->sms, st);
 }
 
 }  // namespace rtpn

@@ -83,6 +83,14 @@ constexpr unsigned STATUS_CHECK = 2u;  // a self-check failed (builds with RTPN_
 // (-k)(-dx) + (-k)(s dy) from column M+1, s = +-1 the same for the whole column.
 constexpr int CPAD = 6;       // constants per slot and type
 constexpr int KPAIRS = CPAD;  // pairs per slot
+// Cells with h_y != h_x (form SC): the y constants carry h / h_y, rounded once from the product, so they are
+// no longer the x ones: four more pairs per slot, to column M+1 and M-1 (l-1, l+1 each).  (Scaling the
+// differences by an FP32 h / h_y instead rounds twice, with one error for all of them: 8 to 10 % more
+// error at h / h_y = 1/1.1, 0.6 and 1/1.7 after forty P15 passes.)
+template <bool SC>
+RTPN_HD constexpr int slot_pairs() {
+    return SC ? 10 : KPAIRS;
+}
 
 // What a pass computes.  FORWARD: targets u_A' = alpha u_A - beta acc (Eq. 5; the u_0 factors for
 // l = 0).  ADJ_SOURCES: the transpose of a substep's coupling for the dual multipliers,
@@ -121,7 +129,7 @@ struct Args {
     long long skip_stage;   // stage index never issued (a wait that must run out); -1 normally
     int px = 0;             // row pitch of the target array and stride of its components
     long long sV = 0;
-    float sy = 1.f;         // h / h_y: scale of the y differences (non-cubic cells)
+    float sy = 1.f;         // scale of the y differences in a host run without form SC (the kernel's is 1)
 };
 
 __host__ __device__ constexpr int pad128(int bytes) { return (bytes + 127) / 128 * 128; }
@@ -138,8 +146,8 @@ __host__ __device__ constexpr int xhalo_width(int tx, int ty, int es) {
     return best;
 }
 
-// NCH: sub-stages of a column (each K = ceil((N/2 + 1) / NCH) source slots).
-template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH = 1>
+// NCH: sub-stages of a column (each K = ceil((N/2 + 1) / NCH) source slots).  SC: with y constants of their own.
+template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH = 1, bool SC = false>
 struct Layout {
     static constexpr int B = 1 - A;
     static constexpr int ES = (int)sizeof(S);
@@ -162,7 +170,8 @@ struct Layout {
     static constexpr int KY = TZ, KZ = TZ + 1, KX = TZ + 2, NKIND = TZ + 3;
     static constexpr int SRC_T = NKIND * REG;
     static constexpr int TGT_T = TZ * REGT;           // tile planes of one type's targets
-    static constexpr int COEF_COL = 2 * K * CPAD * 4;  // a sub-stage's coupling constants
+    static constexpr int PAIRS = slot_pairs<SC>();      // pairs of constants per slot
+    static constexpr int COEF_COL = 2 * K * PAIRS * 4;  // a sub-stage's coupling constants
     // buffer layout: target planes, type-0 sources, type-1 sources, coupling constants.  A block of
     // the sweep may read up to K - 1 slots below a source region; with the targets first, such reads
     // stay on state data (or the zeros the ring starts with) in the same buffer, never on the
@@ -225,12 +234,13 @@ RTPN_HD constexpr float y_sign(int M, int T) { return ((M ^ T) & 1) ? -1.f : 1.f
 // The coupling constants of the staged kernel (host; the library and its host check program):
 // per target class A, the constants of the source class by column and slot q
 // ([N+1][N/2+1][KPAIRS][2], layout above; slots of l < M stay zero), from the model's coupling
-// (win::coef_table).  The kernel applies 1/h of x and scales the y differences by h / h_y; the z
-// constants carry sz = h / h_z (exactly 1 for cubic cells).  col: the first local index of column M in
+// (win::coef_table).  The kernel applies 1/h of x; the z constants carry
+// sz = h / h_z (exactly 1 for cubic cells); scaled: the layout of form SC, whose y constants carry sy = h / h_y.  col: the first local index of column M in
 // class P at col[P (N + 2) + M].  False if the model's x and y couplings do not share their magnitudes
 // and signs as above.
-inline bool coupling_tables(const Model& md, double /*sy*/, double sz, std::vector<float> tab[2], std::vector<int>* col) {
-    const int N = md.N, nl = N / 2 + 1;
+inline bool coupling_tables(const Model& md, double sy, double sz, std::vector<float> tab[2], std::vector<int>* col,
+                            bool scaled = false) {
+    const int N = md.N, nl = N / 2 + 1, pairs = scaled ? slot_pairs<true>() : slot_pairs<false>();
     col->assign(2 * (N + 2), 0);
     for (int P = 0; P < 2; ++P) {
         int acc = 0;
@@ -243,11 +253,11 @@ inline bool coupling_tables(const Model& md, double /*sy*/, double sz, std::vect
         const int B = 1 - A;
         std::vector<float> t10;  // [local source index of class B][10]
         if (!win::coef_table(md, A, &t10)) return false;
-        tab[A].assign((size_t)(N + 1) * nl * 2 * KPAIRS, 0.f);
+        tab[A].assign((size_t)(N + 1) * nl * 2 * pairs, 0.f);
         for (int M = 0; M <= N; ++M)
             for (int j = 0; j < column_len(N, M, B); ++j) {
                 const int q = first_l(M, B) / 2 + j;  // the source's slot (l - B) / 2
-                float* d = &tab[A][((size_t)M * nl + q) * KPAIRS * 2];
+                float* d = &tab[A][((size_t)M * nl + q) * pairs * 2];
                 // relations of the source of type t (null if the type is absent)
                 auto rel = [&](int t) {
                     const int len = column_len(N, M, B);
@@ -263,8 +273,9 @@ inline bool coupling_tables(const Model& md, double /*sy*/, double sz, std::vect
                             const float s = side == 0 ? y_sign(M, T) : -y_sign(M, T);
                             // at |m| = 0 only one of the two sources exists
                             if (M > 0 ? y != s * x : (x != 0.f && y != 0.f)) return false;
-                            const float k = own ? x : s * y;
+                            const float k = own ? x : scaled ? 0.f : s * y;
                             d[(2 + 2 * side + dl) * 2 + T] = side == 0 ? k : -k;
+                            if (scaled) d[(6 + 2 * side + dl) * 2 + T] = (float)(y * sy) * y_sign(M, T);
                         }
                 }
             }
@@ -539,11 +550,11 @@ RTPN_HD constexpr int coef_slots(int C) {
 }
 // bytes that type t's boxes of a sub-stage with runs r bring into the buffer (the coupling constants
 // come with type 0), and those of both types
-template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH>
+template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH, bool SC = false>
 RTPN_HD unsigned type_bytes(const StageRuns& r, int C, int t) {
-    using L = Layout<N, A, S, TX, TY, TZ, NB, NCH>;
+    using L = Layout<N, A, S, TX, TY, TZ, NB, NCH, SC>;
     return (unsigned)(((t < r.nt ? L::NKIND * r.len : 0) + (t < r.ntA ? TZ * r.lenA : 0)) * L::UB) +
-           (t == 0 && r.nt > 0 ? (unsigned)coef_slots<N, NCH>(C) * (2 * CPAD * 4) : 0u);
+           (t == 0 && r.nt > 0 ? (unsigned)coef_slots<N, NCH>(C) * (2 * L::PAIRS * 4) : 0u);
 }
 template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH>
 RTPN_HD unsigned stage_bytes(const StageRuns& r, int C = 0) {
@@ -562,10 +573,10 @@ RTPN_HD constexpr unsigned full_parity(int s, int nb) { return (unsigned)(s / nb
 
 // Producer warp t: issues the copies of type t (and for t = 0 the coupling constants) of every sub-stage
 // of this CTA's sequence into the ring.  One lane issues; everything else is the same for the warp.
-template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH>
+template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH, bool SC>
 __device__ __forceinline__ void stage_producer(const Args& a, unsigned char* bufs, unsigned full0,
                                                unsigned empty0, volatile unsigned* next, int t) {
-    using L = Layout<N, A, S, TX, TY, TZ, NB, NCH>;
+    using L = Layout<N, A, S, TX, TY, TZ, NB, NCH, SC>;
     constexpr int B = 1 - A;
     constexpr int NST = N + 2;
     const int lane = threadIdx.x & 31;
@@ -610,7 +621,7 @@ __device__ __forceinline__ void stage_producer(const Args& a, unsigned char* buf
         }
         const unsigned buf = smem_addr(bufs + b * L::BUF);
         const StageRuns r = stage_runs<N, A, NCH>(i, C);
-        const unsigned bytes = type_bytes<N, A, S, TX, TY, TZ, NB, NCH>(r, C, t);
+        const unsigned bytes = type_bytes<N, A, S, TX, TY, TZ, NB, NCH, SC>(r, C, t);
         auto issue = [&](const BoxJob& bj) {
             // sources: components of the source array (a.nc); targets: of a full state array (u or lam)
             const int cmax = bj.target ? class_size(N, 0) + class_size(N, 1) : a.nc;
@@ -627,8 +638,8 @@ __device__ __forceinline__ void stage_producer(const Args& a, unsigned char* buf
                         issue(source_box<N, A, S, TX, TY, TZ, NB, NCH, decltype(kk)::value>(a, g, i, r, offB, t));
                     });
                     if (t == 0)
-                        bulk_load(buf + L::COEFO, a.coefcol + (long long)(i * L::NLC + C * L::K) * (2 * CPAD),
-                                  coef_slots<N, NCH>(C) * (2 * CPAD * 4), full);
+                        bulk_load(buf + L::COEFO, a.coefcol + (long long)(i * L::NLC + C * L::K) * (2 * L::PAIRS),
+                                  coef_slots<N, NCH>(C) * (2 * L::PAIRS * 4), full);
                 }
                 if (t < r.ntA)
                     static_for<TZ>([&](auto zz) {
@@ -728,8 +739,8 @@ RTPN_HD Operands operand_offsets(const TileGeo& g, int /*T*/, int lx, int ly, in
 }
 
 // What a column's sweep reads beside the sources themselves: the x and y partners (cos, sin) and the z
-// partner, as offsets in a stage buffer, and the factors of the y differences (h / h_y with the
-// column's sign, by target type).  At |m| = 0 the absent sin type's x and y differences are taken as
+// partner, as offsets in a stage buffer, and the factors of the y differences (the column's
+// sign by target type, times sy).  At |m| = 0 the absent sin type's x and y differences are taken as
 // zero: its partners are its own (stale) values.  src_t: offset between the types' regions.
 struct ColumnOps {
     int x0, x1, y0, y1, z;
@@ -750,7 +761,8 @@ RTPN_HD ColumnOps column_operands(const Operands& op, int i, int src_t, float sy
 // One source slot's operands, both types: value, x, y and z partners, and its constants.
 struct SlotOps {
     float c0, c1, x0, x1, y0, y1, z0, z1;
-    float4 kz, ku, kd;  // pairs to l-1, l+1: of column M (z), M+1 and (negated) M-1 (x and y)
+    float4 kz, ku, kd;  // pairs to l-1, l+1: of column M (z), M+1 and (negated) M-1 (x, and y unless SC)
+    float4 kuy, kdy;    // SC: of y to M+1 and M-1
 };
 
 // Scatter the slots of sub-stage C of source column i (in a stage buffer) into the accumulators of target
@@ -759,7 +771,7 @@ struct SlotOps {
 // 4-5).  At |m| = 0 only the cos type exists: the absent type's constants are zero or meet zero
 // differences (its regions hold earlier, finite data), so the same sweep serves every column.  fq: the
 // column's first source slot.
-template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH, int C>
+template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH, int C, bool SC = false>
 RTPN_HD void sweep_pairs(const unsigned char* buf, int c0, const ColumnOps& op, int fq,
                          float2 (&prev)[(N - A) / 2 + 1], float2 (&cur)[(N - A) / 2 + 1],
                          float2 (&next)[(N - A) / 2 + 1]) {
@@ -786,10 +798,15 @@ RTPN_HD void sweep_pairs(const unsigned char* buf, int c0, const ColumnOps& op, 
         o.y1 = lds<S>(py1, e);
         o.z0 = lds<S>(pz, e);
         o.z1 = lds<S>(pz, e + ST);
-        RTPN_CHECK_PTR(kc + (KPAIRS / 2) * k + 2);
-        o.kz = kc[(KPAIRS / 2) * k];
-        o.ku = kc[(KPAIRS / 2) * k + 1];
-        o.kd = kc[(KPAIRS / 2) * k + 2];
+        constexpr int n4 = slot_pairs<SC>() / 2;
+        RTPN_CHECK_PTR(kc + n4 * k + n4 - 1);
+        o.kz = kc[n4 * k];
+        o.ku = kc[n4 * k + 1];
+        o.kd = kc[n4 * k + 2];
+        if constexpr (SC) {
+            o.kuy = kc[n4 * k + 3];
+            o.kdy = kc[n4 * k + 4];
+        }
     };
     auto work = [&](const SlotOps& o, auto ki) {
         constexpr int q = C * K + decltype(ki)::value;
@@ -808,10 +825,12 @@ RTPN_HD void sweep_pairs(const unsigned char* buf, int c0, const ColumnOps& op, 
         if constexpr (has_p) prev[ap] = pair_fma(make_float2(o.kd.z, o.kd.w), nx, prev[ap]);
         if constexpr (has_m) next[am] = pair_fma(make_float2(o.ku.x, o.ku.y), dx, next[am]);
         if constexpr (has_p) next[ap] = pair_fma(make_float2(o.ku.z, o.ku.w), dx, next[ap]);
-        if constexpr (has_m) prev[am] = pair_fma(make_float2(o.kd.x, o.kd.y), dy, prev[am]);
-        if constexpr (has_p) prev[ap] = pair_fma(make_float2(o.kd.z, o.kd.w), dy, prev[ap]);
-        if constexpr (has_m) next[am] = pair_fma(make_float2(o.ku.x, o.ku.y), dy, next[am]);
-        if constexpr (has_p) next[ap] = pair_fma(make_float2(o.ku.z, o.ku.w), dy, next[ap]);
+        const float4& kd = SC ? o.kdy : o.kd;
+        const float4& ku = SC ? o.kuy : o.ku;
+        if constexpr (has_m) prev[am] = pair_fma(make_float2(kd.x, kd.y), dy, prev[am]);
+        if constexpr (has_p) prev[ap] = pair_fma(make_float2(kd.z, kd.w), dy, prev[ap]);
+        if constexpr (has_m) next[am] = pair_fma(make_float2(ku.x, ku.y), dy, next[am]);
+        if constexpr (has_p) next[ap] = pair_fma(make_float2(ku.z, ku.w), dy, next[ap]);
     };
     constexpr int NBLK = KC / kBlock > 0 ? KC / kBlock : 1;  // the last block takes the remainder
     static_for<NBLK>([&](auto bi) {
@@ -915,9 +934,9 @@ RTPN_HD void finish_column(const unsigned char* buf, int tgo, int M, int T, S* t
         make_float2(scale, scale), al0, be0, ga0, p);
 }
 
-template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH, int MODE>
+template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH, int MODE, bool SC>
 __device__ __forceinline__ void stage_kernel_body(const Args& a, unsigned char* smem) {
-    using L = Layout<N, A, S, TX, TY, TZ, NB, NCH>;
+    using L = Layout<N, A, S, TX, TY, TZ, NB, NCH, SC>;
     static_assert(N >= 1, "order N >= 1");
     static_assert(L::NMAP <= kMaxSlots, "tensor maps of a kind");
     constexpr int B = 1 - A;
@@ -953,7 +972,7 @@ __device__ __forceinline__ void stage_kernel_body(const Args& a, unsigned char* 
     __syncthreads();
 
     if (warp >= L::CONSUMER_WARPS) {
-        stage_producer<N, A, S, TX, TY, TZ, NB, NCH>(a, bufs, full0, empty0, next, warp - L::CONSUMER_WARPS);
+        stage_producer<N, A, S, TX, TY, TZ, NB, NCH, SC>(a, bufs, full0, empty0, next, warp - L::CONSUMER_WARPS);
         return;
     }
 
@@ -1008,7 +1027,7 @@ __device__ __forceinline__ void stage_kernel_body(const Args& a, unsigned char* 
         auto column = [&](int i, float2 (&prev)[NLA], float2 (&cur)[NLA], float2 (&next)[NLA]) {
             const int C0 = first_chunk<N, A, NCH>(i), fq = first_source<N, A>(i);
             const bool sources = i <= N && 2 * fq + B <= N;
-            const ColumnOps cop = column_operands(op, i, L::SRC_T, a.sy);
+            const ColumnOps cop = column_operands(op, i, L::SRC_T, 1.f);
             // target column M = i - 1
             const int M = i - 1, q0 = M >= 0 ? first_source<N, B>(M) : 0, lenA = NLA - q0;
             (void)RTPN_SCHECK(M < 0 || comp == (unsigned)(cA0 + colA[M]));
@@ -1028,7 +1047,7 @@ __device__ __forceinline__ void stage_kernel_body(const Args& a, unsigned char* 
                 const unsigned char* buf = bufs + b * (unsigned)L::BUF;
                 // the sweep and the finish run on every thread of the tile (a thread past the grid's edge
                 // works on zero-filled or in-tile shared memory), only global accesses need an active cell
-                if (sources) sweep_pairs<N, A, S, TX, TY, TZ, NB, NCH, C>(buf, op.c, cop, fq, prev, cur, next);
+                if (sources) sweep_pairs<N, A, S, TX, TY, TZ, NB, NCH, C, SC>(buf, op.c, cop, fq, prev, cur, next);
                 if (M >= 0)
                     finish_pairs<N, A, S, TX, TY, TZ, NB, NCH, MODE, C>(buf, tgo, M, q0, t0, t1, vb, active, sin_t, alpha,
                                                                         scale, al0, be0 * a.inv_h, ga0, prev);
