@@ -451,7 +451,7 @@ int set_rows(rtpn_ctx* ctx, int px) {
 // whether the automatic choice may pad the rows for the staged kernel
 bool may_pad(const rtpn_ctx* ctx) {
     return kStageInAuto && ctx->N >= kStageMinN && !ctx->batch_member && !ctx->no_padding && ctx->g.nx >= kPadMinNx &&
-           stage_compiled(ctx->N, ctx->prec);
+           stage_compiled(ctx->N, ctx->prec) && stage_sized(ctx->prec, ctx->g);
 }
 
 // The kernel for the context's selection, with what it needs.  Whatever can fail comes first; the kernel, its
@@ -480,7 +480,7 @@ int choose_kernel(rtpn_ctx* ctx) {
         const bool pad = may_pad(ctx) && !ctx->dense_rows && !tile_set &&
                          stage_has_tile(ctx->N, tx, ty, tz, depth, ctx->prec);
         if (kStageInAuto && (ctx->N >= kStageMinN || !win_ok) &&
-            (stage_supported(ctx->N, ctx->prec, ctx->g.nx) || pad) &&
+            (stage_supported(ctx->N, ctx->prec, ctx->g) || pad) &&
             (!tile_set || stage_has_tile(ctx->N, tx, ty, tz, depth, ctx->prec)))
             k = RTPN_KERNEL_STAGE;
         else
@@ -499,17 +499,20 @@ int choose_kernel(rtpn_ctx* ctx) {
     // the automatic choice runs the staged kernel on any width of rows, padding them; chosen by name it
     // takes 16-byte rows only
     const bool pad = k == RTPN_KERNEL_STAGE && ctx->kernel == RTPN_KERNEL_AUTO &&
-                     !stage_supported(ctx->N, ctx->prec, ctx->g.nx);
+                     !stage_supported(ctx->N, ctx->prec, ctx->g);
     if (k == RTPN_KERNEL_STAGE && !pad) {
-        if (!stage_supported(ctx->N, ctx->prec, ctx->g.nx))
+        if (!stage_supported(ctx->N, ctx->prec, ctx->g))
             return fail(ctx, RTPN_EUNSUPPORTED,
-                        "staged kernel not compiled for this N/precision or nx*elem not 16-byte rows");
+                        "staged kernel not compiled for this N/precision, nx*elem not 16-byte rows or a component of 4 GiB");
         if (!stage_has_tile(ctx->N, tx, ty, tz, depth, ctx->prec))
             return fail(ctx, RTPN_EUNSUPPORTED, "no staged kernel compiled for this tile / stage depth");
     }
     auto unprepared = [&](const char* what, int rc) {
         cudaGetLastError();  // reported here; the next launch check is not to see it
-        return fail(ctx, rc == (int)cudaErrorMemoryAllocation ? RTPN_ENOMEM : RTPN_ECUDA,
+        return fail(ctx,
+                    rc == (int)cudaErrorMemoryAllocation ? RTPN_ENOMEM
+                    : rc == (int)cudaErrorNotSupported   ? RTPN_EUNSUPPORTED
+                                                         : RTPN_ECUDA,
                     std::string(what) + ": " + cudaGetErrorString((cudaError_t)rc));
     };
     const int px = pad ? padded_pitch(ctx) : ctx->g.nx;

@@ -22,7 +22,7 @@ RTPN_STAGE_VARIANTS(RTPN_SDECL)
 #undef RTPN_SDECL1
 
 struct Variant {
-    int N, tx, ty, tz, depth;
+    int N, tx, ty, tz, depth, substages;
     // by form: 0 plain, 1 SC (h_y != h_x)
     int (*launch[2])(int, int, int, const Args&, int, cudaStream_t);  // (cls, precision, mode, ...)
     int (*smem)(int, int);
@@ -30,7 +30,7 @@ struct Variant {
 };
 #define RTPN_SNAME(a, n, x, y, z, b, e, f) a##_##n##_##x##_##y##_##z##_##b##_##e##_##f
 #define RTPN_SENTRY(n, x, y, z, b, e)                                                                                 \
-    Variant{n, x, y, z, b, {RTPN_SNAME(stage_launch, n, x, y, z, b, e, 0), RTPN_SNAME(stage_launch, n, x, y, z, b, e, 1)}, \
+    Variant{n, x, y, z, b, e, {RTPN_SNAME(stage_launch, n, x, y, z, b, e, 0), RTPN_SNAME(stage_launch, n, x, y, z, b, e, 1)}, \
             RTPN_SNAME(stage_smem, n, x, y, z, b, e, 0),                                                              \
             {RTPN_SNAME(stage_geom, n, x, y, z, b, e, 0), RTPN_SNAME(stage_geom, n, x, y, z, b, e, 1)}},
 static const Variant kVariants[] = {RTPN_STAGE_VARIANTS(RTPN_SENTRY)};
@@ -147,8 +147,20 @@ bool stage_compiled(int N, int precision) {
     return precision != RTPN_FP64 && stg::find(N, 0, 0, 0, 0, precision) != nullptr;
 }
 
-bool stage_supported(int N, int precision, int nx) {
-    return stage_compiled(N, precision) && nx % stage_row_group(precision) == 0;
+bool stage_sized(int precision, const Geom& g) {
+    const int grp = stage_row_group(precision);
+    const long long px = (g.nx + grp - 1) / grp * grp;
+    return px * g.ny * g.nz < (1ll << 32) / (precision == RTPN_BF16 ? 2 : 4);
+}
+
+bool stage_supported(int N, int precision, const Geom& g) {
+    return stage_compiled(N, precision) && g.nx % stage_row_group(precision) == 0 && stage_sized(precision, g);
+}
+
+// stages of a pass over the grid, at most: the kernel counts a CTA's in 32 bits
+static long long stages_of(const stg::Variant& v, const Geom& g) {
+    return (long long)((g.nx + v.tx - 1) / v.tx) * ((g.ny + v.ty - 1) / v.ty) * ((g.nz + v.tz - 1) / v.tz) * (v.N + 2) *
+           v.substages;
 }
 
 bool stage_has_tile(int N, int tx, int ty, int tz, int depth, int precision) {
@@ -163,6 +175,7 @@ int stage_prepare(rtpn_ctx* ctx, int tx, int ty, int tz, int depth, int px) {
     cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, dev);
     if (tx == 0)
         if (const stg::Variant* w = stg::best_variant(ctx->N, ctx->prec, depth, ctx->g, px, ctx->sms)) v = w;
+    if (stages_of(*v, ctx->g) >= (1ll << 31)) return (int)cudaErrorNotSupported;
     const int N = ctx->N;
     // the tensor maps live in device global memory (64-byte aligned) and the kernel reads them from
     // there: tile planes / z halo plane, y halo row and x halo group, each for every box length
@@ -240,8 +253,8 @@ static bool base_args(const rtpn_ctx* ctx, const stg::Variant& v, int coef_cls, 
     a.nty = (a.ny + v.ty - 1) / v.ty;
     a.ntz = (a.nz + v.tz - 1) / v.tz;
     a.tiles = (long long)a.ntx * a.nty * a.ntz;
-    // 32-bit stage counts and 32-bit byte strides of a component
-    if (a.tiles * (ctx->N + 2) * 4 >= (1ll << 31) || ctx->sV * (long long)ctx->elem >= (1ll << 32)) return false;
+    // (the selection has seen to both)
+    if (stages_of(v, ctx->g) >= (1ll << 31) || !stage_sized(ctx->prec, ctx->g)) return false;
     // z chunk of the tile walk: the ~one tile per SM at work at a time then spans about as many
     // tile rows in y as layers in z, across the whole x extent
     const double side = std::sqrt((double)(ctx->sms > 0 ? ctx->sms : 1) / a.ntx);

@@ -168,10 +168,12 @@ int use_staged_tile(rtpn_ctx* ctx, int tx, int ty, int tz, int depth);
 HostTable transposed_table(const Model& md, int clsB, const Geom& g);
 
 // ---- TMA-staged kernels (kernels_stage.cu, stage.cu) ----
-// compiled for (N, precision); rows must be 16-byte groups for the tensor maps (stage_row_group values)
+// compiled for (N, precision); rows must be 16-byte groups for the tensor maps (stage_row_group values), and a
+// component's bytes, padded so, below 2^32 (stage_sized: the kernel's byte strides are 32-bit)
 bool stage_compiled(int N, int precision);
 inline int stage_row_group(int precision) { return precision == RTPN_BF16 ? 8 : 4; }
-bool stage_supported(int N, int precision, int nx);
+bool stage_sized(int precision, const Geom& g);
+bool stage_supported(int N, int precision, const Geom& g);
 bool stage_has_tile(int N, int tx, int ty, int tz, int depth, int precision);
 // builds the tensor maps (tile 0,0,0 = default; depth 0 = any) and the coupling tables;
 // returns cudaError_t

@@ -178,3 +178,20 @@ for first, step, best in ((100.0, 1.0, tiles[0]), (1000.0, -1.0, tiles[-1])):
     fail("cudaMemcpy", 0, 719)
     assert code(other.autotune, 1) == rtpn.ECUDA and use(other.info()) == best and other.info().kernel == 3
 """.format(root=fake_runtime.ROOT))
+
+
+def test_components_of_4_gib_are_refused_at_the_selection(so):
+    # the staged kernel's byte strides are 32-bit: AUTO takes another kernel, the kernel by name is refused
+    fake_runtime.run(so, """
+for precision, nz in (("fp32", 1024), ("bf16", 2048)):
+    for nx, kernel in ((1016, 3), (1024, 2)):
+        ctx = rtpn.Context(15, (nz, 1024, nx), 0.1, "periodic", precision)
+        assert ctx.info().kernel == kernel, (precision, nx)
+        assert code(ctx.set_kernel, "stage") == (rtpn.OK if kernel == 3 else rtpn.EUNSUPPORTED)
+        assert ctx.info().kernel == kernel
+        ctx.close()
+    # rows that would reach it by their padding
+    ctx = rtpn.Context(15, (nz, 1024, 1023), 0.1, "periodic", precision)
+    assert ctx.info().kernel == 2
+    ctx.close()
+""")
