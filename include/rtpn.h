@@ -166,7 +166,8 @@ int rtpn_set_stream(rtpn_ctx* ctx, void* stream);
  * RTPN_KERNEL_AUTO picks STAGE (for N >= 15; where nx >= 8 gives no 16-byte rows the state's rows are padded
  * inside the library, except in a batch), then WINDOW, then GENERIC; with non-cubic cells STAGE (any
  * compiled N), else GENERIC; with anisotropic scattering GENERIC.  Moving between padded and dense rows
- * rearranges the state in place.
+ * rearranges the state in place, stream-ordered; RTPN_ESTATE while the context stream is being captured, and a
+ * graph that the caller captured before has to be captured again.
  * RTPN_EUNSUPPORTED if the kernel is not compiled for (N, precision, nx) or does not take the
  * context's cells or scattering; the previous selection then stays. */
 int rtpn_set_kernel(rtpn_ctx* ctx, int kernel, int tile_x, int tile_y, int tile_z);

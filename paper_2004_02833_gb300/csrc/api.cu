@@ -516,6 +516,14 @@ int choose_kernel(rtpn_ctx* ctx) {
                     std::string(what) + ": " + cudaGetErrorString((cudaError_t)rc));
     };
     const int px = pad ? padded_pitch(ctx) : ctx->g.nx;
+    if (px != ctx->px) {
+        // recorded into the caller's graph, the rearranging would run at each replay and not now
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+            cudaGetLastError();
+            return fail(ctx, RTPN_ESTATE, "the state's rows cannot be rearranged while the stream is being captured");
+        }
+    }
     if (k == RTPN_KERNEL_GENERIC && generic_compiled(ctx)) {
         int rc = window64_prepare(ctx->md);
         if (rc) return unprepared("generic kernel constants", rc);

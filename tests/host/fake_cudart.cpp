@@ -28,6 +28,7 @@ auto& g_log = *new std::string;
 auto& g_out = *new std::string;
 size_t g_used = 0, g_limit = (size_t)1 << 60;
 cudaError_t g_last = cudaSuccess;
+bool g_capturing = false;
 float g_ms = 0, g_ms_step = 1;  // the next elapsed time, and how the ones after it change
 
 cudaError_t check(const char* api) {
@@ -58,6 +59,7 @@ extern "C" {
 void fake_fail(const char* api, int after, int code) { g_fail[api] = {after, code}; }
 void fake_limit(size_t bytes) { g_limit = bytes; }
 size_t fake_used() { return g_used; }
+void fake_capturing(int on) { g_capturing = on != 0; }
 void fake_elapsed(float first, float step) {
     g_ms = first;
     g_ms_step = step;
@@ -169,7 +171,7 @@ cudaError_t cudaStreamSynchronize(cudaStream_t) {
 }
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* s) {
-    *s = cudaStreamCaptureStatusNone;
+    *s = g_capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
     return cudaSuccess;
 }
 cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { return cudaSuccess; }

@@ -195,3 +195,21 @@ for precision, nz in (("fp32", 1024), ("bf16", 2048)):
     assert ctx.info().kernel == 2
     ctx.close()
 """)
+
+
+def test_rows_are_not_rearranged_into_the_callers_graph(so):
+    fake_runtime.run(so, COMMON + """
+ctx = context()
+fake.fake_capturing(1)
+for kernel in ("window", "generic"):
+    assert code(ctx.set_kernel, kernel) == rtpn.ESTATE
+    assert layout(ctx) == (3, padded) and kernels(log(), "k_rows") == 0
+ctx.step(1)  # the staged passes can be captured
+assert any("k_stage" in l for l in log())
+fake.fake_capturing(0)
+ctx.set_kernel("window")
+fake.fake_capturing(1)
+ctx.set_kernel("generic")  # dense rows both: nothing to rearrange
+assert code(ctx.set_kernel, "auto") == rtpn.ESTATE
+assert layout(ctx) == (1, dense)
+""")
