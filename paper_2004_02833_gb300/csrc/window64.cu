@@ -33,10 +33,44 @@ __device__ __forceinline__ const double* coef_of() {
     return nullptr;
 }
 
+// The launch over a grid: a.tx > 0, tiles of 32 cells of a row (times 1 x 1 or 2 x 2 rows); a.tx = 0, the cells in
+// the order of memory, so that short rows share a warp.  An FP64-bound warp costs the same with one lane
+// as with 32: tiles only where they keep nine lanes in ten.  (GB300, P7 64 x 64 x nx, a step in us, the table
+// kernel / tiles / this: nx = 5 128 / 212 / 48, 16 188 / 212 / 114, 33 376 / 421 / 216, 65 648 / 626 / 424.)  One warp per block until every SM has eight
+// 128-thread blocks: the FP64 units of every SM then have about the same number of warps to serve.
+void shape64(const Geom& g, win::Args* a, unsigned* blocks, unsigned* threads) {
+    const bool small = g.V < 152ll * 8 * 128;
+    const int row = (g.nx + 31) / 32 * 32;
+    if (10ll * g.nx >= 9ll * row) {
+        a->tx = 32;
+        a->ty = a->tz = small ? 1 : 2;
+        a->ntx = (g.nx + a->tx - 1) / a->tx;
+        a->nty = (g.ny + a->ty - 1) / a->ty;
+        a->ntz = (g.nz + a->tz - 1) / a->tz;
+        *blocks = (unsigned)a->ntx * a->nty * a->ntz;
+        *threads = (unsigned)(a->tx * a->ty * a->tz);
+    } else {
+        a->tx = a->ty = a->tz = a->ntx = a->nty = a->ntz = 0;
+        *threads = small ? 32 : 128;
+        *blocks = (unsigned)((g.V + *threads - 1) / *threads);
+    }
+}
+RTPN_HD bool cell64(const win::Args& a, unsigned blk, unsigned tid, unsigned threads, int* x, int* y, int* z) {
+    if (a.tx > 0) return win::cell_of(a, (int)blk, (int)tid, x, y, z);
+    const long long c = (long long)blk * threads + tid;
+    if (c >= a.V) return false;
+    // 32-bit divisions where they do (a 64-bit one is tens of instructions)
+    const long long row = a.V < (1ll << 32) ? (long long)((unsigned)c / (unsigned)a.nx) : c / a.nx;
+    *x = (int)(c - row * a.nx);
+    *z = a.V < (1ll << 32) ? (int)((unsigned)row / (unsigned)a.ny) : (int)(row / a.ny);
+    *y = (int)(row - (long long)*z * a.ny);
+    return true;
+}
+
 template <int N, int A>
 __global__ void __launch_bounds__(128) k_window64(win::Args a) {
     int x, y, z;
-    if (!win::cell_of(a, blockIdx.x, threadIdx.x, &x, &y, &z)) return;
+    if (!cell64(a, blockIdx.x, threadIdx.x, blockDim.x, &x, &y, &z)) return;
     win::substep_cell<N, A, double, false, false, double>(a, coef_of<N, A>(), x, y, z);
 }
 
@@ -93,15 +127,8 @@ int launch_window64(int N, double* u, const double* fac, const Geom& g, int cls,
     a.fac_ofs = fac_ofs;
     a.inv_h = (float)(1.0 / g.h);
     a.inv_h64 = 1.0 / g.h;
-    // one warp per block until every SM has eight 128-thread blocks: the FP64 units of every SM then have
-    // about the same number of warps to serve
-    const bool small = g.V < 152ll * 8 * 128;
-    a.tx = 32;
-    a.ty = a.tz = small ? 1 : 2;
-    a.ntx = (a.nx + a.tx - 1) / a.tx;
-    a.nty = (a.ny + a.ty - 1) / a.ty;
-    a.ntz = (a.nz + a.tz - 1) / a.tz;
-    const unsigned blocks = (unsigned)a.ntx * a.nty * a.ntz, threads = (unsigned)(a.tx * a.ty * a.tz);
+    unsigned blocks, threads;
+    shape64(g, &a, &blocks, &threads);
     switch (N) {
 #define RTPN_CASE(n)                                                  \
     case n:                                                           \
