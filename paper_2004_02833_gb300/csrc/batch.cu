@@ -55,7 +55,7 @@ __device__ __forceinline__ const float* coef_of() {
 template <int N, int A, typename S>
 __global__ void __launch_bounds__(256) k_batch(const Inst* __restrict__ inst, int count,
                                                long long items, int tx, int ty, int tz,
-                                               int fac_ofs, unsigned long long* counter) {
+                                               int fac_ofs, int prefetch, unsigned long long* counter) {
     __shared__ long long s_item;
     for (;;) {
         if (threadIdx.x == 0) s_item = (long long)atomicAdd(counter, 1ull);
@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(256) k_batch(const Inst* __restrict__ inst, in
         a.nty = I.nty;
         a.ntz = I.ntz;
         if constexpr (win::prefetches(N))
-            win::prefetch_tile<N, A, S, false>(a, (int)(it - I.block0), threadIdx.x, blockDim.x);
+            if (prefetch) win::prefetch_tile<N, A, S, false>(a, (int)(it - I.block0), threadIdx.x, blockDim.x);
         int x, y, z;
         if (win::cell_of(a, (int)(it - I.block0), threadIdx.x, &x, &y, &z))
             win::substep_cell<N, A, S>(a, coef_of<N, A>(), x, y, z);
@@ -151,6 +151,7 @@ struct rtpn_batch {
     unsigned long long* counter = nullptr;  // one work counter per group
     int prec = RTPN_FP32;
     int tx = 32, ty = 4, tz = 2;
+    int prefetch = 0;                   // the instances together do not stay in L2 (win::kPrefetchBytes)
     cudaStream_t stream = nullptr, own = nullptr;
     std::map<int, cudaGraphExec_t> graphs;
     bool media_set_all = false;
@@ -187,6 +188,9 @@ const void* kernel_of(int N) {
 int build_items(rtpn_batch* b) {
     std::vector<bat::Inst> h;
     b->groups.clear();
+    double bytes = 0;
+    for (rtpn_ctx* c : b->ctx) bytes += win::pass_bytes(c->N, (int)c->elem, false) * (double)c->g.V;
+    b->prefetch = bytes >= win::kPrefetchBytes;
     for (int idx : b->order) {
         rtpn_ctx* c = b->ctx[idx];
         if (b->groups.empty() || b->groups.back().N != c->N) {
@@ -238,7 +242,7 @@ void launch_group(const BatchGroup& gr, rtpn_batch* b, int fac_ofs, unsigned lon
 #define RTPN_LAUNCH(n)                                                                              \
     case n:                                                                                         \
         bat::k_batch<n, A, S><<<gr.grid, threads, 0, st>>>(b->d_inst + gr.first, gr.count, gr.items, \
-                                                           b->tx, b->ty, b->tz, fac_ofs, counter);  \
+                                                           b->tx, b->ty, b->tz, fac_ofs, b->prefetch, counter);  \
         break;
         RTPN_BATCH_ORDERS(RTPN_LAUNCH)
 #undef RTPN_LAUNCH

@@ -83,11 +83,13 @@ int launch_window(int N, int precision, const WindowLaunch& w, cudaStream_t st) 
     a.sy = (float)(w.g.h / w.g.hy);  // exactly 1 for cubic cells
     a.sz = (float)(w.g.h / w.g.hz);
     a.aniso = w.aniso ? 1 : 0;
+    a.prefetch = win::prefetches(N) &&
+                 win::pass_bytes(N, precision == RTPN_BF16 ? 2 : 4, w.aniso) * (double)w.g.V >= win::kPrefetchBytes;
     a.tx = w.tx > 0 ? w.tx : 32;
     a.ty = w.ty > 0 ? w.ty : 4;
     // without a tile given: 32 x 4 x 2, or one plane of it where the tile's rows are prefetched (P7 128^3 even /
     // odd pass 0.184 / 0.189 ms with 32 x 2 x 2, 0.180 / 0.183 with 32 x 4 x 1)
-    a.tz = w.tz > 0 ? w.tz : (w.tx == 0 && w.ty == 0 && win::prefetches(N)) ? 1 : 2;
+    a.tz = w.tz > 0 ? w.tz : (w.tx == 0 && w.ty == 0 && a.prefetch) ? 1 : 2;
     if (a.tx * a.ty * a.tz > 256 || (a.tx * a.ty * a.tz) % 32 != 0) return (int)cudaErrorInvalidValue;
     a.ntx = (a.nx + a.tx - 1) / a.tx;
     a.nty = (a.ny + a.ty - 1) / a.ty;

@@ -33,7 +33,8 @@ __constant__ float c_coef[kSources * 10];
 // 1.85; a P3 32^3 step with the state out 9.3 us against 9.8.)
 template <typename S, bool SCALED, bool ANISO>
 __global__ void __launch_bounds__(256) k_window(Args a) {
-    if constexpr (prefetches(kN)) prefetch_tile<kN, kA, S, ANISO>(a, blockIdx.x, threadIdx.x, blockDim.x);
+    if constexpr (prefetches(kN))
+        if (a.prefetch) prefetch_tile<kN, kA, S, ANISO>(a, blockIdx.x, threadIdx.x, blockDim.x);
     int x, y, z;
     if (!cell_of(a, blockIdx.x, threadIdx.x, &x, &y, &z)) return;
     substep_cell<kN, kA, S, SCALED, ANISO>(a, c_coef, x, y, z);

@@ -187,6 +187,7 @@ struct Args {
     int ntx, nty, ntz;  // tiles per axis
     float sy = 1.f, sz = 1.f;  // h / h_y, h / h_z: the y and z differences' scale (non-cubic cells)
     int aniso = 0;             // factors per (sub-grid, order l): anisotropic scattering
+    int prefetch = 0;          // ask L2 for a tile's rows first (only in orders with prefetches(N))
     double inv_h64 = 0;        // 1 / h of the FP64 arithmetic
 };
 
@@ -214,6 +215,15 @@ RTPN_HD bool cell_of(const Args& a, int blk, int tid, int* x, int* y, int* z) {
 // before the sweep comes to them).  Asking for a tile that runs later is slower the later it runs
 // (P7: 0.195 ms for the tile 114 blocks ahead, 0.253 for 760).
 __host__ __device__ constexpr bool prefetches(int N) { return N >= 5 && N <= 9; }
+// ... and where the passes' data do not stay in L2 (129 MB) anyway: there the requests are only in the way.  A
+// step with against without, by the bytes of the state and the factors in use (GB300; N = 5, 7, 9, FP32 and
+// BF16, cubic, non-cubic and per-order factors): 1.05 to 1.35 below 90 MB, 0.95 to 1.05 from there to 110, 0.71 to
+// 0.98 above.
+constexpr double kPrefetchBytes = 100e6;
+// those bytes of a cell: the state, eight (alpha, beta) pairs or one per (sub-grid, order), and u_0's three
+inline double pass_bytes(int N, int elem, bool aniso) {
+    return (N + 1.0) * (N + 1.0) * elem + (aniso ? 32.0 * (N + 1) : 64.0) + 12.0;
+}
 
 // Ask L2 for every row of tile blk: the sources of class 1 - A, then the targets, then with per-order
 // factors (ANISO) the factor rows of the targets.

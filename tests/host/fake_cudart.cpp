@@ -40,10 +40,11 @@ cudaError_t check(const char* api) {
     }
     return cudaSuccess;
 }
-cudaError_t launched(const void* fn) {
+cudaError_t launched(const void* fn, dim3 block) {
     if (cudaError_t e = check("launch")) return e;
     auto it = g_names.find(fn);
-    g_log += "K " + (it == g_names.end() ? std::string("?") : it->second) + "\n";
+    g_log += "K " + (it == g_names.end() ? std::string("?") : it->second) + " threads " +
+             std::to_string(block.x * block.y * block.z) + "\n";
     return cudaSuccess;
 }
 struct Config {
@@ -209,12 +210,14 @@ cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const
     *n = 1;
     return cudaSuccess;
 }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t*, const void* fn, void**) { return launched(fn); }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* fn, void**) { return launched(fn, c->blockDim); }
 cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* fn) {
     *k = (cudaKernel_t)fn;
     return cudaSuccess;
 }
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void**, size_t, cudaStream_t) { return launched((const void*)k); }
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3 block, void**, size_t, cudaStream_t) {
+    return launched((const void*)k, block);
+}
 unsigned __cudaPushCallConfiguration(dim3 grid, dim3 block, size_t smem, void* stream) {
     g_configs.push_back({grid, block, smem, stream});
     return 0;

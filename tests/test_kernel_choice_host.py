@@ -213,3 +213,35 @@ ctx.set_kernel("generic")  # dense rows both: nothing to rearrange
 assert code(ctx.set_kernel, "auto") == rtpn.ESTATE
 assert layout(ctx) == (1, dense)
 """)
+
+
+def test_window_passes_prefetch_where_the_data_do_not_stay_in_l2(so):
+    # the default tile shows the choice: 32 x 4 x 1 with the requests to L2, 32 x 4 x 2 without (every other order too)
+    fake_runtime.run(so, """
+def threads(N, shape, precision, aniso=False, spacing=None):
+    ctx = rtpn.Context(N, shape, 0.1, "periodic", precision)
+    ctx.set_kernel("window")
+    if aniso:
+        ctx.set_scattering([0.8 ** l for l in range(N + 1)])
+    if spacing:
+        ctx.set_spacing(*spacing)
+    m = np.full(shape, 0.5)
+    ctx.set_media(m, m, m)
+    log()
+    ctx.substep(0)
+    t = [int(l.split()[-1]) for l in log() if "k_window" in l]
+    ctx.close()
+    assert len(t) == 1
+    return t[0]
+
+for N in (5, 7, 9):
+    for precision, elem in (("fp32", 4), ("bf16", 2)):
+        for aniso in (False, True):
+            cell = (N + 1) ** 2 * elem + 12 + (32 * (N + 1) if aniso else 64)
+            nz = int(100e6 / (cell * 32 * 32))
+            assert threads(N, (nz, 32, 32), precision, aniso) == 256
+            assert threads(N, (nz + 1, 32, 32), precision, aniso) == 128
+            assert threads(N, (8, 9, 10), precision, aniso, (0.1, 0.12, 0.13)) == 256
+for N in (1, 3, 15):
+    assert threads(N, (64, 64, 64), "fp32") == 256
+""")
