@@ -110,9 +110,15 @@ static bool make_maps(CUtensorMap* out, void* base, int precision, const rtpn::G
 static const Variant* best_variant(int N, int precision, int depth, const rtpn::Geom& g, int px, int sms) {
     const Variant* best = nullptr;
     double best_cost = 0;
+    // From N = 29 on a tile's stages one after another are most of a small grid's pass, and columns in one stage of
+    // 15 or 20 slots take longer than in sub-stages, whatever the rounds: such variants run by name only.  GB300,
+    // us a step, 32x2x2 in one stage / in two: P39 FP32 20x22x32 143 / 117, 40x43x32 387 / 320, BF16 183 / 145, 400 / 338;
+    // P29 FP32 80 / 69, BF16 90 / 80.
+    const bool sub_staged = N >= 29;
     const int es = precision == RTPN_BF16 ? 2 : 4;
     for (const auto& v : kVariants) {
         if (v.N != N || (depth != 0 && v.depth != depth) || !fits(v, precision)) continue;
+        if (sub_staged && depth == 0 && v.substages == 1) continue;
         int geo[4];
         v.geom[form_of(g)](precision, geo);
         const long long tiles = (long long)((g.nx + v.tx - 1) / v.tx) * ((g.ny + v.ty - 1) / v.ty) * ((g.nz + v.tz - 1) / v.tz);

@@ -245,3 +245,27 @@ for N in (5, 7, 9):
 for N in (1, 3, 15):
     assert threads(N, (64, 64, 64), "fp32") == 256
 """)
+
+
+def test_default_tile_of_small_grids_at_high_orders_is_sub_staged(so):
+    # columns in one stage of 15 or 20 slots are slower at any size: they run by name (or by a depth) only
+    fake_runtime.run(so, """
+import itertools, random, re
+text = open({root!r} + "/paper_2004_02833_gb300/csrc/stage_variants.h").read()
+one = {{tuple(map(int, m[:5])) for m in re.findall(r"X\\((\\d+), (\\d+), (\\d+), (\\d+), (\\d+), (\\d+)\\)", text) if m[5] == "1"}}
+assert any(v[0] == 39 for v in one) and any(v[0] == 29 for v in one)
+rng = random.Random(1)
+for N in (29, 39):
+    for precision in ("fp32", "bf16"):
+        for _ in range(60):
+            shape = tuple(rng.randint(1, 64) for _ in range(2)) + (rng.randint(8, 130),)
+            ctx = rtpn.Context(N, shape, 0.1, "periodic", precision)
+            i = ctx.info()
+            assert i.kernel == 3 and (N, *i.tile, i.depth) not in one, (shape, tuple(i.tile), i.depth)
+            ctx.close()
+    ctx = rtpn.Context(N, (4, 4, 64), 0.1)
+    for v in sorted(one):
+        if v[0] == N and not (N == 39 and v[4] == 4):  # (four buffers of 40 cells fit BF16 only)
+            ctx.set_kernel("stage", v[1:4], v[4])
+            assert (N, *ctx.info().tile, ctx.info().depth) == v
+""".format(root=fake_runtime.ROOT))
