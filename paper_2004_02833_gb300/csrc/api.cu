@@ -414,16 +414,18 @@ void release(rtpn_ctx* ctx) {
 constexpr bool kStageInAuto = true;
 constexpr int kStageMinN = 15;
 // Rows of fewer than 8 cells are not padded: up to three cells in four would be padding, and the staged tiles
-// are at least 32 cells wide (P19 64 x 64 x nx FP32, a pass, staged against the generic kernel: nx = 5 0.080 and
-// 0.057 ms, 7 0.079 and 0.077, 9 0.099 and 0.095; 75 0.18 and 1.09 at 61 x 77).
+// are at least 32 cells wide.  (GB300, us a step on n x n x nx cells, staged / the kernel it replaces: P15 window
+// kernel, n = 12, 24, 48: nx = 9 30 / 52, 38 / 54, 40 / 59; nx = 33 31 / 56, 40 / 59, 107 / 123; P39 window kernel:
+// nx = 9 129 / 232, 154 / 223, 407 / 816.  P19 and P29 run the generic kernel otherwise, whose targets are split over
+// blocks on small grids: below some 6000 cells it is the faster one (P19 nx = 9: 40 / 18, 49 / 39, 101 / 117; P29 nx = 33
+// 78 / 70, 91 / 251), though far from the 650 us such a P19 step took before the split.)
 constexpr int kPadMinNx = 8;
 
 // Row pitch of the state: nx, or nx padded to 16-byte rows.  set_rows rearranges the state in place, a component
 // at a time through the staging plane (its buffer holds the padded state if the context can ever need
 // it); the padding holds zeros.
 int padded_pitch(const rtpn_ctx* ctx) {
-    const int grp = stage_row_group(ctx->prec);
-    return (ctx->g.nx + grp - 1) / grp * grp;
+    return stage_row_pitch(ctx->prec, ctx->g.nx);
 }
 int set_rows(rtpn_ctx* ctx, int px) {
     const Geom& g = ctx->g;

@@ -154,9 +154,8 @@ bool stage_compiled(int N, int precision) {
 }
 
 bool stage_sized(int precision, const Geom& g) {
-    const int grp = stage_row_group(precision);
-    const long long px = (g.nx + grp - 1) / grp * grp;
-    return px * g.ny * g.nz < (1ll << 32) / (precision == RTPN_BF16 ? 2 : 4);
+    const int px = g.nx % stage_row_group(precision) == 0 ? g.nx : stage_row_pitch(precision, g.nx);
+    return (long long)px * g.ny * g.nz < (1ll << 32) / (precision == RTPN_BF16 ? 2 : 4);
 }
 
 bool stage_supported(int N, int precision, const Geom& g) {

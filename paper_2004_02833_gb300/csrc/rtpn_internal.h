@@ -172,6 +172,13 @@ HostTable transposed_table(const Model& md, int clsB, const Geom& g);
 // component's bytes, padded so, below 2^32 (stage_sized: the kernel's byte strides are 32-bit)
 bool stage_compiled(int N, int precision);
 inline int stage_row_group(int precision) { return precision == RTPN_BF16 ? 8 : 4; }
+// Pitch of padded rows: 16-byte groups, and FP32 rows below 32 cells whole 32-byte sectors, because short rows
+// that start inside a sector share more of them than they fill (GB300, us a step, 48 x 48 x nx, to groups / to
+// sectors: P15 nx = 17 76 / 53, 27 56 / 52; P39 nx = 9 456 / 407, 17 468 / 404; a P15 window step at nx = 17: 59).
+inline int stage_row_pitch(int precision, int nx) {
+    const int grp = precision == RTPN_FP32 && nx < 32 ? 8 : stage_row_group(precision);
+    return (nx + grp - 1) / grp * grp;
+}
 bool stage_sized(int precision, const Geom& g);
 bool stage_supported(int N, int precision, const Geom& g);
 bool stage_has_tile(int N, int tx, int ty, int tz, int depth, int precision);

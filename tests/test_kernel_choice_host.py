@@ -269,3 +269,26 @@ for N in (29, 39):
             ctx.set_kernel("stage", v[1:4], v[4])
             assert (N, *ctx.info().tile, ctx.info().depth) == v
 """.format(root=fake_runtime.ROOT))
+
+
+def test_pitch_of_padded_rows(so):
+    # 16-byte groups; FP32 rows below 32 cells whole 32-byte sectors; 16-byte rows stay as they are
+    fake_runtime.run(so, """
+for precision, elem in (("fp32", 4), ("bf16", 2)):
+    for N in (15, 39):
+        for nx in range(1, 70):
+            ctx = rtpn.Context(N, (2, 3, nx), 0.1, "periodic", precision)
+            group = 16 // elem
+            if nx % group == 0:
+                px = nx
+            elif nx < 8:
+                px = nx  # not padded: a kernel that takes any width
+            elif precision == "fp32" and nx < 32:
+                px = -(-nx // 8) * 8
+            else:
+                px = -(-nx // group) * group
+            i = ctx.info()
+            assert i.state_bytes == (N + 1) ** 2 * 2 * 3 * px * elem, (precision, nx)
+            assert (i.kernel == 3) == (px % group == 0), (precision, nx, i.kernel)
+            ctx.close()
+""")
