@@ -768,6 +768,49 @@ int rtpn_destroy(rtpn_ctx* ctx) {
     return RTPN_OK;
 }
 
+}  // extern "C"
+
+namespace {
+// The tables that a call replaces, put back if a later part of it fails: the context is then as it was, and its
+// kernels have tables to read.
+struct KeptTables {
+    rtpn_ctx* c;
+    void *mem, *stage = nullptr;
+    bool with_stage;
+    size_t stage_bytes[2];
+    PartnerTable<double> t64[2];
+    PartnerTable<float> t32[2];
+    KeptTables(rtpn_ctx* ctx, bool with_staged) : c(ctx), mem(ctx->table_mem), with_stage(with_staged) {
+        for (int i = 0; i < 2; ++i) {
+            t64[i] = c->tab64[i];
+            t32[i] = c->tab32[i];
+            stage_bytes[i] = c->stage_tab_bytes[i];
+        }
+        c->table_mem = nullptr;
+        if (with_stage) std::swap(stage, c->stage_mem);
+    }
+    void put_back() {
+        if (c->table_mem) cudaFree(c->table_mem);
+        c->table_mem = mem;
+        for (int i = 0; i < 2; ++i) {
+            c->tab64[i] = t64[i];
+            c->tab32[i] = t32[i];
+        }
+        if (with_stage) {
+            if (c->stage_mem) cudaFree(c->stage_mem);
+            c->stage_mem = stage;
+            std::copy(stage_bytes, stage_bytes + 2, c->stage_tab_bytes);
+        }
+    }
+    void drop() {
+        if (mem) cudaFree(mem);
+        if (stage) cudaFree(stage);
+    }
+};
+}  // namespace
+
+extern "C" {
+
 int rtpn_set_spacing(rtpn_ctx* ctx, double hx, double hy, double hz) {
     if (!ctx) return RTPN_EINVAL;
     if (!(hx > 0.0 && hy > 0.0 && hz > 0.0) || !std::isfinite(hx) || !std::isfinite(hy) ||
@@ -791,15 +834,19 @@ int rtpn_set_spacing(rtpn_ctx* ctx, double hx, double hy, double hz) {
                    (ctx->kernel == RTPN_KERNEL_WINDOW && !window_extended(ctx->N))))
         return restore(RTPN_EUNSUPPORTED, "the fused kernel, and the window kernel above N = 15, take cubic cells only");
     // the partner tables and the staged kernel's constants carry the spacing: rebuild them
-    CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
-    if (ctx->table_mem) cudaFree(ctx->table_mem);
-    ctx->table_mem = nullptr;
-    int rc = upload_tables(ctx);
-    if (rc) return rc;
-    if (ctx->stage_mem) cudaFree(ctx->stage_mem);
-    ctx->stage_mem = nullptr;
+    if (cudaError_t e = cudaStreamSynchronize(ctx->stream)) return restore(RTPN_ECUDA, cudaGetErrorString(e));
     drop_graphs(ctx);
-    return choose_kernel(ctx);
+    KeptTables kept(ctx, true);
+    int rc = upload_tables(ctx);
+    if (!rc) rc = choose_kernel(ctx);
+    if (rc) {
+        cudaGetLastError();
+        kept.put_back();
+        ctx->g = old;
+        return rc;
+    }
+    kept.drop();
+    return RTPN_OK;
 }
 
 int rtpn_set_scattering(rtpn_ctx* ctx, const double* f, int count) {
@@ -842,19 +889,32 @@ int rtpn_set_scattering(rtpn_ctx* ctx, const double* f, int count) {
             return fail(ctx, RTPN_ENOMEM, "factor planes of anisotropic scattering");
         }
     }
-    if (ctx->scat) cudaFree(ctx->scat);
+    drop_graphs(ctx);
+    double* const old_scat = ctx->scat;
+    void* const old_fac = ctx->fac;
+    const int old_planes = ctx->fac_planes;
     ctx->scat = scat;
     if (fac) {
-        cudaFree(ctx->fac);
         ctx->fac = fac;
         ctx->fac_planes = planes;
     }
-    drop_graphs(ctx);
-    if (ctx->table_mem) cudaFree(ctx->table_mem);
-    ctx->table_mem = nullptr;
+    KeptTables kept(ctx, false);
     int rc = upload_tables(ctx);
     if (!rc) rc = choose_kernel(ctx);
-    if (!rc && ctx->media_set) {  // the factors of the media already set, with the new moments
+    if (rc) {
+        cudaGetLastError();
+        kept.put_back();
+        if (scat) cudaFree(scat);
+        if (fac) cudaFree(fac);
+        ctx->scat = old_scat;
+        ctx->fac = old_fac;
+        ctx->fac_planes = old_planes;
+        return rc;
+    }
+    kept.drop();
+    if (old_scat) cudaFree(old_scat);
+    if (fac) cudaFree(old_fac);
+    if (ctx->media_set) {  // the factors of the media already set, with the new moments
         const double* m = ctx->media;
         if (ctx->prec == RTPN_FP64)
             launch_media_factors<double>(m, m + V, m + 2 * V, (double*)ctx->fac, ctx->g, ctx->dt,

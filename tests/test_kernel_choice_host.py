@@ -292,3 +292,36 @@ for precision, elem in (("fp32", 4), ("bf16", 2)):
             assert (i.kernel == 3) == (px % group == 0), (precision, nx, i.kernel)
             ctx.close()
 """)
+
+
+def test_spacing_and_scattering_that_fail_leave_the_context(so):
+    fake_runtime.run(so, COMMON + """
+f = [0.8 ** l for l in range(16)]
+for option in ("spacing", "scattering"):
+    failed = 0
+    for after in range(8):
+        for api in ("cudaMalloc", "cudaMemcpy"):
+            ctx = context()
+            call = (lambda: ctx.set_spacing(0.1, 0.13, 0.17)) if option == "spacing" else (lambda: ctx.set_scattering(f))
+            before = fake.fake_used(), layout(ctx), ctx.info().hy, ctx.info().factor_bytes, tuple(ctx.info().tile)
+            fail(api, after, 2)
+            rc = code(call)
+            fake.fake_fail(api.encode(), 1 << 30, 0)
+            if rc == rtpn.OK:
+                continue
+            failed += 1
+            now = fake.fake_used(), layout(ctx), ctx.info().hy, ctx.info().factor_bytes, tuple(ctx.info().tile)
+            assert now == before, (option, api, after, now, before)
+            ctx.step(2)  # its kernels still have their tables
+            assert layout(ctx) == (3, padded)
+            ctx.close()
+    assert failed >= 4, (option, failed)
+ctx = context()
+ctx.set_spacing(0.1, 0.13, 0.17)
+assert ctx.info().hy == 0.13
+ctx.set_spacing(0.1, 0.1, 0.1)
+ctx.set_scattering(f)
+assert layout(ctx) == (2, dense)
+ctx.set_scattering(None)
+assert layout(ctx) == (3, padded)
+""")
