@@ -227,12 +227,6 @@ __global__ void k_dot_u0<double>(const double* __restrict__ u0, const double* __
     }
 }
 
-template <typename A, typename B>
-__global__ void k_copy_cast(const A* __restrict__ in, B* __restrict__ out, long long n) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        out[i] = (B)in[i];
-}
-
 // the same with padded rows of u_0 (nx values, px apart)
 template <typename S>
 __global__ void k_dot_rows(const S* __restrict__ u0, int nx, int px, const double* __restrict__ w, long long n,
@@ -251,6 +245,12 @@ __global__ void k_dot_rows(const S* __restrict__ u0, int nx, int px, const doubl
         for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += ws[i];
         partial[blockIdx.x] = s;
     }
+}
+
+template <typename A, typename B>
+__global__ void k_copy_cast(const A* __restrict__ in, B* __restrict__ out, long long n) {
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        out[i] = (B)in[i];
 }
 
 unsigned blocks_for(long long V, int threads = 256) { return (unsigned)((V + threads - 1) / threads); }

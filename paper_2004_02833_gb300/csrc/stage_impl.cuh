@@ -68,6 +68,9 @@ constexpr int kMaxSlots = 24;  // tensor maps of a kind, at most
 // above them; slots of a block below the first source carry zero constants and read finite shared
 // memory.
 constexpr int kBlock = 2;
+// A sub-stage's last block takes the remainder, so a block has up to 2 kBlock - 1 slots; one that holds the
+// column's first source may start that many less one below it.
+constexpr int kBelow = 2 * kBlock - 2;
 // Producer warps: one for each type's boxes of every stage.
 constexpr int kProducers = 2;
 
@@ -173,7 +176,7 @@ struct Layout {
     static constexpr int PAIRS = slot_pairs<SC>();      // pairs of constants per slot
     static constexpr int COEF_COL = 2 * K * PAIRS * 4;  // a sub-stage's coupling constants
     // buffer layout: target planes, type-0 sources, type-1 sources, coupling constants.  A block of
-    // the sweep may read up to K - 1 slots below a source region; with the targets first, such reads
+    // the sweep may read up to kBelow slots below a source region; with the targets first, such reads
     // stay on state data (or the zeros the ring starts with) in the same buffer, never on the
     // coupling constants, whose bits need not be finite in the storage type.
     static constexpr int TGTO = 0;
@@ -187,7 +190,7 @@ struct Layout {
     static_assert(TX % G == 0, "tile width must be a multiple of the 16-byte group");
     static_assert(CELLS % 32 == 0, "the tile's cells must fill whole warps");
     static_assert(NB >= 2 && NB <= 8, "two to eight stage buffers");
-    static_assert(2 * TGT_T >= (kBlock - 1) * UB, "blocks read at most kBlock - 1 slots below a region");
+    static_assert(2 * TGT_T >= kBelow * UB && REG >= kBelow * UB, "a block's reads below a region stay in the one before");
     static_assert(NCH == 1 || K >= 2, "a sub-stage of class 1 finishes one slot behind its sources");
     // the ring fits 227 KB of shared memory per CTA, and an x halo group exists for this element
     // size (a tile too narrow for RY >= TY rows of 16-byte groups is compiled for FP32 only)
@@ -708,7 +711,7 @@ struct Operands {
     int c, y[2], z[2], x[2][2];
 };
 
-// T: kept for callers that walk a tile type by type; the offsets serve both types
+// T: kept for host programs that walk a tile type by type; the offsets serve both types
 template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH>
 RTPN_HD Operands operand_offsets(const TileGeo& g, int /*T*/, int lx, int ly, int lz) {
     using L = Layout<N, A, S, TX, TY, TZ, NB, NCH>;
@@ -846,7 +849,8 @@ RTPN_HD void sweep_pairs(const unsigned char* buf, int c0, const ColumnOps& op, 
     });
 }
 
-// The lane of type T of sweep_pairs over a whole column, for callers that walk a tile type by type.
+#ifdef RTPN_HOST_CHECK
+// The lane of type T of sweep_pairs over a whole column, for host programs that walk a tile type by type.
 template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH>
 RTPN_HD void sweep_column(const unsigned char* buf, const Operands& op, int T, int i,
                           float (&prev)[(N - A) / 2 + 1], float (&cur)[(N - A) / 2 + 1],
@@ -868,6 +872,7 @@ RTPN_HD void sweep_column(const unsigned char* buf, const Operands& op, int T, i
         next[q] = T ? n[q].y : n[q].x;
     }
 }
+#endif
 
 // Finish the slots of target column M that sub-stage C completes, both types (accumulators in prev),
 // from their old values in the stage's target planes (at byte offset tgo for this cell; the sin type
@@ -916,8 +921,9 @@ RTPN_HD void finish_pairs(const unsigned char* buf, int tgo, int M, int q0, char
     });
 }
 
+#ifdef RTPN_HOST_CHECK
 // The same for type T alone over a whole column (accumulators, factors and the run's first component
-// tp of that type), for callers that walk a tile type by type.
+// tp of that type), for host programs that walk a tile type by type.
 template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH, int MODE>
 RTPN_HD void finish_column(const unsigned char* buf, int tgo, int M, int T, S* tp, long long V, bool active,
                            float alpha, float beta, float al0, float be0, float ga0, float inv_h,
@@ -933,6 +939,7 @@ RTPN_HD void finish_column(const unsigned char* buf, int tgo, int M, int T, S* t
         (unsigned)(V * (long long)sizeof(S)), active && T == 0, active && T == 1, make_float2(alpha, alpha),
         make_float2(scale, scale), al0, be0, ga0, p);
 }
+#endif
 
 template <int N, int A, typename S, int TX, int TY, int TZ, int NB, int NCH, int MODE, bool SC>
 __device__ __forceinline__ void stage_kernel_body(const Args& a, unsigned char* smem) {
