@@ -52,10 +52,11 @@ __device__ __forceinline__ const float* coef_of() {
 
 // Persistent, for the instances of one order N: each CTA repeatedly takes the next tile index from
 // *counter until all of the group's tiles are done.
-template <int N, int A, typename S>
+// PREFETCH: a tile asks L2 for its rows before its sweep (orders with win::prefetches).
+template <int N, int A, typename S, bool PREFETCH>
 __global__ void __launch_bounds__(256) k_batch(const Inst* __restrict__ inst, int count,
                                                long long items, int tx, int ty, int tz,
-                                               int fac_ofs, int prefetch, unsigned long long* counter) {
+                                               int fac_ofs, unsigned long long* counter) {
     __shared__ long long s_item;
     for (;;) {
         if (threadIdx.x == 0) s_item = (long long)atomicAdd(counter, 1ull);
@@ -85,8 +86,8 @@ __global__ void __launch_bounds__(256) k_batch(const Inst* __restrict__ inst, in
         a.ntx = I.ntx;
         a.nty = I.nty;
         a.ntz = I.ntz;
-        if constexpr (win::prefetches(N))
-            if (prefetch) win::prefetch_tile<N, A, S, false>(a, (int)(it - I.block0), threadIdx.x, blockDim.x);
+        if constexpr (PREFETCH)
+            win::prefetch_tile<N, A, S, false>(a, (int)(it - I.block0), threadIdx.x, blockDim.x);
         int x, y, z;
         if (win::cell_of(a, (int)(it - I.block0), threadIdx.x, &x, &y, &z))
             win::substep_cell<N, A, S>(a, coef_of<N, A>(), x, y, z);
@@ -151,7 +152,7 @@ struct rtpn_batch {
     unsigned long long* counter = nullptr;  // one work counter per group
     int prec = RTPN_FP32;
     int tx = 32, ty = 4, tz = 2;
-    int prefetch = 0;                   // the instances together do not stay in L2 (win::kPrefetchBytes)
+    bool prefetch = false;              // the instances together do not stay in L2 (win::kPrefetchBytes)
     cudaStream_t stream = nullptr, own = nullptr;
     std::map<int, cudaGraphExec_t> graphs;
     bool media_set_all = false;
@@ -170,13 +171,16 @@ void drop_graphs(rtpn_batch* b) {
     b->graphs.clear();
 }
 
-// the kernel of order N, class A, storage S (for the occupancy query)
+// the kernel of order N, class A, storage S
+using BatchKernel = void (*)(const bat::Inst*, int, long long, int, int, int, int, unsigned long long*);
 template <int A, typename S>
-const void* kernel_of(int N) {
+BatchKernel kernel_of(int N, bool prefetch) {
     switch (N) {
-#define RTPN_KER(n) \
-    case n:         \
-        return (const void*)bat::k_batch<n, A, S>;
+#define RTPN_KER(n)                                                     \
+    case n:                                                             \
+        if constexpr (win::prefetches(n))                               \
+            if (prefetch) return bat::k_batch<n, A, S, true>;           \
+        return bat::k_batch<n, A, S, false>;
         RTPN_BATCH_ORDERS(RTPN_KER)
 #undef RTPN_KER
         default:
@@ -225,7 +229,8 @@ int build_items(rtpn_batch* b) {
     const int threads = b->tx * b->ty * b->tz;
     for (auto& gr : b->groups) {
         // the two classes' kernels differ little in registers: size the grid by the even one's
-        const void* k = b->prec == RTPN_BF16 ? kernel_of<0, __nv_bfloat16>(gr.N) : kernel_of<0, float>(gr.N);
+        const void* k = b->prec == RTPN_BF16 ? (const void*)kernel_of<0, __nv_bfloat16>(gr.N, b->prefetch)
+                                             : (const void*)kernel_of<0, float>(gr.N, b->prefetch);
         int per_sm = 0;
         e = k ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, 0) : cudaErrorInvalidValue;
         if (e != cudaSuccess || per_sm < 1) per_sm = 1;
@@ -237,18 +242,9 @@ int build_items(rtpn_batch* b) {
 
 template <int A, typename S>
 void launch_group(const BatchGroup& gr, rtpn_batch* b, int fac_ofs, unsigned long long* counter, cudaStream_t st) {
-    const int threads = b->tx * b->ty * b->tz;
-    switch (gr.N) {
-#define RTPN_LAUNCH(n)                                                                              \
-    case n:                                                                                         \
-        bat::k_batch<n, A, S><<<gr.grid, threads, 0, st>>>(b->d_inst + gr.first, gr.count, gr.items, \
-                                                           b->tx, b->ty, b->tz, fac_ofs, b->prefetch, counter);  \
-        break;
-        RTPN_BATCH_ORDERS(RTPN_LAUNCH)
-#undef RTPN_LAUNCH
-        default:
-            break;
-    }
+    if (const BatchKernel k = kernel_of<A, S>(gr.N, b->prefetch))
+        k<<<gr.grid, b->tx * b->ty * b->tz, 0, st>>>(b->d_inst + gr.first, gr.count, gr.items, b->tx, b->ty, b->tz, fac_ofs,
+                                                     counter);
 }
 
 int batch_pass(rtpn_batch* b, int cls, int fac_ofs, cudaStream_t st) {

@@ -31,24 +31,30 @@ __constant__ float c_coef[kSources * 10];
 // all but the smallest grids, because the compiler then keeps loads behind the stores to the same state: GB300,
 // FP32, ten steps, P7 128^3 4.05 ms against 3.50, ragged 67 x 90 x 101 1.45 against 1.22, per-order factors 96^3 2.72 against
 // 1.85; a P3 32^3 step with the state out 9.3 us against 9.8.)
-template <typename S, bool SCALED, bool ANISO>
+// PREFETCH is a form of its own: beside the requests' code the sweep alone lost 3 %, 5 to 17 % with per-order factors.
+template <typename S, bool SCALED, bool ANISO, bool PREFETCH>
 __global__ void __launch_bounds__(256) k_window(Args a) {
-    if constexpr (prefetches(kN))
-        if (a.prefetch) prefetch_tile<kN, kA, S, ANISO>(a, blockIdx.x, threadIdx.x, blockDim.x);
+    if constexpr (PREFETCH) prefetch_tile<kN, kA, S, ANISO>(a, blockIdx.x, threadIdx.x, blockDim.x);
     int x, y, z;
     if (!cell_of(a, blockIdx.x, threadIdx.x, &x, &y, &z)) return;
     substep_cell<kN, kA, S, SCALED, ANISO>(a, c_coef, x, y, z);
 }
 
-template <bool SCALED, bool ANISO>
-int launch_form(int precision, const Args& a, cudaStream_t st) {
+template <bool SCALED, bool ANISO, bool PREFETCH>
+int launch_one(int precision, const Args& a, cudaStream_t st) {
     const int threads = a.tx * a.ty * a.tz;
     const unsigned blocks = (unsigned)a.ntx * a.nty * a.ntz;
     if (precision == RTPN_BF16)
-        k_window<__nv_bfloat16, SCALED, ANISO><<<blocks, threads, 0, st>>>(a);
+        k_window<__nv_bfloat16, SCALED, ANISO, PREFETCH><<<blocks, threads, 0, st>>>(a);
     else
-        k_window<float, SCALED, ANISO><<<blocks, threads, 0, st>>>(a);
+        k_window<float, SCALED, ANISO, PREFETCH><<<blocks, threads, 0, st>>>(a);
     return (int)cudaGetLastError();
+}
+template <bool SCALED, bool ANISO>
+int launch_form(int precision, const Args& a, cudaStream_t st) {
+    if constexpr (prefetches(kN))
+        if (a.prefetch) return launch_one<SCALED, ANISO, true>(precision, a, st);
+    return launch_one<SCALED, ANISO, false>(precision, a, st);
 }
 
 // the form a launch needs; the non-cubic and anisotropic forms exist up to kExtendedMaxN (a
