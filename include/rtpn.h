@@ -66,7 +66,8 @@ extern "C" {
 
 /* ---- step kernels ---- */
 #define RTPN_KERNEL_AUTO    0  /* fastest available for (N, precision)                            */
-#define RTPN_KERNEL_GENERIC 1  /* any N and precision: one thread per cell, partner-table gather   */
+#define RTPN_KERNEL_GENERIC 1  /* any N and precision: one thread per cell, partner-table gather (FP64 at
+                                  N = 1, 3, 5, 7, 9, cubic cells, isotropic: a compiled form)     */
 #define RTPN_KERNEL_WINDOW  2  /* FP32/BF16, compiled N: register-window scatter over m-columns  */
 #define RTPN_KERNEL_STAGE   3  /* FP32/BF16, compiled N, nx*elem a multiple of 16 B (AUTO: any nx, see
                                   rtpn_set_kernel): column loop with TMA-staged shared-memory
@@ -140,17 +141,16 @@ int rtpn_destroy(rtpn_ctx* ctx);
  * RTPN_EUNSUPPORTED if another kernel is selected explicitly, for a batch instance, and later for
  * rtpn_adjoint; RTPN_KERNEL_AUTO moves to the window kernel where it applies, else to the generic
  * one.  Allocates 32 (N + 1) more factor
- * planes (RTPN_ENOMEM leaves the context unchanged) and recomputes the factors of the media already
+ * planes (a failure leaves the context unchanged) and recomputes the factors of the media already
  * set; synchronises the context stream.  RTPN_EINVAL on a bad count or f. */
 int rtpn_set_scattering(rtpn_ctx* ctx, const double* f, int count);
 
 /* Cell sizes along x, y and z (rtpn_create sets all three to h): the differences of Section 2.1
  * divide by the cell size of their own axis, and dt must stay below min(hx, hy, hz)/3 (RTPN_ECFL
- * otherwise; the spacing is then unchanged).  Non-cubic cells run on the staged and generic kernels
- * (and the adjoint): RTPN_EUNSUPPORTED if the window or fused kernel is selected explicitly, and
- * for a batch instance (its spacing is fixed at rtpn_batch_create); RTPN_KERNEL_AUTO moves to the
- * staged or generic kernel.  Rebuilds the
- * coupling tables (synchronises the context stream); the media factors do not depend on h. */
+ * otherwise; the spacing is then unchanged, as after any failure).  Non-cubic cells run on the staged and
+ * generic kernels, on the window kernel up to N = 15 (and in the adjoint): RTPN_EUNSUPPORTED if the fused kernel
+ * or the window kernel above N = 15 is selected explicitly, and for a batch instance (its spacing is fixed at
+ * rtpn_batch_create); RTPN_KERNEL_AUTO moves to a kernel that takes them.  Rebuilds the coupling tables (synchronises the context stream); the media factors do not depend on h. */
 int rtpn_set_spacing(rtpn_ctx* ctx, double hx, double hy, double hz);
 
 /* Order all later work of the context on `stream` (a cudaStream_t; NULL = legacy default). */
@@ -158,14 +158,17 @@ int rtpn_set_stream(rtpn_ctx* ctx, void* stream);
 
 /* Select the step kernel (RTPN_KERNEL_*) and its CTA tile (tile_x * tile_y * tile_z threads, one
  * cell each; all 0 = default).  RTPN_KERNEL_WINDOW: the tile must hold a multiple of 32 threads, at
- * most 256 (RTPN_EINVAL); default 32 x 4 x 2.  RTPN_KERNEL_STAGE: the tile must be one compiled for
+ * most 256 (RTPN_EINVAL); default 32 x 4 x 2 (32 x 4 x 1 at N = 5, 7, 9 where state and factors are
+ * 100 MB and more).  RTPN_KERNEL_STAGE: the tile must be one compiled for
  * N (RTPN_EUNSUPPORTED otherwise).  RTPN_KERNEL_FUSED: the CTA tile is fixed at 32 x 8 cells, so
  * tile_x and tile_y must be 0 (or 32 and 8); tile_z is the number of z planes a CTA streams through
  * (0 = one wave of resident CTAs).  Selecting it allocates a second state buffer (RTPN_ENOMEM if
  * that fails); RTPN_EUNSUPPORTED for a batch instance.
  * RTPN_KERNEL_AUTO picks STAGE (for N >= 15; where nx >= 8 gives no 16-byte rows the state's rows are padded
- * inside the library, except in a batch), then WINDOW, then GENERIC; with non-cubic cells STAGE (any
- * compiled N), else GENERIC; with anisotropic scattering GENERIC.  Moving between padded and dense rows
+ * inside the library, except in a batch, and unless a tile, or a depth that no variant has, is asked for), then
+ * WINDOW, then GENERIC; with non-cubic cells the same, where WINDOW takes them up to N = 15 and STAGE any
+ * compiled N without a WINDOW form; with anisotropic scattering WINDOW up to N = 15, else GENERIC.  STAGE takes
+ * components below 4 GiB (rows padded).  Moving between padded and dense rows
  * rearranges the state in place, stream-ordered; RTPN_ESTATE while the context stream is being captured, and a
  * graph that the caller captured before has to be captured again.
  * RTPN_EUNSUPPORTED if the kernel is not compiled for (N, precision, nx) or does not take the

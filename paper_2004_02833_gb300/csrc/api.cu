@@ -415,10 +415,10 @@ constexpr bool kStageInAuto = true;
 constexpr int kStageMinN = 15;
 // Rows of fewer than 8 cells are not padded: up to three cells in four would be padding, and the staged tiles
 // are at least 32 cells wide.  (GB300, us a step on n x n x nx cells, staged / the kernel it replaces: P15 window
-// kernel, n = 12, 24, 48: nx = 9 30 / 52, 38 / 54, 40 / 59; nx = 33 31 / 56, 40 / 59, 107 / 123; P39 window kernel:
-// nx = 9 129 / 232, 154 / 223, 407 / 816.  P19 and P29 run the generic kernel otherwise, whose targets are split over
-// blocks on small grids: below some 6000 cells it is the faster one (P19 nx = 9: 40 / 18, 49 / 39, 101 / 117; P29 nx = 33
-// 78 / 70, 91 / 251), though far from the 650 us such a P19 step took before the split.)
+// kernel, n = 12, 24, 48: nx = 9 30 / 52, 32 / 54, 37 / 59; nx = 33 29 / 56, 35 / 59, 88 / 123; P39 window kernel:
+// nx = 9 114 / 232, 119 / 223, 390 / 816.  P19 and P29 run the generic kernel otherwise, whose targets are split over
+// blocks on small grids: below some 5000 cells it is the faster one (P19 nx = 9: 41 / 18, 44 / 38, 91 / 117; P29 nx = 33
+// 69 / 70, 88 / 251), though far from the 650 us such a P19 step took before the split.)
 constexpr int kPadMinNx = 8;
 
 // Row pitch of the state: nx, or nx padded to 16-byte rows.  set_rows rearranges the state in place, a component

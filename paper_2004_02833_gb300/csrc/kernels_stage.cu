@@ -65,13 +65,14 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     return fn;
 }
 
-// px, sV: row pitch and component stride of the array
+// px, sV: row pitch and component stride of the array.  The map spans the padding of padded rows too: it holds zeros,
+// as the columns outside the map would read.
 static bool make_map(CUtensorMap* m, void* base, int precision, const rtpn::Geom& g, int px, long long sV, int nc,
                      int bx, int by, int bz, int bc) {
     auto fn = encode_fn();
     if (!fn) return false;
     const cuuint64_t es = precision == RTPN_BF16 ? 2 : 4;
-    const cuuint64_t dims[4] = {(cuuint64_t)g.nx, (cuuint64_t)g.ny, (cuuint64_t)g.nz, (cuuint64_t)nc};
+    const cuuint64_t dims[4] = {(cuuint64_t)px, (cuuint64_t)g.ny, (cuuint64_t)g.nz, (cuuint64_t)nc};
     const cuuint64_t strides[3] = {px * es, (cuuint64_t)px * g.ny * es, (cuuint64_t)sV * es};
     const cuuint32_t box[4] = {(cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)bz, (cuuint32_t)bc};
     const cuuint32_t estr[4] = {1, 1, 1, 1};

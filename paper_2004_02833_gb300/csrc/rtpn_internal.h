@@ -172,11 +172,12 @@ HostTable transposed_table(const Model& md, int clsB, const Geom& g);
 // component's bytes, padded so, below 2^32 (stage_sized: the kernel's byte strides are 32-bit)
 bool stage_compiled(int N, int precision);
 inline int stage_row_group(int precision) { return precision == RTPN_BF16 ? 8 : 4; }
-// Pitch of padded rows: 16-byte groups, and FP32 rows below 32 cells whole 32-byte sectors, because short rows
-// that start inside a sector share more of them than they fill (GB300, us a step, 48 x 48 x nx, to groups / to
-// sectors: P15 nx = 17 76 / 53, 27 56 / 52; P39 nx = 9 456 / 407, 17 468 / 404; a P15 window step at nx = 17: 59).
+// Pitch of padded rows: 16-byte groups, and FP32 rows below 40 cells whole 32-byte sectors: the TMA unit fetches rows
+// of 3, 5 or 9 groups of 16 bytes in far more requests than rows of 4, 6 or 10 (ncu, P15 48 x 48 cells: 3.9 M requests
+// to L2 a pass at nx = 20, 2.2 M at nx = 24).  The tensor maps span the padding.  GB300, P15 48 x 48 x nx, us a pass, rows
+// of groups / of sectors: nx = 9 to 11 20.6 / 18.6, 17 to 19 37 / 27, 25 to 31 26.8 / 26.7, 33 to 35 51 / 45, 41 to 43 45 / 45.
 inline int stage_row_pitch(int precision, int nx) {
-    const int grp = precision == RTPN_FP32 && nx < 32 ? 8 : stage_row_group(precision);
+    const int grp = precision == RTPN_FP32 && nx < 40 ? 8 : stage_row_group(precision);
     return (nx + grp - 1) / grp * grp;
 }
 bool stage_sized(int precision, const Geom& g);

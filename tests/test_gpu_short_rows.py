@@ -1,4 +1,4 @@
-"""Short rows padded to whole sectors (FP32 below 32 cells): steps against the oracle at every remainder."""
+"""Short rows padded to whole sectors (FP32 below 40 cells): steps against the oracle at every remainder."""
 import pytest
 
 from paper_2004_02833_gb300 import rtpn, synth
@@ -7,7 +7,7 @@ from test_gpu_parity import assert_parity, oracle_problem
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("nx", [9, 11, 14, 17, 18, 19, 25, 27, 31, 33])
+@pytest.mark.parametrize("nx", [9, 11, 14, 17, 18, 19, 25, 27, 31, 33, 35, 37, 41])
 @pytest.mark.parametrize("bc", ["periodic", "vacuum"])
 def test_steps_on_short_padded_rows(cuda_device, coupling_cache, nx, bc):
     inst, u0 = synth.random_instance(15, (3, 5, nx), seed=1600 + nx, bc=bc)

@@ -272,7 +272,7 @@ for N in (29, 39):
 
 
 def test_pitch_of_padded_rows(so):
-    # 16-byte groups; FP32 rows below 32 cells whole 32-byte sectors; 16-byte rows stay as they are
+    # 16-byte groups; FP32 rows below 40 cells whole 32-byte sectors; 16-byte rows stay as they are
     fake_runtime.run(so, """
 for precision, elem in (("fp32", 4), ("bf16", 2)):
     for N in (15, 39):
@@ -283,7 +283,7 @@ for precision, elem in (("fp32", 4), ("bf16", 2)):
                 px = nx
             elif nx < 8:
                 px = nx  # not padded: a kernel that takes any width
-            elif precision == "fp32" and nx < 32:
+            elif precision == "fp32" and nx < 40:
                 px = -(-nx // 8) * 8
             else:
                 px = -(-nx // group) * group
