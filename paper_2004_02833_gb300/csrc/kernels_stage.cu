@@ -108,6 +108,10 @@ static bool make_maps(CUtensorMap* out, void* base, int precision, const rtpn::G
 // excess is felt.  GB300, FP32, a round: P15 96^3 13.2 us with two CTAs of 32x2x2, 17.1 with one of 96x2x2,
 // 23.8 with one of 32x4x4 (0.303, 0.274 and 0.286 ms a pass; P19 80^3 0.246 ms with 80x2x2, 0.289 with two CTAs
 // of 40x2x2); P39 69 us with 192 cells, 82 with 320, and 32x3x3 tiles 82 us at 96^3 (aligned), 113 at 120^3.
+// Measured on FP32 grids at N = 15, 19 and 39; N = 29, N = 7 and BF16 take the constants over.  Against every variant by
+// name on 18 grids of 320 to 262144 cells (N = 15 to 39, both storages) the choice is within 5 % of the best but at P15
+// (up to 18 % on grids of one or two rounds) and, at P29 and P39 near one round, where it was the one-stage variants
+// that it no longer takes.
 static const Variant* best_variant(int N, int precision, int depth, const rtpn::Geom& g, int px, int sms) {
     const Variant* best = nullptr;
     double best_cost = 0;
