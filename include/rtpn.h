@@ -150,7 +150,8 @@ int rtpn_set_scattering(rtpn_ctx* ctx, const double* f, int count);
  * otherwise; the spacing is then unchanged, as after any failure).  Non-cubic cells run on the staged and
  * generic kernels, on the window kernel up to N = 15 (and in the adjoint): RTPN_EUNSUPPORTED if the fused kernel
  * or the window kernel above N = 15 is selected explicitly, and for a batch instance (its spacing is fixed at
- * rtpn_batch_create); RTPN_KERNEL_AUTO moves to a kernel that takes them.  Rebuilds the coupling tables (synchronises the context stream); the media factors do not depend on h. */
+ * rtpn_batch_create); RTPN_KERNEL_AUTO moves to a kernel that takes them.  Rebuilds the coupling tables
+ * (synchronises the context stream); the media factors do not depend on h. */
 int rtpn_set_spacing(rtpn_ctx* ctx, double hx, double hy, double hz);
 
 /* Order all later work of the context on `stream` (a cudaStream_t; NULL = legacy default). */
